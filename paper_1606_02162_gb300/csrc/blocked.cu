@@ -87,7 +87,7 @@ struct BlockedArgs {
     int32_t wmax, rmax;
     const int64_t* row;
     const int32_t* col;
-    double d, t;
+    ForceConsts c;
     int p;
     void* pos_out;
     void* disp_out;
@@ -610,7 +610,7 @@ __device__ __forceinline__ void finish_row(const BlockedArgs& A, const Att<T, MO
 {
     using P2 = typename V2<T>::type;
     const P2 pu = reinterpret_cast<const P2*>(A.pos)[u0 + i];
-    const T d2 = (T)(A.d * A.d);
+    const T d2 = const_d2<T>(A.c);
     Acc<T, COMP> rep;
     const P2 c0 = cells[2 * i];
     rep.sx = c0.x * d2;
@@ -621,7 +621,7 @@ __device__ __forceinline__ void finish_row(const BlockedArgs& A, const Att<T, MO
         rep.cy = c1.y * d2;
     }
     rep.merge(at.sx, at.sy, at.cx, at.cy);
-    apply_move<T>(A.t, A.pos_out, A.disp_out, u0 + i, pu.x, pu.y, rep.fx(), rep.fy());
+    apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u0 + i, pu.x, pu.y, rep.fx(), rep.fy());
 }
 
 template <class T, int MODEL, bool COMP>
@@ -635,7 +635,7 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
     Att<T, MODEL, COMP, kSrcShared> att;
     att.src.set_shared(tile, (uint32_t)tb);
-    att.inv_d = (T)(1.0 / A.d);
+    att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
     const uint32_t* col = reinterpret_cast<const uint32_t*>(A.col);
     // warp w takes rows [32 w, 32 w + 32), then 1024 further on: each lane
@@ -683,7 +683,7 @@ struct CombineArgs {
     const int32_t* col;
     int64_t n;
     int32_t nt;
-    double d, t;
+    ForceConsts c;
     int p;
     const void* pos_in;
     const void* part;
@@ -744,13 +744,13 @@ template <class T, bool COMP>
 __device__ __forceinline__ void finish_vertex(const CombineArgs& A, int64_t u, T xu, T yu,
                                               Acc<T, COMP> rep, const Acc<T, COMP>& att)
 {
-    const T d2 = (T)(A.d * A.d);
+    const T d2 = const_d2<T>(A.c);
     rep.sx *= d2;
     rep.sy *= d2;
     rep.cx *= d2;
     rep.cy *= d2;
     rep.merge(att.sx, att.sy, att.cx, att.cy);
-    apply_move<T>(A.t, A.pos_out, A.disp_out, u, xu, yu, rep.fx(), rep.fy());
+    apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u, xu, yu, rep.fx(), rep.fy());
 }
 
 template <class T, int MODEL, bool COMP>
@@ -760,7 +760,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
     Att<T, MODEL, COMP> att;
     att.src.pos = pos;
-    att.inv_d = (T)(1.0 / A.d);
+    att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
     Acc<T, COMP> rep, at;
     if ((int)blockIdx.x < A.nhub) {
@@ -1795,8 +1795,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     B.rmax = P.rmax;
     B.row = g->row;
     B.col = g->col;
-    B.d = prm->d;
-    B.t = t;
+    B.c = force_consts(prm->d, t);
     B.p = prm->p;
     B.pos_out = pos_out;
     B.disp_out = disp_out;
@@ -1811,8 +1810,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     C.col = g->col;
     C.n = g->n;
     C.nt = P.nt;
-    C.d = prm->d;
-    C.t = t;
+    C.c = B.c;
     C.p = prm->p;
     C.pos_in = pos_in;
     C.part = P.part;

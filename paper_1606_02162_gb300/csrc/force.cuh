@@ -17,6 +17,33 @@ template <> struct V2<double> { using type = double2; };
 
 enum Model { kFR = 0, kGeneric = 1 };
 
+// What a launch's threads need of d and t, formed once on the host in both
+// widths. GB300 runs two FP64 operations a clock per SM, so that a 1.0 / d
+// and two conversions in every thread of an FP32 kernel kept its FP64 pipe
+// 64% busy (combine_kernel on BA n = 100,000, k = 2). Per iteration: BA
+// n = 10,000, k = 2 (plain kernel) 17.8 -> 15.7 us, BA n = 100,000, k = 2
+// 33.7 -> 32.5 us, the 1000 x 1000 mesh, k = 3 68.0 -> 63.5 us. (batch_kernel
+// keeps its own expressions: with these it measured 8% slower, the
+// compiler's scheduling of its loops.)
+struct ForceConsts {
+    double d2, inv_d, t;
+    float d2f, inv_df, tf;
+};
+
+inline ForceConsts force_consts(double d, double t)
+{
+    return {d * d, 1.0 / d, t, (float)(d * d), (float)(1.0 / d), (float)t};
+}
+
+template <class T> __device__ __forceinline__ T const_d2(const ForceConsts& c);
+template <> __device__ __forceinline__ float const_d2<float>(const ForceConsts& c) { return c.d2f; }
+template <> __device__ __forceinline__ double const_d2<double>(const ForceConsts& c) { return c.d2; }
+template <class T> __device__ __forceinline__ T const_inv_d(const ForceConsts& c);
+template <> __device__ __forceinline__ float const_inv_d<float>(const ForceConsts& c) { return c.inv_df; }
+template <> __device__ __forceinline__ double const_inv_d<double>(const ForceConsts& c) { return c.inv_d; }
+template <class T> __device__ __forceinline__ T const_t(const ForceConsts& c);
+template <> __device__ __forceinline__ float const_t<float>(const ForceConsts& c) { return c.tf; }
+template <> __device__ __forceinline__ double const_t<double>(const ForceConsts& c) { return c.t; }
 
 // Streaming load of four ids: read once per iteration, kept out of L1 so
 // that L1 serves the position gathers.
@@ -312,11 +339,10 @@ __device__ __forceinline__ void row_sum_rel(const uint32_t* __restrict__ ids, in
 }
 
 template <class T>
-__device__ __forceinline__ void apply_move(double t_, void* pos_out, void* disp_out, int64_t u,
+__device__ __forceinline__ void apply_move(T t, void* pos_out, void* disp_out, int64_t u,
                                            T xu, T yu, T fx, T fy)
 {
     using P2 = typename V2<T>::type;
-    const T t = (T)t_;
     const T fn = sqrt(fx * fx + fy * fy);
     T mx = fx, my = fy;
     if (fn > t) {

@@ -44,7 +44,7 @@ struct IterArgs {
     double* partials;
     int32_t n0, n1, n2, nchunks;
     int32_t b3, b2, b1, b0;  // blocks per class, launched in the order 3, 2, 1, 0
-    double d, t;
+    ForceConsts c;
     int p, q;
     const void* pos_in;
     void* pos_out;
@@ -56,7 +56,7 @@ template <class T>
 __device__ __forceinline__ void apply_move_it(const IterArgs& A, int64_t u, T xu, T yu, T fx,
                                               T fy)
 {
-    apply_move<T>(A.t, A.pos_out, A.disp_out, u, xu, yu, fx, fy);
+    apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u, xu, yu, fx, fy);
 }
 
 // Block-wide sum of an accumulator in a fixed order (warps, then warp 0).
@@ -123,12 +123,12 @@ iteration_kernel(const IterArgs A)
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
     Rep<T, MODEL, COMP, kSrcGlobal, false, W> rep;
     rep.src.pos = pos;
-    rep.d2 = (T)(A.d * A.d);
+    rep.d2 = const_d2<T>(A.c);
     rep.q = A.q;
     rep.wt = reinterpret_cast<const T*>(A.wt);
     Att<T, MODEL, COMP> att;
     att.src.pos = pos;
-    att.inv_d = (T)(1.0 / A.d);
+    att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
     int b = blockIdx.x;
     if (b < A.b3) {
@@ -512,8 +512,7 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
     A.b2 = B.n2;
     A.b1 = (B.n1 + kWarpsPerBlock - 1) / kWarpsPerBlock;
     A.b0 = (B.n0 + (kThreads / 8) - 1) / (kThreads / 8);
-    A.d = prm->d;
-    A.t = t;
+    A.c = force_consts(prm->d, t);
     A.p = prm->p;
     A.q = prm->q;
     A.pos_in = pos_in;
