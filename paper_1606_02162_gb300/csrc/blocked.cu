@@ -1099,9 +1099,11 @@ struct MetricArgs {
     const int4* bdesc;     // nb: first row, end row and tile of block b
     const int64_t* wbase;  // window mode: 2 nb (first id, length), else null
     int64_t n;
-    int32_t nt, tv, tcap;
-    double d;
+    int32_t nt, tv;
+    double d2;
+    float d2hi, d2lo;      // d2 as a double-float
     int q;
+    int unit;              // d = 1 and q = 1
     const float2* pos;
     double* partial;       // one per CTA
     uint64_t wait_ns;
@@ -1116,7 +1118,7 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
     __shared__ double s_part[kMetWarps];
     __shared__ int s_wsum[kMetWarps];
     __shared__ int s_pre[kMetBatch + 1];
-    __shared__ int64_t s_lo[kMetBatch];
+    __shared__ int64_t s_off[kMetBatch];  // entry i of the batch is kcol[s_off[its row] + i]
     __shared__ float2 s_q[kMetBatch];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 bd = A.bdesc[blockIdx.x];
@@ -1145,14 +1147,11 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
     double part = 0.0;
     if (tile_ok) {
         mbar_wait(&tile_bar, 0, A.wait_ns);
-        const Ff d2f = ff_from_double(A.d * A.d);
-        const bool unit = A.d == 1.0 && A.q == 1;
+        const Ff d2f = {A.d2hi, A.d2lo};
+        const bool unit = A.unit != 0;
         Ff s = {0.f, 0.f};
-        int cnt = 0;
-        // one pair {u, v}: d^2 / delta^q in double-float, sixteen terms of a
-        // lane summed as a double-float, then added to its FP64 sum
-        auto term = [&](float2 qu, uint32_t v) {
-            const float2 pv = tile[v - tb];
+        // one pair {u, v}: d^2 / delta^q in double-float
+        auto term = [&](float2 qu, float2 pv) {
             const Ff r2 = ff_dist2(qu.x, qu.y, pv.x, pv.y);
             if (r2.hi >= 1e-30f && r2.hi <= 1e30f) {
                 // d = 1, q = 1 (the defaults): the products by 1 are exact
@@ -1165,13 +1164,8 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
                 if (dl > 0.0) {
                     double w = 1.0;
                     for (int i = 0; i < A.q; ++i) w *= dl;
-                    part += A.d * A.d / w;
+                    part += A.d2 / w;
                 }
-            }
-            if (++cnt == 16) {
-                part += (double)s.hi + (double)s.lo;
-                s = {0.f, 0.f};
-                cnt = 0;
             }
         };
         // rows by batches of kMetBatch: thread t finds row r0 + t's run of
@@ -1226,7 +1220,7 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
             __syncthreads();
             if (threadIdx.x < kMetBatch) {
                 s_pre[threadIdx.x] = s_wsum[warp] + incl - len;
-                s_lo[threadIdx.x] = lo;
+                s_off[threadIdx.x] = lo - (s_wsum[warp] + incl - len);
                 float2 q = make_float2(0.f, 0.f);
                 if (u < u1) q = A.pos[u];
                 s_q[threadIdx.x] = q;
@@ -1242,14 +1236,54 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
                     const int mid = (r + hr + 1) >> 1;
                     if (s_pre[mid] <= beg + lane) r = mid; else hr = mid - 1;
                 }
-                for (int i = beg + lane; i < end; i += 32) {
-                    while (s_pre[r + 1] <= i) ++r;
-                    term(s_q[r], A.kcol[s_lo[r] + (i - s_pre[r])]);
+                // sixteen terms of a lane summed as a double-float, then
+                // added to its FP64 sum: an inner loop of its own (with a
+                // counter tested after every term the compiler formed the
+                // FP64 sum each time, and the FP64 pipe was 83% busy: BA
+                // n = 100,000, k = 3, 1311 us)
+                // The row's bound, offset and position stay in registers
+                // until it changes, and the ids and positions of four terms
+                // are read before the first of them is formed (BA
+                // n = 100,000, k = 3: 860 us with the inner loop alone, 497 now)
+                int bound = s_pre[r + 1];
+                int64_t off = s_off[r];
+                float2 q = s_q[r];
+                auto follow = [&](int i) {
+                    if (bound <= i) {
+                        do bound = s_pre[++r + 1]; while (bound <= i);
+                        off = s_off[r];
+                        q = s_q[r];
+                    }
+                };
+                int i = beg + lane;
+                for (; i + 15 * 32 < end;) {
+                    s = {0.f, 0.f};
+#pragma unroll 1
+                    for (int g4 = 0; g4 < 4; ++g4, i += 128) {
+                        float2 qu[4], pv[4];
+                        uint32_t id[4];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            follow(i + 32 * c);
+                            id[c] = A.kcol[off + (i + 32 * c)];
+                            qu[c] = q;
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) pv[c] = tile[id[c] - tb];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) term(qu[c], pv[c]);
+                    }
+                    part += (double)s.hi + (double)s.lo;
                 }
+                s = {0.f, 0.f};
+                for (; i < end; i += 32) {
+                    follow(i);
+                    term(q, tile[A.kcol[off + i] - tb]);
+                }
+                part += (double)s.hi + (double)s.lo;
             }
             __syncthreads();  // the next batch reuses the arrays
         }
-        part += (double)s.hi + (double)s.lo;
     }
     // fixed-order block sum: lanes, then warps in order
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
@@ -1262,13 +1296,20 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
     }
 }
 
-__global__ void sum_in_order_kernel(const double* __restrict__ v, int count, double* out)
+// The sum of count values in a fixed order: every 256th by one thread, then
+// the threads' sums in a tree (one thread over 456 values took 27 us).
+__global__ void __launch_bounds__(256)
+sum_partials_kernel(const double* __restrict__ v, int count, double* out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < count; ++i) t += v[i];
-        *out = t;
+    __shared__ double sh[256];
+    double t = 0.0;
+    for (int i = threadIdx.x; i < count; i += 256) t += v[i];
+    sh[threadIdx.x] = t;
+    for (int o = 128; o > 0; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     }
+    if (threadIdx.x == 0) *out = sh[0];
 }
 
 }  // namespace
@@ -1844,20 +1885,24 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     return GILA_OK;
 }
 
-gila_status blocked_khop_metric(gila_graph* g, const gila_params* prm, const void* pos,
-                                bool* done, double* rep_total)
+int64_t blocked_metric_partials(const gila_graph* g, const gila_params* prm, const void* pos)
 {
-    *done = false;
     const TilePlan& P = g->tplan[0];
-    if (is_f64(prm->precision) || !P.ready || !P.use || g->n == 0 || g->wt64) return GILA_OK;
-    if (((uintptr_t)pos & 15) != 0) return GILA_OK;
+    if (is_f64(prm->precision) || !P.ready || !P.use || g->n == 0 || g->wt64) return 0;
+    if (((uintptr_t)pos & 15) != 0) return 0;
     // the tile (or window) beside the kernel's own shared arrays; a larger
     // window leaves the term to the generic reduction
+    if (((size_t)P.tv + 1) * sizeof(float2) > (size_t)kMetSmemMax) return 0;
+    return P.nb;
+}
+
+gila_status blocked_khop_metric(gila_graph* g, const gila_params* prm, const void* pos,
+                                double* partials, double* rep_total)
+{
+    const TilePlan& P = g->tplan[0];
     const size_t smem = ((size_t)P.tv + 1) * sizeof(float2);
-    if (smem > (size_t)kMetSmemMax) return GILA_OK;
     const int grid = P.nb;
-    gila_status s = ensure((void**)&g->red, &g->red_cap, sizeof(double) * ((size_t)grid + 8));
-    if (s != GILA_OK) return s;
+    const double d2 = prm->d * prm->d;
     MetricArgs M;
     M.krow = g->krow;
     M.len = P.window ? nullptr : P.len;
@@ -1867,11 +1912,13 @@ gila_status blocked_khop_metric(gila_graph* g, const gila_params* prm, const voi
     M.n = g->n;
     M.nt = P.nt;
     M.tv = P.tv;
-    M.tcap = P.tv;
-    M.d = prm->d;
+    M.d2 = d2;
+    M.d2hi = (float)d2;
+    M.d2lo = (float)(d2 - (double)M.d2hi);
+    M.unit = prm->d == 1.0 && prm->q == 1;
     M.q = prm->q;
     M.pos = reinterpret_cast<const float2*>(pos);
-    M.partial = g->red;
+    M.partial = partials;
     M.wait_ns = kWaitNs;
     static std::atomic<uint64_t> configured{0};
     const uint64_t bit = 1ull << (g->device & 63);
@@ -1883,15 +1930,9 @@ gila_status blocked_khop_metric(gila_graph* g, const gila_params* prm, const voi
     }
     khop_metric_kernel<<<grid, kMetThreads, smem, g->stream>>>(M);
     count_launch();
-    sum_in_order_kernel<<<1, 32, 0, g->stream>>>(g->red, grid, g->red + grid);
+    sum_partials_kernel<<<1, 256, 0, g->stream>>>(partials, grid, rep_total);
     count_launch();
     GILA_CUDA(cudaGetLastError());
-    double h = 0.0;
-    GILA_CUDA(cudaMemcpyAsync(&h, g->red + grid, sizeof(double), cudaMemcpyDeviceToHost,
-                              g->stream));
-    GILA_CUDA(cudaStreamSynchronize(g->stream));
-    *rep_total = h;
-    *done = true;
     return GILA_OK;
 }
 

@@ -38,12 +38,6 @@ __device__ __forceinline__ Ff ff_two_prod(float a, float b)
     return {p, __fmaf_rn(a, b, -p)};
 }
 
-__device__ __forceinline__ Ff ff_from_double(double x)
-{
-    const float h = (float)x;
-    return {h, (float)(x - (double)h)};
-}
-
 __device__ __forceinline__ Ff ff_add(Ff a, Ff b)
 {
     const Ff s = ff_two_sum(a.hi, b.hi);
@@ -63,17 +57,29 @@ __device__ __forceinline__ Ff ff_mul(Ff a, Ff b)
 // 2^-48 of the result) is left out.
 __device__ __forceinline__ Ff ff_dist2(float ax, float ay, float bx, float by)
 {
-    const Ff dx = ff_two_sum(ax, -bx);
-    const Ff dy = ff_two_sum(ay, -by);
+    // both differences' two-sums in packed two-lane arithmetic (sm_100 and
+    // later; the same roundings, half the instructions)
+    uint64_t a, b, d, t, e;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(ax), "f"(ay));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(bx), "f"(by));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));  // d = a - b
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(d), "l"(a));  // t = d - a, about -b
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e) : "l"(d), "l"(t));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e) : "l"(a), "l"(e));  // a - (d - t)
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(b), "l"(t));  // b + t
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e) : "l"(e), "l"(t));  // the differences' low parts
+    Ff dx, dy;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(dx.hi), "=f"(dy.hi) : "l"(d));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(dx.lo), "=f"(dy.lo) : "l"(e));
     const Ff px = ff_two_prod(dx.hi, dx.hi);
     const Ff py = ff_two_prod(dy.hi, dy.hi);
     const Ff s = ff_two_sum(px.hi, py.hi);
-    const float cross = __fmaf_rn(2.0f * dx.hi, dx.lo, __fmul_rn(2.0f * dy.hi, dy.lo));
-    const float low = __fadd_rn(__fadd_rn(s.lo, __fadd_rn(px.lo, py.lo)), cross);
+    const float half_cross = __fmaf_rn(dx.hi, dx.lo, __fmul_rn(dy.hi, dy.lo));
+    const float low = __fmaf_rn(2.0f, half_cross, __fadd_rn(s.lo, __fadd_rn(px.lo, py.lo)));
     return ff_fast_two_sum(s.hi, low);
 }
 
-// 1 / sqrt(r2) for r2 = hi + lo > 0: the hardware's approximate reciprocal
+// 1 / sqrt(r2) for r2 = hi + lo, hi normal and > 0: the hardware's approximate reciprocal
 // square root y0 of hi (relative error below 2^-22) refined by the series
 // y = y0 (1 + e/2 + 3e^2/8) of y0 / sqrt(1 - e), with e = 1 - r2 y0^2 formed
 // exactly up to the rounding of its low parts (the classical Newton step for
@@ -83,7 +89,7 @@ __device__ __forceinline__ Ff ff_dist2(float ax, float ay, float bx, float by)
 __device__ __forceinline__ Ff ff_rsqrt(Ff r2)
 {
     float y0;
-    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y0) : "f"(r2.hi));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(r2.hi));
     const Ff y2 = ff_two_prod(y0, y0);
     const Ff t = ff_two_prod(r2.hi, y2.hi);
     const float tl = __fadd_rn(t.lo, __fmaf_rn(r2.hi, y2.lo, __fmul_rn(r2.lo, y2.hi)));

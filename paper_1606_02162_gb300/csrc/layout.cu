@@ -308,91 +308,144 @@ __device__ __forceinline__ double dipow(double x, int e)
     return r;
 }
 
-// pass 0: [sum delta, count, sum delta^p/d, sum over k-hop pairs d^2/delta^q]
-// pass 1: [sum (delta - mean)^2, 0, 0, 0]
-// Each warp owns a fixed set of vertices; partial sums are combined in a
-// fixed order, so the result does not depend on timing.
+// pass 0: [sum delta, count, sum delta^p, sum over k-hop pairs d^2/delta^q]
+// pass 1: [sum (delta - mean)^2, 0, 0, 0], the mean read from the reduced
+//         results of pass 0
+// The adjacency is taken by runs of kEdgeRun consecutive entries per warp,
+// whatever rows they belong to, and the entries above their row's id (each
+// edge once) are queued in shared memory and taken 32 at a time, so that
+// every lane carries an edge: the edge terms are FP64 (two operations a clock
+// per SM), and with a warp per vertex a row of six neighbours issued them for
+// 32 lanes (BA n = 100,000, 300k edges: 150 us a pass, 60 by runs without the
+// queue, 36 with it). The k-hop rows are taken by a warp per
+// vertex. Each warp owns a fixed set of runs and rows and partial sums are
+// combined in a fixed order, so the result does not depend on timing.
+constexpr int kEdgeRun = 256;
+
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
 metrics_kernel(int pass, int64_t n, const int64_t* __restrict__ row,
                const int32_t* __restrict__ col, const int64_t* __restrict__ krow,
-               const uint32_t* __restrict__ kcol, const void* pos, double d, int p, int q,
-               double mean, double* __restrict__ partials, int skip_khop)
+               const uint32_t* __restrict__ kcol, const void* pos, double d2, float d2hi,
+               float d2lo, int p, int q, const double* __restrict__ mean_src,
+               double* __restrict__ partials, int skip_khop)
 {
     __shared__ double sh[kRedThreads / 32][4];
+    __shared__ int2 s_queue[kRedThreads / 32][64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * (kRedThreads / 32);
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int64_t u = (int64_t)blockIdx.x * (kRedThreads / 32) + warp; u < n; u += nw) {
-        const double2 pu = load_pos<T>(pos, u);
-        for (int64_t e = row[u] + lane; e < row[u + 1]; e += 32) {
-            const int64_t v = col[e];
-            if (v <= u) continue;
-            const double2 pv = load_pos<T>(pos, v);
-            const double dx = pu.x - pv.x, dy = pu.y - pv.y;
-            const double dl = sqrt(dx * dx + dy * dy);
-            if (pass == 0) {
-                a0 += dl;
-                a1 += 1.0;
-                if (dl > 0.0) a2 += dipow(dl, p) / d;
-            } else {
-                a0 += (dl - mean) * (dl - mean);
+    const int64_t gw = (int64_t)blockIdx.x * (kRedThreads / 32) + warp;
+    double a0 = 0.0, a2 = 0.0, a3 = 0.0;
+    int64_t cnt = 0;
+    const double mean = pass == 0 ? 0.0 : *mean_src;
+    const int64_t nnz = row[n];
+    auto edge = [&](int2 uv) {
+        const double2 pu = load_pos<T>(pos, uv.x);
+        const double2 pv = load_pos<T>(pos, uv.y);
+        const double dx = pu.x - pv.x, dy = pu.y - pv.y;
+        const double r2 = dx * dx + dy * dy;
+        const double dl = sqrt(r2);
+        if (pass == 0) {
+            a0 += dl;
+            ++cnt;
+            if (dl > 0.0) a2 += p == 2 ? r2 : dipow(dl, p);
+        } else {
+            a0 += (dl - mean) * (dl - mean);
+        }
+    };
+    int2* queue = s_queue[warp];
+    int qn = 0;  // edges waiting in the warp's queue
+    for (int64_t r = gw; r * kEdgeRun < nnz; r += nw) {
+        const int64_t e1 = (r + 1) * kEdgeRun < nnz ? (r + 1) * kEdgeRun : nnz;
+        int64_t e = r * kEdgeRun + lane;
+        int64_t u = 0;
+        if (e < e1) {
+            int64_t hi = n - 1;  // the last row that starts at or before e
+            while (u < hi) {
+                const int64_t mid = (u + hi + 1) >> 1;
+                if (row[mid] <= e) u = mid; else hi = mid - 1;
             }
         }
-        if (pass == 0 && sizeof(T) == 4 && !skip_khop) {
-            // FP32 placements: each pair's term d^2 / delta^q in double-float
-            // arithmetic (pairs of FP32 numbers, relative error about 1e-14,
-            // far below FP32's 6e-8), eight terms per lane summed as a
-            // double-float, then added in FP64. The FP64 pipe of GB300 is a
-            // small fraction of its FP32 rate, and a per-pair FP64 sqrt and
-            // divide made this pass ALU-bound; the pair form keeps FP64
-            // accuracy at FP32 throughput.
-            const float2* pf = reinterpret_cast<const float2*>(pos);
-            const float2 qu = pf[u];
-            const Ff d2f = ff_from_double(d * d);
-            const int64_t e1 = krow[u + 1];
-            for (int64_t e0 = krow[u]; e0 < e1; e0 += 256) {
-                Ff s = {0.f, 0.f};
+        for (int64_t e0 = r * kEdgeRun; e0 < e1; e0 += 32, e += 32) {
+            int32_t v = -1;
+            if (e < e1) {
+                while (row[u + 1] <= e) ++u;
+                v = col[e];
+            }
+            const bool keep = v > u;
+            const unsigned m = __ballot_sync(kFull, keep);
+            if (keep) queue[qn + __popc(m & lanemask_lt())] = make_int2((int)u, v);
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) {
+                edge(queue[lane]);
+                qn -= 32;
+                const int2 left = queue[32 + lane];
+                __syncwarp();
+                if (lane < qn) queue[lane] = left;
+                __syncwarp();
+            }
+        }
+    }
+    if (lane < qn) edge(queue[lane]);
+    if (pass == 0 && !skip_khop) {
+        for (int64_t u = gw; u < n; u += nw) {
+            if (sizeof(T) == 4) {
+                // FP32 placements: each pair's term d^2 / delta^q in
+                // double-float arithmetic (pairs of FP32 numbers, relative
+                // error about 1e-14, far below FP32's 6e-8), eight terms per
+                // lane summed as a double-float, then added in FP64. The FP64
+                // pipe of GB300 is a small fraction of its FP32 rate, and a
+                // per-pair FP64 sqrt and divide made this pass ALU-bound; the
+                // pair form keeps FP64 accuracy at FP32 throughput.
+                const float2* pf = reinterpret_cast<const float2*>(pos);
+                const float2 qu = pf[u];
+                const Ff d2f = {d2hi, d2lo};
+                const int64_t e1 = krow[u + 1];
+                for (int64_t e0 = krow[u]; e0 < e1; e0 += 256) {
+                    Ff s = {0.f, 0.f};
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int64_t e = e0 + j * 32 + lane;
-                    if (e >= e1) continue;
+                    for (int j = 0; j < 8; ++j) {
+                        const int64_t e = e0 + j * 32 + lane;
+                        if (e >= e1) continue;
+                        const int64_t v = kcol[e];
+                        if (v <= u) continue;
+                        const float2 pv = pf[v];
+                        const Ff r2 = ff_dist2(qu.x, qu.y, pv.x, pv.y);
+                        if (r2.hi >= 1e-30f && r2.hi <= 1e30f) {
+                            s = ff_add(s, ff_mul(d2f, ff_rsqrt_pow(r2, q)));
+                        } else {
+                            // distances outside the pair form's safe range (or
+                            // coincident vertices): the FP64 term from the exact
+                            // FP64 differences, none at distance 0
+                            const double dx = (double)qu.x - (double)pv.x;
+                            const double dy = (double)qu.y - (double)pv.y;
+                            const double dl = sqrt(dx * dx + dy * dy);
+                            if (dl > 0.0) a3 += d2 / dipow(dl, q);
+                        }
+                    }
+                    a3 += (double)s.hi + (double)s.lo;
+                }
+            } else {
+                const double2 pu = load_pos<T>(pos, u);
+                for (int64_t e = krow[u] + lane; e < krow[u + 1]; e += 32) {
                     const int64_t v = kcol[e];
                     if (v <= u) continue;
-                    const float2 pv = pf[v];
-                    const Ff r2 = ff_dist2(qu.x, qu.y, pv.x, pv.y);
-                    if (r2.hi >= 1e-30f && r2.hi <= 1e30f) {
-                        s = ff_add(s, ff_mul(d2f, ff_rsqrt_pow(r2, q)));
-                    } else {
-                        // distances outside the pair form's safe range (or
-                        // coincident vertices): the FP64 term from the exact
-                        // FP64 differences, none at distance 0
-                        const double dx = (double)qu.x - (double)pv.x;
-                        const double dy = (double)qu.y - (double)pv.y;
-                        const double dl = sqrt(dx * dx + dy * dy);
-                        if (dl > 0.0) a3 += d * d / dipow(dl, q);
-                    }
+                    const double2 pv = load_pos<T>(pos, v);
+                    const double dx = pu.x - pv.x, dy = pu.y - pv.y;
+                    const double dl = sqrt(dx * dx + dy * dy);
+                    if (dl > 0.0) a3 += d2 / dipow(dl, q);
                 }
-                a3 += (double)s.hi + (double)s.lo;
-            }
-        } else if (pass == 0 && !skip_khop) {
-            for (int64_t e = krow[u] + lane; e < krow[u + 1]; e += 32) {
-                const int64_t v = kcol[e];
-                if (v <= u) continue;
-                const double2 pv = load_pos<T>(pos, v);
-                const double dx = pu.x - pv.x, dy = pu.y - pv.y;
-                const double dl = sqrt(dx * dx + dy * dy);
-                if (dl > 0.0) a3 += d * d / dipow(dl, q);
             }
         }
     }
     a0 = group_sum(a0, 32);
-    a1 = group_sum(a1, 32);
+    cnt = group_sum(cnt, 32);
     a2 = group_sum(a2, 32);
     a3 = group_sum(a3, 32);
     if (lane == 0) {
         sh[warp][0] = a0;
-        sh[warp][1] = a1;
+        sh[warp][1] = (double)cnt;
         sh[warp][2] = a2;
         sh[warp][3] = a3;
     }
@@ -404,15 +457,25 @@ metrics_kernel(int pass, int64_t n, const int64_t* __restrict__ row,
     }
 }
 
-// Sum the per-block partials in block order (one thread per component).
-__global__ void reduce_partials_kernel(const double* __restrict__ partials, int nblocks,
-                                       double* __restrict__ out)
+// Sum the per-block partials: 64 threads per component add every 64th block
+// in block order, then their sums in a fixed tree (four threads that added
+// 1,216 partials one after the other took 90 us). out[0..3] the sums,
+// out[4] = out[0] / out[1], the mean edge length after pass 0.
+__global__ void __launch_bounds__(256)
+reduce_partials_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out)
 {
-    if (threadIdx.x < 4) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partials[b * 4 + threadIdx.x];
-        out[threadIdx.x] = s;
+    __shared__ double sh[256];
+    const int c = threadIdx.x & 3;
+    double s = 0.0;
+    for (int b = threadIdx.x >> 2; b < nblocks; b += 64) s += partials[b * 4 + c];
+    sh[threadIdx.x] = s;
+    for (int o = 128; o >= 4; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     }
+    __syncthreads();
+    if (threadIdx.x < 4) out[threadIdx.x] = sh[threadIdx.x];
+    if (threadIdx.x == 0) out[4] = sh[1] > 0.0 ? sh[0] / sh[1] : 0.0;
 }
 
 template <class T>
@@ -546,44 +609,43 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
 gila_status compute_metrics(gila_graph* g, const gila_params* prm, const void* pos,
                             gila_metrics* out)
 {
-    gila_status s = ensure_red(g, (size_t)kRedBlocks * 4 + 8);
-    if (s != GILA_OK) return s;
-    double* part = g->red;
-    double* res = g->red + (size_t)kRedBlocks * 4;
-    double h[4];
-    const bool f64 = is_f64(prm->precision);
     // FP32 placements with a blocked plan take the k-hop term over the
     // plan's shared-memory position tiles (the pairs' positions are
-    // otherwise random gathers through L2); the edge terms stay here
-    bool tiled = false;
-    double rep_tiled = 0.0;
-    {
-        gila_status bs = blocked_khop_metric(g, prm, pos, &tiled, &rep_tiled);
-        if (bs != GILA_OK) return bs;
-    }
-    auto run = [&](int pass, double mean) -> cudaError_t {
-        if (f64)
+    // otherwise random gathers through L2); the edge terms stay here.
+    // Scratch: the results, the blocks' partials, the tiles' partials
+    const int64_t ntile = blocked_metric_partials(g, prm, pos);
+    constexpr size_t kRes = 16;
+    gila_status s = ensure_red(g, kRes + (size_t)kRedBlocks * 4 + (size_t)ntile);
+    if (s != GILA_OK) return s;
+    double* res = g->red;            // pass 0 at 0, pass 1 at 5, tiled k-hop term at 10
+    double* part = g->red + kRes;
+    double h[kRes] = {};
+    if (ntile > 0 &&
+        (s = blocked_khop_metric(g, prm, pos, part + (size_t)kRedBlocks * 4, res + 10)) != GILA_OK)
+        return s;
+    const double d2 = prm->d * prm->d;
+    const float d2hi = (float)d2, d2lo = (float)(d2 - (double)d2hi);
+    // both passes in one go: the second reads the mean on the device
+    for (int pass = 0; pass < 2; ++pass) {
+        if (is_f64(prm->precision))
             metrics_kernel<double><<<kRedBlocks, kRedThreads, 0, g->stream>>>(
-                pass, g->n, g->row, g->col, g->krow, g->kcol, pos, prm->d, prm->p, prm->q, mean,
-                part, 0);
+                pass, g->n, g->row, g->col, g->krow, g->kcol, pos, d2, d2hi, d2lo, prm->p, prm->q,
+                res + 4, part, 0);
         else
             metrics_kernel<float><<<kRedBlocks, kRedThreads, 0, g->stream>>>(
-                pass, g->n, g->row, g->col, g->krow, g->kcol, pos, prm->d, prm->p, prm->q, mean,
-                part, tiled ? 1 : 0);
+                pass, g->n, g->row, g->col, g->krow, g->kcol, pos, d2, d2hi, d2lo, prm->p, prm->q,
+                res + 4, part, ntile > 0 ? 1 : 0);
         count_launch();
-        reduce_partials_kernel<<<1, 32, 0, g->stream>>>(part, kRedBlocks, res);
+        reduce_partials_kernel<<<1, 256, 0, g->stream>>>(part, kRedBlocks, res + 5 * pass);
         count_launch();
-        cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, g->stream);
-        return cudaStreamSynchronize(g->stream);
-    };
-    cudaError_t e = run(0, 0.0);
-    if (e != cudaSuccess) return cuda_fail(e, "metrics pass 0");
+    }
+    GILA_CUDA(cudaGetLastError());
+    GILA_CUDA(cudaMemcpyAsync(h, res, sizeof(double) * 11, cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));
     const double m = h[1];
     const double mean = m > 0 ? h[0] / m : 0.0;
-    const double att = h[2], rep = tiled ? rep_tiled : h[3];
-    e = run(1, mean);
-    if (e != cudaSuccess) return cuda_fail(e, "metrics pass 1");
-    const double var = m > 0 ? h[0] / m : 0.0;
+    const double att = h[2] / prm->d, rep = ntile > 0 ? h[10] : h[3];
+    const double var = m > 0 ? h[5] / m : 0.0;
     out->edge_mean = mean;
     out->edge_std = sqrt(var);
     out->edge_cv = mean > 0 ? out->edge_std / mean : 0.0;

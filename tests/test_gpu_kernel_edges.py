@@ -1,0 +1,53 @@
+"""Kernels at the sizes where they can go wrong: remainders, the edges of
+runs, tiles and windows, empty rows and hubs, each against the FP64 oracle.
+
+Tolerances: k-hop lists exact; one step within 1e-4 (FP32 modes) and 1e-12
+(FP64) of the largest move; quality figures within 1e-11 relative.
+"""
+import numpy as np
+import pytest
+
+import __graft_entry__
+import oracle as O
+from paper_1606_02162_gb300 import gila as G
+from paper_1606_02162_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TOL = {G.GILA_FP32: 1e-4, G.GILA_FP32_COMPENSATED: 1e-4, G.GILA_FP64: 1e-12}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+    import torch
+    torch.cuda.set_device(0)
+
+
+def hub_and_gaps(edges, n, isolated):
+    """A hub joined to the first `edges` vertices after it, a path along the
+    rest, and `isolated` vertices without edges at the end."""
+    a = np.concatenate([np.zeros(edges, dtype=np.int64), np.arange(edges, n - 1)])
+    b = np.concatenate([np.arange(1, edges + 1), np.arange(edges + 1, n)])
+    return I.csr_from_edges(n + isolated, a, b)
+
+
+# entries of the adjacency (2 E): below, at and above one run of 256 entries,
+# a hub longer than a run, trailing and leading empty rows
+@pytest.mark.parametrize("g", [
+    hub_and_gaps(5, 20, 0), hub_and_gaps(20, 129, 3), hub_and_gaps(20, 130, 0),
+    hub_and_gaps(1000, 1300, 700), I.csr_from_edges(600, [598], [599]), I.csr_from_edges(3, [], []),
+], ids=["small", "one_run", "run_and_two", "hub", "last_edge", "no_edges"])
+@pytest.mark.parametrize("p", [0, 2, 3])
+def test_edge_figures(g, p):
+    import torch
+    pos = I.uniform_positions(g.n, 11).astype(np.float32).astype(np.float64)
+    pos[1] = pos[0]  # an edge (or pair) of length 0
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 2)
+    want = O.metrics(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, d=1.3, p=p)
+    for prec, dt in ((G.GILA_FP64, torch.float64), (G.GILA_FP32, torch.float32)):
+        with G.Graph.from_inputs(g) as h:
+            got = G.gila_layout_metrics(h.handle, G.params(k=2, d=1.3, p=p, precision=prec),
+                                        torch.tensor(pos, dtype=dt, device="cuda"))
+        for key in ("edge_mean", "edge_std", "edge_cv", "rep_total", "att_total"):
+            assert abs(got[key] - want[key]) <= 1e-11 * max(1.0, abs(want[key])), (key, prec)
