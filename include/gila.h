@@ -113,9 +113,10 @@ typedef struct gila_tuning {
                               shared memory instead of gathering them through L2. Graphs
                               whose row ranges touch narrow id windows get one window per
                               range, and each range's CTA finishes its rows (automatic mode:
-                              where the windows' positions stay below the id stream's
-                              bytes); other graphs get tiles of positions and a second
-                              kernel that adds each row's tile partials */
+                              where rows are short and of about equal length, a row per
+                              lane; otherwise where the windows' positions stay below the
+                              id stream's bytes); other graphs get tiles of positions and a
+                              second kernel that adds each row's tile partials */
     int32_t tile_vertices; /* positions per tile; 0 = as many as fit in 200 KiB */
     int32_t min_segment;   /* automatic mode tiles placements with at least 4 10^6 k-hop
                               entries when nnz_khop / (n * tiles) >= this (0: always) */

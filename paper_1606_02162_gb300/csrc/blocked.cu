@@ -678,6 +678,250 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
     }
 }
 
+// Window mode with a row per lane, for graphs whose rows are of about equal
+// length (meshes, grids): a slice is 32 consecutive rows, stored step-major
+// (four 16-bit ids of every lane, 256 bytes a step), each row padded with the
+// far slot's id to the slice's longest. A lane sums its row in registers and
+// moves its vertex: no row changes inside a step, no scan over lanes, no
+// cells, no second pass over the rows. The first ids of a row are its
+// neighbours (A is part of N(k)), whose attraction is formed from the same
+// shared-memory positions, so the adjacency is not read at all. A warp takes
+// consecutive slices, one stream of steps, four steps ahead in registers.
+// Consecutive rows of a mesh read consecutive positions in each step, which
+// keeps their gathers free of bank conflicts without any reordering. 512
+// threads at 64 registers put two CTAs on an SM, one loading its window
+// while the other computes.
+// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration
+// against the shares of blocked_kernel; 700 x 700, FP32: 35.3 -> 17.6.
+//
+// Automatic mode takes it where (us per iteration, FP32, before -> this):
+// - mean rows reach kRowMeanLen: random ids within a band conflict in this
+//   order and long rows amortise the shares' costs (rows of 151 ids 48 -> 37,
+//   183: 54 -> 44, 413: 82 -> 94; a mesh at k = 8, 213 ids: 50 -> 35);
+// - a window fits two CTAs on an SM, with up to 16 times as many ranges,
+//   else one (random 4-regular graphs of 25,000 vertices, whose every window
+//   is the whole graph: rows of 479 ids 21 -> 33);
+// - the padding stays within kRowPadding (band graphs at 1.8 slots an
+//   entry: 39 -> 29, 30 -> 17);
+// - the windows' bytes stay within kRowWindowBytes an entry: they come from
+//   L2 once an iteration, and the alternative for a mesh is tiles that most
+//   rows have nothing in (mesh 2000 x 2000, k = 2: 4478 -> 77; grid
+//   1000 x 1000, k = 2: 364 -> 17; the FP64 mesh 1000 x 1000, k = 3:
+//   2453 -> 913, bound by its FP64 operations).
+constexpr int kRowThreads = 512;
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowAhead = 4;       // steps of ids in registers ahead
+constexpr int kRowMaxDeg = 64;     // longest adjacency row taken
+constexpr size_t kRowWindow = 110 * 1024;  // a window's bytes for two CTAs per SM
+constexpr int64_t kRowWindowBytes = 8;     // automatic mode: windows' bytes per k-hop entry
+constexpr double kRowMeanLen = 256.0;      // automatic mode: longest mean row
+constexpr double kRowPadding = 2.0;  // most slots per k-hop entry
+
+struct RowsArgs {
+    const uint16_t* tk;
+    const int4* sdesc;
+    const uint16_t* deg;
+    const int4* bdesc;
+    const int64_t* wbase;
+    int64_t n;
+    int q, p;
+    ForceConsts c;
+    const void* pos;
+    void* pos_out;
+    void* disp_out;
+    uint64_t wait_ns;
+    int skip_copy;
+};
+
+__device__ __forceinline__ uint2 ld_ids2(const uint2* p)
+{
+    uint2 r;
+    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));
+    return r;
+}
+
+template <class T, int MODEL, bool COMP>
+__global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kernel(const RowsArgs A)
+{
+    using P2 = typename V2<T>::type;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    P2* tile = reinterpret_cast<P2*>(smem_raw);
+    __shared__ __align__(8) uint64_t tile_bar;
+    __shared__ int tile_ok;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
+    const int64_t tb = A.wbase[2 * blockIdx.x], tn = A.wbase[2 * blockIdx.x + 1];
+    if (threadIdx.x == 0) {
+        // the window by the bulk-copy engine (its first id is even: 16-byte
+        // aligned); an odd float2 tail by hand; the far slot after it
+        const uint32_t bytes = (uint32_t)(((size_t)tn * sizeof(P2)) & ~size_t(15));
+        mbar_init(&tile_bar, 1);
+        mbar_arrive_expect_tx(&tile_bar, bytes);
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(pos + tb);
+        for (uint32_t o = 0; o < bytes && !A.skip_copy; o += kBulkChunk)
+            bulk_g2s(smem_raw + o, src + o, (bytes - o < kBulkChunk) ? bytes - o : kBulkChunk,
+                     &tile_bar);
+        if ((size_t)tn * sizeof(P2) != bytes) tile[tn - 1] = pos[tb + tn - 1];
+        P2 far;
+        far.x = FarSlot<T>::v;
+        far.y = FarSlot<T>::v;
+        tile[tn] = far;
+    }
+    // this warp's slices and the first steps of their stream
+    const int4 bd = A.bdesc[blockIdx.x];
+    const int s0 = bd.x >> 5, ns = ((bd.y + 31) >> 5) - s0;
+    const int sa = s0 + ns * warp / kRowWarps, sb = s0 + ns * (warp + 1) / kRowWarps;
+    int4 sd = make_int4(0, 0, 0, 0);
+    uint2 next[kRowAhead];
+    const uint2* ids = reinterpret_cast<const uint2*>(A.tk) + lane;
+    if (sa < sb) {
+        sd = A.sdesc[sa];
+#pragma unroll
+        for (int i = 0; i < kRowAhead; ++i)
+            if (i < sd.y) next[i] = ld_ids2(ids + 32 * ((int64_t)sd.x + i));
+    }
+    if (threadIdx.x == 0) {
+        bool ok = mbar_wait(&tile_bar, 0, A.wait_ns);
+        if (!ok) {
+            atomicExch(&g_tile_wait_failed, 1);
+            mbar_wait(&tile_bar, 0, A.wait_ns);  // let the copy land before the CTA ends
+        }
+        tile_ok = ok ? 1 : 0;
+    }
+    __syncthreads();
+    if (!tile_ok) return;  // uniform across the CTA
+    mbar_wait(&tile_bar, 0, A.wait_ns);  // completed: acquires the window for this thread
+
+    Rep<T, MODEL, COMP, kSrcShared, true> f;
+    f.src.set_shared(tile, 0u);
+    f.d2 = T(1);
+    f.q = A.q;
+    Att<T, MODEL, COMP, kSrcShared> att;
+    att.src.set_shared(tile, 0u);
+    att.inv_d = const_inv_d<T>(A.c);
+    att.p = A.p;
+    for (int s = sa; s < sb; ++s) {
+        const int64_t u = (int64_t)s * 32 + lane;
+        const bool live = u < A.n;
+        P2 pu;
+        pu.x = T(0);
+        pu.y = T(0);
+        int deg = 0;
+        if (live) {
+            pu = pos[u];
+            deg = A.deg[u];
+        }
+        f.xu = att.xu = pu.x;
+        f.yu = att.yu = pu.y;
+        const int dmax = __reduce_max_sync(kFull, deg);
+        const int steps = sd.y;
+        const int64_t start = sd.x;
+        const int4 sn = (s + 1 < sb) ? A.sdesc[s + 1] : make_int4(0, 0, 0, 0);
+        Acc<T, COMP> acc, at;
+        for (int k0 = 0; k0 < steps || k0 == 0; k0 += kRowAhead) {
+            uint2 cur[kRowAhead];
+#pragma unroll
+            for (int i = 0; i < kRowAhead; ++i) cur[i] = next[i];
+            // refill: the next steps of this slice, or the next slice's first
+            const bool more = k0 + kRowAhead < steps;
+            const int64_t from = more ? start + k0 + kRowAhead : (int64_t)sn.x;
+            const int left = more ? steps - k0 - kRowAhead : sn.y;
+#pragma unroll
+            for (int i = 0; i < kRowAhead; ++i)
+                if (i < left) next[i] = ld_ids2(ids + 32 * (from + i));
+            Acc<T, false> pend;
+#pragma unroll
+            for (int i = 0; i < kRowAhead; ++i) {
+                if (k0 + i >= steps) break;
+                const uint32_t v0 = cur[i].x & 0xffffu, v1 = cur[i].x >> 16;
+                const uint32_t v2 = cur[i].y & 0xffffu, v3 = cur[i].y >> 16;
+                if constexpr (COMP) {
+                    f(v0, pend);
+                    f(v1, pend);
+                    f(v2, pend);
+                    f(v3, pend);
+                } else {
+                    f(v0, acc);
+                    f(v1, acc);
+                    f(v2, acc);
+                    f(v3, acc);
+                }
+                const int e = 4 * (k0 + i);
+                if (e < dmax) {  // the rows' first ids are their neighbours
+                    if (e < deg) att(v0, at);
+                    if (e + 1 < deg) att(v1, at);
+                    if (e + 2 < deg) att(v2, at);
+                    if (e + 3 < deg) att(v3, at);
+                }
+            }
+            // compensated mode: up to sixteen terms summed plainly, then
+            // added with their error term
+            if constexpr (COMP) add_compensated(acc, pend.sx, pend.sy);
+        }
+        if (live) {
+            const T d2 = const_d2<T>(A.c);
+            acc.sx *= d2;
+            acc.sy *= d2;
+            acc.cx *= d2;
+            acc.cy *= d2;
+            acc.merge(at.sx, at.sy, at.cx, at.cy);
+            apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u, pu.x, pu.y, acc.fx(),
+                          acc.fy());
+        }
+        sd = sn;
+    }
+}
+
+// The slices of rows_kernel from the k-hop lists: a warp per slice, a row per
+// lane. The neighbours first, then the other ids (both lists ascending, one
+// merge), then the far slot's id (the window's length). A row whose
+// neighbours are not all found among its k-hop ids (an unsorted or repeated
+// adjacency, a self-loop) sets *bad, and the plan takes another form.
+__global__ void __launch_bounds__(128)
+rows_fill_kernel(int64_t n, int64_t nslices, const int64_t* __restrict__ row,
+                 const int32_t* __restrict__ col, const int64_t* __restrict__ krow,
+                 const uint32_t* __restrict__ kcol, const int4* __restrict__ sdesc,
+                 uint16_t* __restrict__ tk, uint16_t* __restrict__ deg_out, int* __restrict__ bad)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= nslices) return;  // warp-uniform
+    const int4 sd = sdesc[s];
+    const int64_t u = s * 32 + lane;
+    int64_t kb = 0, ke = 0, ab = 0;
+    int deg = 0;
+    if (u < n) {
+        kb = krow[u];
+        ke = krow[u + 1];
+        ab = row[u];
+        deg = (int)(row[u + 1] - ab);
+        deg_out[u] = (uint16_t)deg;
+    }
+    uint64_t* out = reinterpret_cast<uint64_t*>(tk) + (int64_t)sd.x * 32 + lane;
+    const int slots = sd.y * 4;
+    uint64_t four = 0;
+    int w = 0;
+    auto put = [&](uint32_t id) {
+        if (w >= slots) return;
+        four |= (uint64_t)(uint16_t)id << (16 * (w & 3));
+        if ((w & 3) == 3) {
+            out[32 * (w >> 2)] = four;
+            four = 0;
+        }
+        ++w;
+    };
+    for (int a = 0; a < deg; ++a) put((uint32_t)col[ab + a] - (uint32_t)sd.z);
+    int a = 0, found = 0;
+    for (int64_t i = kb; i < ke; ++i) {
+        const uint32_t x = kcol[i];
+        while (a < deg && (uint32_t)col[ab + a] < x) ++a;
+        if (a < deg && (uint32_t)col[ab + a] == x) ++found;
+        else put(x - (uint32_t)sd.z);
+    }
+    if (found != deg) atomicExch(bad, 1);
+    while (w < slots) put((uint32_t)sd.w);
+}
+
 struct CombineArgs {
     const int64_t* row;
     const int32_t* col;
@@ -1066,6 +1310,27 @@ cudaError_t launch_blocked_typed(gila_graph* g, const BlockedArgs& B, const Comb
 }
 
 template <class T, int MODEL, bool COMP>
+cudaError_t launch_rows(gila_graph* g, const RowsArgs& R, const TilePlan& P)
+{
+    static std::atomic<uint64_t> configured{0};  // one bit per device; callers may race
+    const uint64_t bit = 1ull << (g->device & 63);
+    if (!(configured.load() & bit)) {
+        cudaError_t e = cudaFuncSetAttribute(rows_kernel<T, MODEL, COMP>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kSmemCap - 4096);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    cudaEvent_t pa = prof_kernel_begin(g);
+    rows_kernel<T, MODEL, COMP>
+        <<<P.nb, kRowThreads, ((size_t)P.tv + 1) * 2 * sizeof(T), g->stream>>>(R);
+    count_launch();
+    cudaError_t e = cudaGetLastError();
+    prof_kernel_end(g, pa, "blocked_kernel (window, row per lane)");
+    return e;
+}
+
+template <class T, int MODEL, bool COMP>
 cudaError_t launch_pair(gila_graph* g, const BlockedArgs& B, const CombineArgs& C, int grid,
                         size_t smem, cudaStream_t st, int device, bool win)
 {
@@ -1342,6 +1607,8 @@ void free_tile_plans(gila_graph* g)
         cudaFree(P.hubs);
         cudaFree(P.wtile);
         cudaFree(P.rowspan);
+        cudaFree(P.sdesc);
+        cudaFree(P.deg);
         cudaFree(P.bdesc);
         cudaFree(P.rdir);
         cudaFree(P.blk);
@@ -1479,6 +1746,124 @@ size_t window_smem(int64_t wmax, int64_t rmax, size_t esz)
            (size_t)rmax * 2 * esz;
 }
 
+// Window mode with a row per lane (rows_kernel): ranges of whole slices with
+// a window each, where every window fits, the slices' padding stays within
+// kRowPadding of the lists (rows of about equal length), no adjacency row is
+// longer than kRowMaxDeg, and every row's neighbours are among its k-hop ids
+// (checked while the slices are filled). *done = false leaves the graph to
+// the shares of blocked_kernel. krow and span: the lists' offsets and the
+// rows' first and last ids, on the host.
+gila_status plan_rows(gila_graph* g, size_t esz, TilePlan& P, const std::vector<int64_t>& krow,
+                      const std::vector<int32_t>& span, bool* done)
+{
+    *done = false;
+    const int64_t n = g->n, nsl = (n + 31) / 32;
+    std::vector<int64_t> arow((size_t)n + 1);
+    GILA_CUDA(cudaMemcpyAsync(arow.data(), g->row, sizeof(int64_t) * (n + 1),
+                              cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));
+    std::vector<int32_t> sd(4 * (size_t)nsl);
+    std::vector<int64_t> pre((size_t)nsl + 1, 0);
+    int64_t units = 0;
+    for (int64_t s = 0; s < nsl; ++s) {
+        int64_t most = 0;
+        for (int64_t u = s * 32; u < std::min<int64_t>(n, s * 32 + 32); ++u) {
+            most = std::max<int64_t>(most, krow[(size_t)u + 1] - krow[(size_t)u]);
+            if (arow[(size_t)u + 1] - arow[(size_t)u] > kRowMaxDeg) return GILA_OK;
+        }
+        const int64_t steps = (most + 3) / 4;
+        if (units + steps > INT32_MAX) return GILA_OK;
+        sd[4 * (size_t)s] = (int32_t)units;
+        sd[4 * (size_t)s + 1] = (int32_t)steps;
+        units += steps;
+        // a slice costs its steps and about two more (positions, the move)
+        pre[(size_t)s + 1] = pre[(size_t)s] + steps + 2;
+    }
+    if ((double)units * 128.0 > kRowPadding * (double)g->nnz_khop) return GILA_OK;
+    const bool automatic = g->tune.tiled < 0;
+    if (automatic && (double)g->nnz_khop > kRowMeanLen * (double)n) return GILA_OK;
+    // two CTAs per SM, resident together, at least about 16 steps per warp of
+    // a CTA; more and shorter ranges where their windows are too wide for two
+    // CTAs' shared memory, or, failing that, for one's
+    const int64_t by_work = std::max<int64_t>(1, pre[(size_t)nsl] / (kRowWarps * 16));
+    const int64_t base_target = std::min<int64_t>(blocks_target(g, true), by_work);
+    std::vector<int32_t> rs;
+    std::vector<int64_t> wb;
+    int64_t nr = 0, wmax = 0, wsum = 0;
+    auto windows = [&](int64_t target) {
+        rs = partition_blocks(pre, nsl, 1, target, nsl)[0];
+        nr = (int64_t)rs.size() - 1;
+        wb.assign(2 * (size_t)nr, 0);
+        wmax = wsum = 0;
+        for (int64_t r = 0; r < nr; ++r) {
+            const int64_t u0 = (int64_t)rs[(size_t)r] * 32;
+            const int64_t u1 = std::min<int64_t>(n, (int64_t)rs[(size_t)r + 1] * 32);
+            int64_t lo = INT64_MAX, hi = -1;
+            for (int64_t u = u0; u < u1; ++u) {
+                lo = std::min<int64_t>(lo, span[2 * (size_t)u]);
+                hi = std::max<int64_t>(hi, span[2 * (size_t)u + 1]);
+            }
+            if (hi < 0) lo = hi = u0;  // no entries: a one-id window
+            const int64_t base = lo & ~int64_t(1);  // even: a 16-byte aligned float2 window
+            wb[2 * (size_t)r] = base;
+            wb[2 * (size_t)r + 1] = hi - base + 1;
+            wmax = std::max<int64_t>(wmax, hi - base + 1);
+            wsum += hi - base + 1;
+        }
+    };
+    bool fits = false;
+    for (int one = 0; one < 2 && !fits; ++one)
+        for (int64_t m = 1; m <= 16 && !fits; m *= 2) {
+            windows(base_target * m);
+            fits = wmax <= kMaxTile &&  // 16-bit relative ids
+                   (size_t)(wmax + 1) * esz <= (one ? (size_t)(kSmemCap - 4096) : kRowWindow);
+        }
+    if (!fits) return GILA_OK;
+    // the windows (from L2) against the id stream
+    if (automatic && wsum * (int64_t)esz > kRowWindowBytes * g->nnz_khop) return GILA_OK;
+    std::vector<int32_t> bdesc(4 * (size_t)nr, 0);
+    for (int64_t r = 0; r < nr; ++r) {
+        bdesc[4 * (size_t)r] = rs[(size_t)r] * 32;
+        bdesc[4 * (size_t)r + 1] =
+            (int32_t)std::min<int64_t>(n, (int64_t)rs[(size_t)r + 1] * 32);
+        for (int64_t s = rs[(size_t)r]; s < rs[(size_t)r + 1]; ++s) {
+            sd[4 * (size_t)s + 2] = (int32_t)wb[2 * (size_t)r];
+            sd[4 * (size_t)s + 3] = (int32_t)wb[2 * (size_t)r + 1];
+        }
+    }
+    gila_status s;
+    const size_t sd_bytes = sizeof(int32_t) * sd.size();
+    if ((s = ensure((void**)&P.sdesc, &P.sdesc_cap, sd_bytes + 16)) != GILA_OK ||
+        (s = ensure((void**)&P.deg, &P.deg_cap, sizeof(uint16_t) * (size_t)n)) != GILA_OK ||
+        (s = ensure((void**)&P.tk, &P.tk_cap, (size_t)units * 256 + 16)) != GILA_OK ||
+        (s = ensure((void**)&P.bdesc, &P.bdesc_cap, sizeof(int32_t) * bdesc.size())) != GILA_OK ||
+        (s = ensure((void**)&P.wtile, &P.wtile_cap, sizeof(int64_t) * wb.size())) != GILA_OK)
+        return s;
+    int* bad = reinterpret_cast<int*>(reinterpret_cast<char*>(P.sdesc) + sd_bytes);
+    GILA_CUDA(cudaMemcpyAsync(P.sdesc, sd.data(), sd_bytes, cudaMemcpyHostToDevice, g->stream));
+    GILA_CUDA(cudaMemcpyAsync(P.bdesc, bdesc.data(), sizeof(int32_t) * bdesc.size(),
+                              cudaMemcpyHostToDevice, g->stream));
+    GILA_CUDA(cudaMemcpyAsync(P.wtile, wb.data(), sizeof(int64_t) * wb.size(),
+                              cudaMemcpyHostToDevice, g->stream));
+    GILA_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), g->stream));
+    rows_fill_kernel<<<(unsigned)((nsl + 3) / 4), 128, 0, g->stream>>>(
+        n, nsl, g->row, g->col, g->krow, g->kcol, reinterpret_cast<const int4*>(P.sdesc), P.tk,
+        P.deg, bad);
+    count_launch();
+    GILA_CUDA(cudaGetLastError());
+    int h_bad = 0;
+    GILA_CUDA(cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));  // the host vectors go out of scope too
+    if (h_bad) return GILA_OK;
+    P.nt = 1;
+    P.nb = (int32_t)nr;
+    P.tv = (int32_t)wmax;
+    P.rmax = 0;
+    P.window = P.rows = P.use = true;
+    *done = true;
+    return GILA_OK;
+}
+
 // Window mode: rows are cut into ranges, and each range's rows, whose k-hop
 // ids span a window [b, b + len) of consecutive ids narrow enough for
 // shared memory (meshes, grids, locality-preserving orders, and every graph
@@ -1506,6 +1891,8 @@ gila_status plan_window(gila_graph* g, size_t esz, TilePlan& P, bool* fits,
     GILA_CUDA(cudaMemcpyAsync(span.data(), P.rowspan, sizeof(int32_t) * 2 * n,
                               cudaMemcpyDeviceToHost, g->stream));
     GILA_CUDA(cudaStreamSynchronize(g->stream));
+    bool done = false;
+    if ((s = plan_rows(g, esz, P, krow, span, &done)) != GILA_OK || done) return s;
     len.assign((size_t)n, 0);
     std::vector<int64_t> pre((size_t)n + 1, 0);
     for (int64_t u = 0; u < n; ++u) {
@@ -1693,6 +2080,7 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
     P.ready = true;
     P.use = false;
     P.window = false;
+    P.rows = false;
     const int64_t n = g->n;
     if (n == 0 || g->nnz_khop == 0 || g->tune.tiled == 0) return GILA_OK;
     // tiles for a row directory of rmax entries: positions per tile (one
@@ -1721,7 +2109,7 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
             std::vector<int32_t> rs;
             int64_t wmax = 0, rmax = 0;
             gila_status s = plan_window(g, esz, P, &fits, len, rs, wb, &wmax, &rmax);
-            if (s != GILA_OK) return s;
+            if (s != GILA_OK || P.rows) return s;
             if (fits) {
                 if ((s = build_layout(g, esz, P, 1, 0, len, {rs}, &wb)) != GILA_OK) return s;
                 P.window = true;
@@ -1818,6 +2206,39 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
         if (s != GILA_OK) return s;
     }
     if (!P.use || ((uintptr_t)pos_in & 15) != 0) return GILA_OK;
+    if (P.rows) {
+        RowsArgs R;
+        R.tk = P.tk;
+        R.sdesc = reinterpret_cast<const int4*>(P.sdesc);
+        R.deg = P.deg;
+        R.bdesc = reinterpret_cast<const int4*>(P.bdesc);
+        R.wbase = P.wtile;
+        R.n = g->n;
+        R.q = prm->q;
+        R.p = prm->p;
+        R.c = force_consts(prm->d, t);
+        R.pos = pos_in;
+        R.pos_out = pos_out;
+        R.disp_out = disp_out;
+        R.wait_ns = g->wait_test ? kTestWaitNs : kWaitNs;
+        R.skip_copy = g->wait_test ? 1 : 0;
+        const bool fr = prm->p == 2 && prm->q == 1;
+        cudaError_t e;
+        switch (prm->precision) {
+        case GILA_FP64:
+            e = fr ? launch_rows<double, kFR, false>(g, R, P) : launch_rows<double, kGeneric, false>(g, R, P);
+            break;
+        case GILA_FP32_COMPENSATED:
+            e = fr ? launch_rows<float, kFR, true>(g, R, P) : launch_rows<float, kGeneric, true>(g, R, P);
+            break;
+        default:
+            e = fr ? launch_rows<float, kFR, false>(g, R, P) : launch_rows<float, kGeneric, false>(g, R, P);
+            break;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "rows_kernel");
+        *handled = true;
+        return GILA_OK;
+    }
     BlockedArgs B;
     B.tk = P.tk;
     B.toff = P.toff;

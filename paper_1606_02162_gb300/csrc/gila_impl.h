@@ -122,6 +122,12 @@ struct TilePlan {
     size_t wtile_cap = 0;
     int32_t* rowspan = nullptr;      // 2 n: first and last id of each row (plan scratch)
     size_t rowspan_cap = 0;
+    // window mode with a row per lane: slices of 32 consecutive rows
+    bool rows = false;
+    int32_t* sdesc = nullptr;        // 4 per slice: start in tk (units of 128 ids), steps of
+    size_t sdesc_cap = 0;            // four ids a lane, window's first id and length
+    uint16_t* deg = nullptr;         // n: adjacency degrees (their ids come first in the rows)
+    size_t deg_cap = 0;
 };
 
 struct ProfileRec {

@@ -51,3 +51,52 @@ def test_edge_figures(g, p):
                                         torch.tensor(pos, dtype=dt, device="cuda"))
         for key in ("edge_mean", "edge_std", "edge_cv", "rep_total", "att_total"):
             assert abs(got[key] - want[key]) <= 1e-11 * max(1.0, abs(want[key])), (key, prec)
+
+
+def mesh_with_tail(rows, cols, extra):
+    """A triangulated mesh followed by `extra` vertices without edges."""
+    m = I.tri_mesh(rows, cols)
+    a, b = m.edge_list()
+    return I.csr_from_edges(m.n + extra, a, b)
+
+
+def unsorted_rows(g):
+    """The same graph with every adjacency row in descending order."""
+    col = g.col_idx.copy()
+    for u in range(g.n):
+        col[g.row_ptr[u]:g.row_ptr[u + 1]] = col[g.row_ptr[u]:g.row_ptr[u + 1]][::-1]
+    return I.Graph(g.name, g.n, g.row_ptr, col)
+
+
+# rows of one, two, nine and more steps; a last slice of 1, 31 and 32 rows;
+# empty slices; k-hop rows longer than the adjacency's; an unsorted adjacency,
+# which the row-per-lane plan refuses
+@pytest.mark.parametrize("name,g,k,rows", [
+    ("path", I.path(1025), 2, True), ("cycle", I.cycle(2047), 3, True),
+    ("grid", I.grid(40, 41), 1, True), ("mesh", I.tri_mesh(61, 67), 3, True),
+    ("mesh_k5", I.tri_mesh(100, 90), 5, True), ("tail", mesh_with_tail(50, 64, 100), 2, True),
+    ("unsorted", unsorted_rows(I.grid(40, 41)), 2, False), ("short", I.path(33), 2, False),
+    ("star", I.star(300), 1, False),
+], ids=lambda v: v if isinstance(v, str) else "")
+@pytest.mark.parametrize("pq", [(2, 1), (3, 2)], ids=["fr", "p3q2"])
+def test_row_per_lane_step(name, g, k, rows, pq):
+    import torch
+    p, q = pq
+    pos = I.uniform_positions(g.n, 21).astype(np.float32).astype(np.float64)
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, k)
+    t = 0.3
+    _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, t, d=1.2, p=p, q=q)
+    for prec in TOL:
+        dt = torch.float64 if prec == G.GILA_FP64 else torch.float32
+        with G.Graph.from_inputs(g) as h:
+            G.gila_graph_tune(h.handle, tiled=1)
+            G.gila_profile_enable(h.handle, 2)
+            x = torch.tensor(pos, dtype=dt, device="cuda")
+            y, disp = torch.empty_like(x), torch.empty_like(x)
+            G.gila_layout_step(h.handle, G.params(k=k, d=1.2, p=p, q=q, precision=prec), t, x, y,
+                               disp)
+            torch.cuda.synchronize()
+            kernel = G.gila_profile_read_kernel(h.handle)["name"]
+        assert ("row per lane" in kernel) == rows, kernel
+        assert torch.equal(y, x + disp)
+        assert np.abs(disp.double().cpu().numpy() - want).max() <= TOL[prec] * np.abs(want).max()
