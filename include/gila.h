@@ -248,8 +248,9 @@ gila_status gila_layout_metrics(gila_graph* g, const gila_params* prm, const voi
  * Batches: many independent graphs laid out together (thousands of small
  * graphs of uneven sizes). The batch is the disjoint union of
  * its graphs, so one k-hop build serves all of them; the layouts then run in
- * one persistent kernel launch in which each CTA takes one graph at a time
- * and carries it through all iterations with its placement staged in shared
+ * one persistent kernel launch (two, side by side, where some graphs have long
+ * rows) in which a CTA or a cluster of CTAs takes one graph at a time and
+ * carries it through all iterations with its placement staged in shared
  * memory. The launch is captured in a CUDA graph and replayed while the
  * arguments stay the same. Every graph follows its own temperature schedule
  * (default t0 from its own n and initial bounding box). A graph's result
@@ -263,6 +264,9 @@ typedef struct gila_batch gila_batch;
 typedef struct gila_batch_tuning {
     int32_t threads;     /* threads per CTA: 256, 512 or 1024; 0 = 512 */
     int32_t ctas_per_sm; /* CTAs per SM (1..8); 0 = 2 when two graphs fit in shared memory */
+    /* all three 0 (default): graphs of short rows (mean at most 64) take a lane
+       per vertex, the others the groups below; any of them set: every graph
+       takes groups */
     int32_t group4_max;  /* graphs whose mean k-hop row length is <= this use 4 lanes per
                             vertex; 0 = 8 */
     int32_t group8_max;  /* ... 8 lanes; 0 = 24 */

@@ -2,27 +2,28 @@
 //
 // A batch is the disjoint union of its graphs (ids offset per graph), so one
 // k-hop build serves all of them. The layout of every graph then runs inside
-// a single CTA from its first to its last iteration: the CTA stages the
-// graph's placement in shared memory (two buffers, Jacobi), streams the
-// graph's k-hop rows (small enough to stay in L2 across iterations) and
-// separates iterations with __syncthreads, so no grid-wide barrier and no
-// per-iteration launch exists. CTAs take graphs from a global counter,
-// largest first. Graphs too large for shared memory iterate on two global
-// buffers in the same way.
-//
-// Lanes per vertex (4, 8, 16 or 32) follow the graph's own mean k-hop row
-// length; a graph's result therefore does not depend on the other graphs of
-// the batch. The temperature of each graph follows its own schedule: the
-// default t0 uses that graph's n (and, for geometric cooling, the aspect of
-// its own initial bounding box).
+// a single CTA, or a cluster of CTAs, from its first to its last iteration:
+// the placement is staged in shared memory (two buffers, Jacobi), the graph's
+// k-hop rows are streamed (small enough to stay in L2 across iterations), and
+// iterations are separated by a block barrier or an exchange within the
+// cluster, so no grid-wide barrier and no per-iteration launch exists. CTAs
+// take graphs from global counters, largest first. Graphs of short rows take
+// a lane per row (batch_rows_kernel); the others take 4, 8, 16 or 32 lanes per
+// vertex by their own mean row length (batch_kernel), and those too large for
+// shared memory iterate on two global buffers in the same way. A graph's
+// result does not depend on the other graphs of the batch. The temperature of
+// each graph follows its own schedule: the default t0 uses that graph's n
+// (and, for geometric cooling, the aspect of its own initial bounding box).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
 #include <numeric>
 #include <string>
+#include <type_traits>
 #include <vector>
 
+#include "device_util.cuh"
 #include "force.cuh"
 #include "gila_impl.h"
 
@@ -30,6 +31,7 @@ struct gila_batch {
     gila_graph* g = nullptr;  // disjoint union of the graphs
     int32_t count = 0;
     std::vector<int64_t> voff_h;  // vertex offsets, count + 1
+    std::vector<int32_t> order_h; // graphs, largest first
     int64_t* voff = nullptr;
     int32_t* order = nullptr;     // graphs in processing order
     int* work = nullptr;          // next position in `order`
@@ -48,6 +50,27 @@ struct gila_batch {
     cudaGraphExec_t exec = nullptr;
     std::vector<unsigned char> exec_key;  // arguments the captured graph was made with
     gila_batch_tuning tune = {0, 0, 0, 0, 0};
+    // row-per-lane plan of the current k-hop lists, by position width
+    // (0: float2, 1: double2; the widths share the arrays, see batch_plan)
+    int64_t plan_serial = -1;      // the build it was made for
+    std::vector<int32_t> big[2], small[2], rest[2];  // graphs by the form that serves them
+    int64_t max_rows_n[2] = {0, 0};                  // largest graph of big and small
+    int cluster[2] = {1, 1};                         // CTAs of a cluster
+    int32_t* rorder[2] = {nullptr, nullptr};         // big, small, rest
+    int32_t* soff = nullptr;
+    int32_t* sgraph = nullptr;
+    int32_t* base = nullptr;
+    int32_t* units = nullptr;
+    uint8_t* skip = nullptr;       // 2 count: skip, bad
+    int2* sdesc = nullptr;
+    uint16_t* deg = nullptr;
+    uint16_t* perm = nullptr;
+    uint16_t* rank = nullptr;
+    uint16_t* cuts = nullptr;
+    uint16_t* tk = nullptr;
+    size_t tk_cap = 0;
+    cudaStream_t side = nullptr;   // capture fork: the group kernel beside the row-per-lane one
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 namespace gila {
@@ -91,7 +114,7 @@ template <class T, int MODEL, bool COMP>
 __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 {
     using P2 = typename V2<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_g;
     __shared__ double s_box[32][4];
     P2* sbuf0 = reinterpret_cast<P2*>(smem_raw);
@@ -220,6 +243,509 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
     }
 }
 
+// Row-per-lane form of the batched layout, for graphs of short rows. At plan
+// time (once per k-hop build) each graph's vertices are sorted by row length,
+// and 32 consecutive ones of that order form a slice, stored step-major (four
+// 16-bit ids of every lane, 256 bytes a step) and padded to the slice's
+// longest row with the id of a far slot. A row's first ids are its neighbours,
+// whose attraction is formed from the same shared-memory positions. A lane
+// sums its row in registers and moves its vertex: no reduction over lanes, no
+// lane without a row in the finish (a square root and a division per vertex,
+// which a group of eight lanes issued for four vertices at a time), and ids
+// that arrive as 16-byte-aligned streams ahead of their use.
+//
+// CTAs come in clusters of 1, 2, 4 or 8. A graph that would keep one CTA busy
+// for longer than its share of the batch is taken by a whole cluster: every
+// CTA holds the placement, computes a contiguous part of the slices (equal
+// steps), and pushes its new positions into the other CTAs' shared memory
+// with bulk copies that complete on their mbarriers, one mbarrier per parity
+// of the iteration (a CTA can be at most one iteration ahead of another: it
+// needs the other's positions to go on). After the large graphs each CTA
+// takes small ones on its own. The order of a row's additions is the same in
+// every case and depends on the graph alone.
+//
+// Against groups of lanes per vertex (batch_kernel, which the longer rows
+// keep), whose bound was the latency of one group's chain (offsets, ids,
+// positions, reduction) and, in FP64, lanes without work on the two FP64
+// operations a clock of an SM: 500 graphs of 50..5000 vertices, k = 2, 50
+// iterations in FP32 6.5 -> 0.60 ms, 3000 graphs 9.2 -> 1.6 ms (30
+// iterations), 250 graphs in FP64 20.8 -> 3.9 ms (20 iterations; its FP64
+// pipe is 63% busy, the FP32 form issues in 52% of the cycles, the rest mostly
+// the barrier between iterations).
+constexpr int kBrCluster = 8;             // largest cluster
+constexpr int kBrBins = 1024;             // row lengths told apart by the sort
+constexpr int64_t kBrMeanLen = 64;        // longest mean row taken
+constexpr double kBrPadding = 2.0;        // most slots per entry
+constexpr int kBrAhead = 4;               // steps of ids in registers ahead
+constexpr int kBrSmem = 227 * 1024 - 2048;
+// fewest slices worth a cluster: below, an exchange an iteration costs more
+// than the split saves (FP64 slices take about ten times as long)
+constexpr int64_t kBrBigSlices[2] = {16, 4};
+constexpr uint64_t kBrWaitNs = 1000000000ull;  // bound on a wait for peers' positions
+
+// Set when a wait for peers' positions ran out; read and cleared by the next
+// synchronising batch call.
+__device__ int g_batch_wait_failed = 0;
+
+struct BatchRowsArgs {
+    const int64_t* voff;
+    const int32_t* order;    // large graphs, then small ones, largest first
+    int32_t nbig, nall;
+    const int32_t* soff;     // first slice of every graph
+    const int2* sdesc;       // per slice: start in tk (units of 128 ids), steps
+    const uint16_t* deg;     // adjacency degrees in sorted order
+    const uint16_t* perm;    // vertex of each place of the sorted order
+    const uint16_t* cuts;    // kBrCluster + 1 slice bounds per graph
+    const uint16_t* tk;
+    int* work;               // next large, next small
+    const double* geo;
+    int iters, schedule;
+    double d, t0;
+    ForceConsts c;           // its t is unused: every graph cools on its own
+    int p, q;
+    void* pos;
+    int stride;              // positions per buffer, far slot included (even)
+    uint64_t wait_ns;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t cluster_size()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(r));
+    return r;
+}
+
+// Address in CTA `rank`'s shared memory of the same place as `a` in this one's.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+
+// Bulk copy from this CTA's shared memory to another's, completing on the
+// other's mbarrier.
+__device__ __forceinline__ void bulk_s2s(uint32_t dst_cluster, uint32_t src, uint32_t bytes,
+                                         uint32_t bar_cluster)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+            "r"(dst_cluster),
+        "r"(src), "r"(bytes), "r"(bar_cluster)
+        : "memory");
+}
+
+template <class T, int MODEL, bool COMP>
+__global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
+{
+    using P2 = typename V2<T>::type;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ int s_g;
+    __shared__ double s_t0;
+    __shared__ T s_t[2];  // this and the next iteration's temperature
+    __shared__ double s_box[32][4];
+    P2* const buf0 = reinterpret_cast<P2*>(smem_raw);
+    P2* const buf1 = buf0 + A.stride;
+    P2* const gpos = reinterpret_cast<P2*>(A.pos);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t rank = cluster_rank(), csize = cluster_size();
+    if (threadIdx.x == 0) {
+        mbar_init(&s_bar[0], 1);
+        mbar_init(&s_bar[1], 1);
+    }
+    uint32_t done_iters = 0;  // iterations exchanged so far: parity and phase of the mbarriers
+    bool failed = false;
+
+    // one graph, its slices [s0 + ca, s0 + cb) on this CTA
+    auto layout = [&](int gid, bool big) {
+        const int64_t v0 = A.voff[gid];
+        const int n = (int)(A.voff[gid + 1] - v0);
+        const int npad = (n + 31) & ~31;
+        const int s0 = A.soff[gid];
+        const int ns = npad >> 5;
+        const uint16_t* cuts = A.cuts + (kBrCluster + 1) * (int64_t)gid;
+        const int part = kBrCluster / (int)csize;  // eighths of the graph per CTA
+        const int ca = big ? cuts[rank * part] : 0;
+        const int cb = big ? cuts[(rank + 1) * part] : ns;
+        const uint16_t* perm = A.perm + v0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) buf0[i] = gpos[v0 + perm[i]];
+        if (threadIdx.x == 0) {
+            P2 far;
+            far.x = FarSlot<T>::v;
+            far.y = FarSlot<T>::v;
+            buf0[npad] = far;
+            buf1[npad] = far;
+        }
+        __syncthreads();
+        // initial temperature of this graph
+        if (!(A.t0 > 0.0) && A.schedule == GILA_COOL_GEOMETRIC) {
+            double x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                const P2 p = buf0[i];
+                x0 = fmin(x0, (double)p.x);
+                x1 = fmax(x1, (double)p.x);
+                y0 = fmin(y0, (double)p.y);
+                y1 = fmax(y1, (double)p.y);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                x0 = fmin(x0, __shfl_xor_sync(kFull, x0, o));
+                x1 = fmax(x1, __shfl_xor_sync(kFull, x1, o));
+                y0 = fmin(y0, __shfl_xor_sync(kFull, y0, o));
+                y1 = fmax(y1, __shfl_xor_sync(kFull, y1, o));
+            }
+            if (lane == 0) {
+                s_box[warp][0] = x0;
+                s_box[warp][1] = x1;
+                s_box[warp][2] = y0;
+                s_box[warp][3] = y1;
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            double t0 = A.t0;
+            if (!(t0 > 0.0)) {
+                t0 = 0.1 * sqrt((double)n);
+                if (A.schedule == GILA_COOL_GEOMETRIC) {
+                    double x0 = s_box[0][0], x1 = s_box[0][1], y0 = s_box[0][2], y1 = s_box[0][3];
+                    for (int w = 1; w < nwarps; ++w) {
+                        x0 = fmin(x0, s_box[w][0]);
+                        x1 = fmax(x1, s_box[w][1]);
+                        y0 = fmin(y0, s_box[w][2]);
+                        y1 = fmax(y1, s_box[w][3]);
+                    }
+                    const double w = x1 - x0, h = y1 - y0;
+                    const double a = (w > 0.0 && h > 0.0) ? h / w : 1.0;
+                    t0 = sqrt((double)n * A.d / a);
+                }
+            }
+            s_t0 = t0;
+            s_t[0] = (T)(A.schedule == GILA_COOL_GEOMETRIC
+                             ? t0 * A.geo[0]
+                             : t0 * (double)A.iters / (double)A.iters);
+        }
+        __syncthreads();
+        Rep<T, MODEL, COMP, kSrcShared, true> f;
+        f.d2 = T(1);
+        f.q = A.q;
+        Att<T, MODEL, COMP, kSrcShared> att;
+        att.inv_d = const_inv_d<T>(A.c);
+        att.p = A.p;
+        const T d2 = const_d2<T>(A.c);
+        P2* cur = buf0;
+        P2* nxt = buf1;
+        const uint2* ids = reinterpret_cast<const uint2*>(A.tk) + lane;
+        const int first = ca + warp;  // this warp's slices: first, first + nwarps, ...
+        int2 sd = make_int2(0, 0);
+        uint2 next[kBrAhead];
+        if (first < cb) {
+            sd = A.sdesc[s0 + first];
+#pragma unroll
+            for (int i = 0; i < kBrAhead; ++i)
+                if (i < sd.y) next[i] = ld_ids2(ids + 32 * ((int64_t)sd.x + i));
+        }
+        for (int it = 0; it < A.iters; ++it) {
+            const T t = s_t[it & 1];
+            if (threadIdx.x == 0 && it + 1 < A.iters)
+                s_t[(it + 1) & 1] = (T)(A.schedule == GILA_COOL_GEOMETRIC
+                                            ? s_t0 * A.geo[it + 1]
+                                            : s_t0 * (double)(A.iters - it - 1) / (double)A.iters);
+            f.src.set_shared(cur, 0u);
+            att.src.set_shared(cur, 0u);
+            for (int s = first; s < cb; s += nwarps) {
+                const int i = s * 32 + lane;
+                const bool live = i < n;
+                P2 pu;
+                pu.x = T(0);
+                pu.y = T(0);
+                int deg = 0;
+                if (live) {
+                    pu = cur[i];
+                    deg = A.deg[v0 + i];
+                }
+                f.xu = att.xu = pu.x;
+                f.yu = att.yu = pu.y;
+                const int dmax = __reduce_max_sync(kFull, deg);
+                const int steps = sd.y;
+                const int64_t start = sd.x;
+                // the slice after this one: the warp's next, or its first
+                // again for the next iteration
+                const int2 sn = A.sdesc[s0 + (s + nwarps < cb ? s + nwarps : first)];
+                Acc<T, COMP> acc, at;
+                for (int k0 = 0; k0 < steps || k0 == 0; k0 += kBrAhead) {
+                    uint2 c4[kBrAhead];
+#pragma unroll
+                    for (int x = 0; x < kBrAhead; ++x) c4[x] = next[x];
+                    const bool more = k0 + kBrAhead < steps;
+                    const int64_t from = more ? start + k0 + kBrAhead : (int64_t)sn.x;
+                    const int left = more ? steps - k0 - kBrAhead : sn.y;
+#pragma unroll
+                    for (int x = 0; x < kBrAhead; ++x)
+                        if (x < left) next[x] = ld_ids2(ids + 32 * (from + x));
+                    Acc<T, false> pend;
+#pragma unroll
+                    for (int x = 0; x < kBrAhead; ++x) {
+                        if (k0 + x >= steps) break;
+                        const uint32_t i0 = c4[x].x & 0xffffu, i1 = c4[x].x >> 16;
+                        const uint32_t i2 = c4[x].y & 0xffffu, i3 = c4[x].y >> 16;
+                        if constexpr (COMP) {
+                            f(i0, pend);
+                            f(i1, pend);
+                            f(i2, pend);
+                            f(i3, pend);
+                        } else {
+                            f(i0, acc);
+                            f(i1, acc);
+                            f(i2, acc);
+                            f(i3, acc);
+                        }
+                        const int e = 4 * (k0 + x);
+                        if (e < dmax) {  // the rows' first ids are their neighbours
+                            if (e < deg) att(i0, at);
+                            if (e + 1 < deg) att(i1, at);
+                            if (e + 2 < deg) att(i2, at);
+                            if (e + 3 < deg) att(i3, at);
+                        }
+                    }
+                    if constexpr (COMP) add_compensated(acc, pend.sx, pend.sy);
+                }
+                acc.sx *= d2;
+                acc.sy *= d2;
+                acc.cx *= d2;
+                acc.cy *= d2;
+                acc.merge(at.sx, at.sy, at.cx, at.cy);
+                T mx, my;
+                capped<T>(t, acc.fx(), acc.fy(), mx, my);
+                P2 o;
+                o.x = pu.x + mx;
+                o.y = pu.y + my;
+                nxt[i] = o;
+                sd = sn;
+            }
+            if (big) {
+                // push this CTA's new positions to its peers and wait for theirs
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncthreads();
+                uint64_t* bar = &s_bar[done_iters & 1];
+                const uint32_t mine = (uint32_t)(cb - ca) * 32u * (uint32_t)sizeof(P2);
+                if (threadIdx.x == 0)
+                    mbar_arrive_expect_tx(bar, (uint32_t)npad * (uint32_t)sizeof(P2) - mine);
+                if (threadIdx.x == 0 && mine > 0 && !failed) {
+                    const uint32_t src = smem_addr(nxt + ca * 32), b = smem_addr(bar);
+                    for (uint32_t r = 1; r < csize; ++r) {
+                        const uint32_t to = (rank + r) & (csize - 1);
+                        bulk_s2s(cluster_map(src, to), src, mine, cluster_map(b, to));
+                    }
+                }
+                if (!failed && !mbar_wait(bar, (done_iters >> 1) & 1, A.wait_ns)) {
+                    // give up: flag it, let what is in flight land (bounded),
+                    // push and wait no more; the cluster leaves together
+                    failed = true;
+                    atomicExch(&g_batch_wait_failed, 1);
+                    mbar_wait(bar, (done_iters >> 1) & 1, A.wait_ns);
+                }
+                ++done_iters;
+                // s_t of the next iteration is visible: written before the
+                // __syncthreads above
+            } else {
+                __syncthreads();
+            }
+            P2* x = cur;
+            cur = nxt;
+            nxt = x;
+        }
+        for (int i = ca * 32 + threadIdx.x; i < n && i < cb * 32; i += blockDim.x)
+            gpos[v0 + perm[i]] = cur[i];
+    };
+
+    // large graphs, a cluster each
+    for (;;) {
+        cluster_sync();  // mbarriers initialised; every CTA is done with the graph before
+        if (rank == 0 && threadIdx.x == 0) {
+            const int g = atomicAdd(&A.work[0], 1);
+            const uint32_t a = smem_addr(&s_g);
+            for (uint32_t r = 0; r < csize; ++r)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(a, r)), "r"(g)
+                             : "memory");
+        }
+        cluster_sync();
+        const int gi = s_g;
+        if (gi >= A.nbig) break;  // uniform over the cluster
+        layout(A.order[gi], true);
+    }
+    // small graphs, a CTA each
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_g = atomicAdd(&A.work[1], 1);
+        __syncthreads();
+        const int gi = A.nbig + s_g;
+        if (gi >= A.nall) break;
+        layout(A.order[gi], false);
+    }
+}
+
+// First k-hop entry of every graph (count + 1 values).
+__global__ void graph_bounds_kernel(int32_t count, const int64_t* __restrict__ voff,
+                                    const int64_t* __restrict__ krow, int64_t* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i <= count) out[i] = krow[voff[i]];
+}
+
+// Plan, one block per graph: its vertices sorted by row length (longest
+// first; a counting sort, the order within a length left to the atomics: no
+// result depends on it), the steps of every slice and their starts within the
+// graph, the total, and the slice bounds of a cluster's CTAs (equal steps,
+// two more a slice for its positions and moves). Graphs with skip[g] set are
+// left out.
+__global__ void __launch_bounds__(256)
+batch_sort_kernel(const int64_t* __restrict__ voff, const int32_t* __restrict__ soff,
+                  const uint8_t* __restrict__ skip, const int64_t* __restrict__ krow,
+                  uint16_t* __restrict__ perm, uint16_t* __restrict__ rank,
+                  int2* __restrict__ sdesc, int32_t* __restrict__ units,
+                  uint16_t* __restrict__ cuts)
+{
+    __shared__ int hist[kBrBins];
+    __shared__ int wt[256 / 32 + 1];
+    const int g = blockIdx.x, tid = threadIdx.x;
+    if (skip[g]) return;
+    const int64_t v0 = voff[g];
+    const int n = (int)(voff[g + 1] - v0);
+    for (int b = tid; b < kBrBins; b += 256) hist[b] = 0;
+    __syncthreads();
+    auto bin = [&](int i) {
+        const int64_t len = krow[v0 + i + 1] - krow[v0 + i];
+        return kBrBins - 1 - (len < kBrBins ? (int)len : kBrBins - 1);
+    };
+    for (int i = tid; i < n; i += 256) atomicAdd(&hist[bin(i)], 1);
+    __syncthreads();
+    int carry = 0;
+    for (int b0 = 0; b0 < kBrBins; b0 += 256) {
+        const int c = hist[b0 + tid];
+        int total;
+        const int incl = block_inclusive_scan<int, 256>(c, wt, &total);
+        hist[b0 + tid] = carry + incl - c;
+        carry += total;
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += 256) {
+        const int at = atomicAdd(&hist[bin(i)], 1);
+        perm[v0 + at] = (uint16_t)i;
+        rank[v0 + i] = (uint16_t)at;
+    }
+    __syncthreads();
+    const int ns = (n + 31) >> 5;
+    int2* sd = sdesc + soff[g];
+    carry = 0;
+    for (int b0 = 0; b0 < ns; b0 += 256) {
+        const int s = b0 + tid;
+        int steps = 0;
+        if (s < ns) {
+            int64_t most = 0;
+            for (int i = s * 32; i < n && i < s * 32 + 32; ++i) {
+                const int64_t v = v0 + perm[v0 + i];
+                const int64_t len = krow[v + 1] - krow[v];
+                most = len > most ? len : most;
+            }
+            steps = (int)((most + 3) >> 2);
+        }
+        int total;
+        const int incl = block_inclusive_scan<int, 256>(steps, wt, &total);
+        if (s < ns) sd[s] = make_int2(carry + incl - steps, steps);
+        carry += total;
+    }
+    if (tid == 0) units[g] = carry;
+    __syncthreads();
+    if (tid <= kBrCluster) {
+        // the first slice whose cost before it reaches the share
+        const int64_t want = (int64_t)(carry + 2 * ns) * tid / kBrCluster;
+        int lo = 0, hi = ns;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sd[mid].x + 2 * mid < want) lo = mid + 1; else hi = mid;
+        }
+        cuts[(kBrCluster + 1) * g + tid] = (uint16_t)(tid == kBrCluster ? ns : lo);
+    }
+}
+
+// Plan, a warp per slice and a row per lane: the slice's start becomes its
+// place in tk, and its ids are written, neighbours first (both lists
+// ascending, one merge), then the rest, then the far slot's id. A row whose
+// neighbours are not all among its k-hop ids (an unsorted or repeated
+// adjacency, a self-loop) sets bad[g]: the graph keeps the group kernel.
+__global__ void __launch_bounds__(128)
+batch_fill_kernel(int64_t nslices, const int32_t* __restrict__ sgraph,
+                  const int64_t* __restrict__ voff, const int32_t* __restrict__ soff,
+                  const int32_t* __restrict__ base, const uint8_t* __restrict__ skip,
+                  const int64_t* __restrict__ row, const int32_t* __restrict__ col,
+                  const int64_t* __restrict__ krow, const uint32_t* __restrict__ kcol,
+                  const uint16_t* __restrict__ perm, const uint16_t* __restrict__ rank,
+                  int2* __restrict__ sdesc, uint16_t* __restrict__ deg_out,
+                  uint16_t* __restrict__ tk, uint8_t* __restrict__ bad)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= nslices) return;  // warp-uniform
+    const int g = sgraph[s];
+    if (skip[g]) return;
+    const int64_t v0 = voff[g];
+    const int n = (int)(voff[g + 1] - v0);
+    const int npad = (n + 31) & ~31;
+    int2 sd = sdesc[s];
+    __syncwarp();
+    sd.x += base[g];
+    if (lane == 0) sdesc[s] = sd;
+    const int i = (int)(s - soff[g]) * 32 + lane;
+    int64_t kb = 0, ke = 0, ab = 0;
+    int deg = 0;
+    if (i < n) {
+        const int64_t u = v0 + perm[v0 + i];
+        kb = krow[u];
+        ke = krow[u + 1];
+        ab = row[u];
+        const int64_t d64 = row[u + 1] - ab;
+        deg = d64 <= ke - kb ? (int)d64 : 0;
+        if (d64 != deg) bad[g] = 1;
+        deg_out[v0 + i] = (uint16_t)deg;
+    }
+    uint64_t* out = reinterpret_cast<uint64_t*>(tk) + (int64_t)sd.x * 32 + lane;
+    const int slots = sd.y * 4;
+    uint64_t four = 0;
+    int w = 0;
+    auto put = [&](uint32_t id) {
+        if (w >= slots) return;
+        four |= (uint64_t)(uint16_t)id << (16 * (w & 3));
+        if ((w & 3) == 3) {
+            out[32 * (w >> 2)] = four;
+            four = 0;
+        }
+        ++w;
+    };
+    for (int a = 0; a < deg; ++a) put(rank[col[ab + a]]);
+    int a = 0, found = 0;
+    for (int64_t x = kb; x < ke; ++x) {
+        const uint32_t id = kcol[x];
+        while (a < deg && (uint32_t)col[ab + a] < id) ++a;
+        if (a < deg && (uint32_t)col[ab + a] == id) ++found;
+        else put(rank[id]);
+    }
+    if (found != deg) bad[g] = 1;
+    while (w < slots) put((uint32_t)npad);
+}
+
 // Pack graphs given as device CSRs into the union CSR (one block per graph).
 struct PackSrc {
     const int64_t* row;
@@ -263,6 +789,33 @@ cudaError_t launch_batch(const BatchArgs& A, int grid, int threads, size_t smem,
     return cudaGetLastError();
 }
 
+template <class T, bool COMP>
+struct Form {
+    using type = T;
+    static constexpr bool comp = COMP;
+};
+
+template <class T, int MODEL, bool COMP>
+cudaError_t launch_batch_rows(const BatchRowsArgs& R, int grid, int cluster, int threads,
+                              size_t smem, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cluster;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, batch_rows_kernel<T, MODEL, COMP>, R);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // Shared-memory opt-in for every instantiation on the current device
 // (outside any stream capture); once per device, callers may race.
 cudaError_t configure_batch_kernels()
@@ -278,7 +831,10 @@ cudaError_t configure_batch_kernels()
 #define GILA_OPT_IN(T, M, C)                                                                 \
     if (e == cudaSuccess)                                                                    \
         e = cudaFuncSetAttribute(batch_kernel<T, M, C>,                                      \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 2048);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 2048);   \
+    if (e == cudaSuccess)                                                                    \
+        e = cudaFuncSetAttribute(batch_rows_kernel<T, M, C>,                                 \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kBrSmem);
     GILA_OPT_IN(float, kFR, false)
     GILA_OPT_IN(float, kGeneric, false)
     GILA_OPT_IN(float, kFR, true)
@@ -299,18 +855,22 @@ gila_status batch_finish_create(gila_batch* b)
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t c) {
         return b->voff_h[a + 1] - b->voff_h[a] > b->voff_h[c + 1] - b->voff_h[c];
     });
+    b->order_h = order;
     b->max_n = 0;
     for (int32_t i = 0; i < count; ++i)
         b->max_n = std::max<int64_t>(b->max_n, b->voff_h[i + 1] - b->voff_h[i]);
     GILA_CUDA(cudaMalloc(&b->voff, sizeof(int64_t) * (count + 1)));
     GILA_CUDA(cudaMalloc(&b->order, sizeof(int32_t) * std::max(count, 1)));
-    GILA_CUDA(cudaMalloc(&b->work, sizeof(int)));
+    GILA_CUDA(cudaMalloc(&b->work, sizeof(int) * 3));  // group kernel, large, small graphs
     GILA_CUDA(cudaMemcpy(b->voff, b->voff_h.data(), sizeof(int64_t) * (count + 1),
                          cudaMemcpyHostToDevice));
     if (count > 0)
         GILA_CUDA(cudaMemcpy(b->order, order.data(), sizeof(int32_t) * count,
                              cudaMemcpyHostToDevice));
     GILA_CUDA(cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking));
+    GILA_CUDA(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
+    GILA_CUDA(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
+    GILA_CUDA(cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
     GILA_CUDA(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
     GILA_CUDA(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
     return GILA_OK;
@@ -334,6 +894,170 @@ gila_status check_batch_params(const gila_params* p)
     return GILA_OK;
 }
 
+// The row-per-lane plan (see batch_rows_kernel), made once per k-hop build.
+// A graph takes it when its rows are short (mean at most kBrMeanLen: longer
+// rows keep groups of lanes), its slots at most kBrPadding per entry, its two
+// buffers fit shared memory, and its neighbours are among its k-hop ids. All
+// of that depends on the graph alone.
+gila_status batch_plan(gila_batch* b)
+{
+    gila_graph* g = b->g;
+    if (b->plan_serial == g->khop_serial) return GILA_OK;
+    b->plan_serial = -1;
+    const int32_t count = b->count;
+    cudaStream_t st = b->user;
+    const std::vector<int64_t>& vo = b->voff_h;
+    std::vector<int32_t> soff((size_t)count + 1, 0);
+    for (int32_t i = 0; i < count; ++i)
+        soff[(size_t)i + 1] = soff[(size_t)i] + (int32_t)((vo[(size_t)i + 1] - vo[(size_t)i] + 31) / 32);
+    const int64_t nsl = soff[(size_t)count];
+    if (!b->soff) {
+        std::vector<int32_t> sg((size_t)nsl);
+        for (int32_t i = 0; i < count; ++i)
+            std::fill(sg.begin() + soff[(size_t)i], sg.begin() + soff[(size_t)i + 1], i);
+        const size_t n1 = (size_t)std::max<int64_t>(g->n, 1), s1 = (size_t)std::max<int64_t>(nsl, 1);
+        GILA_CUDA(cudaMalloc(&b->sgraph, sizeof(int32_t) * s1));
+        GILA_CUDA(cudaMalloc(&b->sdesc, sizeof(int2) * s1));
+        GILA_CUDA(cudaMalloc(&b->base, sizeof(int32_t) * (size_t)count));
+        GILA_CUDA(cudaMalloc(&b->units, sizeof(int32_t) * (size_t)count));
+        GILA_CUDA(cudaMalloc(&b->skip, 2 * (size_t)count));
+        GILA_CUDA(cudaMalloc(&b->deg, sizeof(uint16_t) * n1));
+        GILA_CUDA(cudaMalloc(&b->perm, sizeof(uint16_t) * n1));
+        GILA_CUDA(cudaMalloc(&b->rank, sizeof(uint16_t) * n1));
+        GILA_CUDA(cudaMalloc(&b->cuts, sizeof(uint16_t) * (kBrCluster + 1) * (size_t)count));
+        for (int w = 0; w < 2; ++w)
+            GILA_CUDA(cudaMalloc(&b->rorder[w], sizeof(int32_t) * (size_t)count));
+        GILA_CUDA(cudaMemcpyAsync(b->sgraph, sg.data(), sizeof(int32_t) * (size_t)nsl,
+                                  cudaMemcpyHostToDevice, st));
+        int32_t* so = nullptr;
+        GILA_CUDA(cudaMalloc(&so, sizeof(int32_t) * ((size_t)count + 1)));
+        b->soff = so;  // last: marks the set complete
+        GILA_CUDA(cudaMemcpyAsync(so, soff.data(), sizeof(int32_t) * soff.size(),
+                                  cudaMemcpyHostToDevice, st));
+        GILA_CUDA(cudaStreamSynchronize(st));  // the host vectors go out of scope
+    }
+    // rows' totals per graph
+    std::vector<int64_t> koff((size_t)count + 1);
+    int64_t* dk = nullptr;
+    GILA_CUDA(cudaMalloc(&dk, sizeof(int64_t) * ((size_t)count + 1)));
+    graph_bounds_kernel<<<(unsigned)((count + 256) / 256), 256, 0, st>>>(count, b->voff, g->krow, dk);
+    count_launch();
+    cudaMemcpyAsync(koff.data(), dk, sizeof(int64_t) * koff.size(), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaStreamSynchronize(st);
+    cudaFree(dk);
+    if (e != cudaSuccess) return cuda_fail(e, "batch plan");
+    constexpr int64_t max_n = kBrSmem / 16 - 64;  // float2, two buffers and their far slots
+    std::vector<uint8_t> skip(2 * (size_t)count, 0);
+    for (int32_t i = 0; i < count; ++i) {
+        const int64_t n = vo[(size_t)i + 1] - vo[(size_t)i];
+        const int64_t nnz = koff[(size_t)i + 1] - koff[(size_t)i];
+        skip[(size_t)i] = n == 0 || n > max_n || nnz > kBrMeanLen * n;
+    }
+    std::vector<int32_t> units((size_t)count, 0), base((size_t)count, 0);
+    GILA_CUDA(cudaMemcpyAsync(b->skip, skip.data(), skip.size(), cudaMemcpyHostToDevice, st));
+    GILA_CUDA(cudaMemsetAsync(b->units, 0, sizeof(int32_t) * (size_t)count, st));
+    batch_sort_kernel<<<(unsigned)count, 256, 0, st>>>(b->voff, b->soff, b->skip, g->krow, b->perm,
+                                                       b->rank, b->sdesc, b->units, b->cuts);
+    count_launch();
+    GILA_CUDA(cudaGetLastError());
+    GILA_CUDA(cudaMemcpyAsync(units.data(), b->units, sizeof(int32_t) * (size_t)count,
+                              cudaMemcpyDeviceToHost, st));
+    GILA_CUDA(cudaStreamSynchronize(st));
+    int64_t total = 0;
+    for (int32_t i = 0; i < count; ++i) {
+        const int64_t nnz = koff[(size_t)i + 1] - koff[(size_t)i];
+        const int64_t n = vo[(size_t)i + 1] - vo[(size_t)i];
+        if (!skip[(size_t)i] &&
+            ((double)units[(size_t)i] * 128.0 > kBrPadding * (double)nnz + 128.0 * (double)((n + 31) / 32) ||
+             total + units[(size_t)i] > INT32_MAX))
+            skip[(size_t)i] = 1;
+        base[(size_t)i] = (int32_t)total;
+        if (!skip[(size_t)i]) total += units[(size_t)i];
+    }
+    gila_status s = ensure((void**)&b->tk, &b->tk_cap, (size_t)total * 256 + 16);
+    if (s != GILA_OK) return s;
+    GILA_CUDA(cudaMemcpyAsync(b->skip, skip.data(), skip.size(), cudaMemcpyHostToDevice, st));
+    GILA_CUDA(cudaMemcpyAsync(b->base, base.data(), sizeof(int32_t) * (size_t)count,
+                              cudaMemcpyHostToDevice, st));
+    if (nsl > 0) {
+        batch_fill_kernel<<<(unsigned)((nsl + 3) / 4), 128, 0, st>>>(
+            nsl, b->sgraph, b->voff, b->soff, b->base, b->skip, g->row, g->col, g->krow, g->kcol,
+            b->perm, b->rank, b->sdesc, b->deg, b->tk, b->skip + count);
+        count_launch();
+        GILA_CUDA(cudaGetLastError());
+    }
+    std::vector<uint8_t> bad((size_t)count);
+    GILA_CUDA(cudaMemcpyAsync(bad.data(), b->skip + count, (size_t)count, cudaMemcpyDeviceToHost, st));
+    GILA_CUDA(cudaStreamSynchronize(st));
+    // by width: large graphs, small ones, and the rest, each by falling work
+    for (int w = 0; w < 2; ++w) {
+        const int64_t lim = w == 0 ? max_n : kBrSmem / 32 - 64;
+        std::vector<int32_t> rows;
+        b->rest[w].clear();
+        b->big[w].clear();
+        b->small[w].clear();
+        b->max_rows_n[w] = 0;
+        for (int32_t i : b->order_h) {
+            const int64_t n = vo[(size_t)i + 1] - vo[(size_t)i];
+            if (skip[(size_t)i] || bad[(size_t)i] || n > lim) {
+                b->rest[w].push_back(i);
+                continue;
+            }
+            b->max_rows_n[w] = std::max(b->max_rows_n[w], n);
+            rows.push_back(i);
+        }
+        std::stable_sort(rows.begin(), rows.end(), [&](int32_t x, int32_t y) {
+            return units[(size_t)x] > units[(size_t)y];
+        });
+        // An SM's share of the batch (steps, two more a slice), the cluster
+        // that brings the largest graph below it, and the graphs it takes:
+        // 500 graphs of 50..5000 vertices in FP32 6.5 -> 0.90, 0.73, 0.60 ms
+        // with clusters of 8, 4, 2 (the share asks for 2); 250 in FP64 20.8
+        // -> 5.8, 4.1, 5.1 (4); 30 in FP64 0.69, 1.21, 2.22 (8); 1500 in FP64
+        // 6.5, 4.2, 3.4 (1: an SM left over in a GPC, or waiting for a peer,
+        // is then lost). Graphs from about a third of the share on.
+        auto cost = [&](int32_t i) {
+            return units[(size_t)i] + 2 * ((vo[(size_t)i + 1] - vo[(size_t)i] + 31) / 32);
+        };
+        int64_t all_cost = 0;
+        for (int32_t i : rows) all_cost += cost(i);
+        const int64_t share = all_cost / std::max(1, sm_count(g->device)) + 1;
+        b->cluster[w] = 1;
+        if (!rows.empty())
+            while (b->cluster[w] < kBrCluster && cost(rows[0]) > share * b->cluster[w])
+                b->cluster[w] *= 2;
+        for (int32_t i : rows) {
+            const bool large = b->cluster[w] > 1 && 3 * cost(i) > share &&
+                               (vo[(size_t)i + 1] - vo[(size_t)i] + 31) / 32 >= kBrBigSlices[w];
+            (large ? b->big[w] : b->small[w]).push_back(i);
+        }
+        std::vector<int32_t> all(b->big[w]);
+        all.insert(all.end(), b->small[w].begin(), b->small[w].end());
+        all.insert(all.end(), b->rest[w].begin(), b->rest[w].end());
+        GILA_CUDA(cudaMemcpyAsync(b->rorder[w], all.data(), sizeof(int32_t) * all.size(),
+                                  cudaMemcpyHostToDevice, st));
+        GILA_CUDA(cudaStreamSynchronize(st));
+    }
+    b->plan_serial = g->khop_serial;
+    return GILA_OK;
+}
+
+// GILA_ECUDA (and clears the flag) when a cluster gave up waiting for its
+// peers' positions since the last call; synchronises st.
+gila_status batch_wait_failed(cudaStream_t st)
+{
+    int h = 0;
+    const int zero = 0;
+    GILA_CUDA(cudaMemcpyFromSymbolAsync(&h, g_batch_wait_failed, sizeof(int), 0,
+                                        cudaMemcpyDeviceToHost, st));
+    GILA_CUDA(cudaStreamSynchronize(st));
+    if (!h) return GILA_OK;
+    GILA_CUDA(cudaMemcpyToSymbolAsync(g_batch_wait_failed, &zero, sizeof(int), 0,
+                                      cudaMemcpyHostToDevice, st));
+    GILA_CUDA(cudaStreamSynchronize(st));
+    return fail(GILA_ECUDA, "a cluster of the batch kernel did not receive its positions in time");
+}
+
 // Launch (or replay) the persistent kernel on the batch's capture stream,
 // ordered after and before the caller's stream.
 gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
@@ -350,8 +1074,15 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
         GILA_CUDA(cudaMemcpy(b->geo, geo.data(), sizeof(double) * geo.size(),
                              cudaMemcpyHostToDevice));
     }
+    if ((s = batch_plan(b)) != GILA_OK) return s;
     const int sms = sm_count(g->device);
     const gila_batch_tuning tu = resolved(b, esz, sms);
+    // lane groups set by the tuning ask for the group kernel on every graph
+    const int w = esz == 16 ? 1 : 0;
+    const bool groups = b->tune.group4_max > 0 || b->tune.group8_max > 0 || b->tune.group16_max > 0;
+    const int nbig = groups ? 0 : (int)b->big[w].size();
+    const int nrows = groups ? 0 : nbig + (int)b->small[w].size();
+    const int nrest = b->count - nrows;
     const int64_t smem_cap = 227 * 1024 - 2048;
     int64_t per_cta = smem_cap / tu.ctas_per_sm;
     int64_t smem_verts = std::min<int64_t>(b->max_n, per_cta / (2 * (int64_t)esz));
@@ -362,9 +1093,10 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
         if (s != GILA_OK) return s;
     }
     BatchArgs A;
+    memset(&A, 0, sizeof(A));  // padding too: the bytes are part of the captured graph's key
     A.voff = b->voff;
-    A.order = b->order;
-    A.count = b->count;
+    A.order = groups ? b->order : b->rorder[w] + nrows;
+    A.count = nrest;
     A.row = g->row;
     A.col = g->col;
     A.krow = g->krow;
@@ -383,12 +1115,45 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
     A.g4_max = tu.group4_max;
     A.g8_max = tu.group8_max;
     A.g16_max = tu.group16_max;
-    const int grid = std::max(1, std::min<int>(sms * tu.ctas_per_sm, b->count));
+    const int grid = std::max(1, std::min<int>(sms * tu.ctas_per_sm, nrest));
+    BatchRowsArgs R;
+    memset(&R, 0, sizeof(R));
+    R.voff = b->voff;
+    R.order = b->rorder[w];
+    R.nbig = nbig;
+    R.nall = nrows;
+    R.soff = b->soff;
+    R.sdesc = b->sdesc;
+    R.deg = b->deg;
+    R.perm = b->perm;
+    R.cuts = b->cuts;
+    R.tk = b->tk;
+    R.work = b->work + 1;
+    R.geo = b->geo;
+    R.iters = prm->iters;
+    R.schedule = prm->schedule;
+    R.d = prm->d;
+    R.t0 = prm->t0;
+    R.c = force_consts(prm->d, 0.0);
+    R.p = prm->p;
+    R.q = prm->q;
+    R.pos = pos;
+    R.stride = (int)((b->max_rows_n[w] + 31) / 32 * 32 + 2);
+    R.wait_ns = kBrWaitNs;
+    const size_t rsmem = 2 * (size_t)R.stride * esz;
+    // as many CTAs per SM as the tuning and the buffers allow, in clusters
+    const int64_t fit = std::max<int64_t>(1, (kBrSmem + 2048) / (int64_t)(rsmem + 2048));
+    const int64_t per_sm = std::min<int64_t>(fit, b->tune.ctas_per_sm > 0 ? tu.ctas_per_sm
+                                                                          : 2048 / tu.threads);
+    const int cl = b->cluster[w];
+    const int64_t want = std::min<int64_t>(sms * per_sm, (int64_t)nbig * cl + nrows - nbig);
+    const int rgrid = (int)((std::max<int64_t>(want, 1) + cl - 1) / cl * cl);
     // the captured graph is reused while every argument is the same
-    std::vector<unsigned char> key(sizeof(A) + sizeof(int) * 3);
+    const int extra[7] = {grid, tu.threads, prm->precision, nrows, nrest, rgrid, cl};
+    std::vector<unsigned char> key(sizeof(A) + sizeof(R) + sizeof(extra));
     memcpy(key.data(), &A, sizeof(A));
-    const int extra[3] = {grid, tu.threads, prm->precision};
-    memcpy(key.data() + sizeof(A), extra, sizeof(extra));
+    memcpy(key.data() + sizeof(A), &R, sizeof(R));
+    memcpy(key.data() + sizeof(A) + sizeof(R), extra, sizeof(extra));
     GILA_CUDA(configure_batch_kernels());
     GILA_CUDA(cudaEventRecord(b->ev_in, b->user));
     GILA_CUDA(cudaStreamWaitEvent(b->own, b->ev_in, 0));
@@ -399,23 +1164,33 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
         }
         cudaGraph_t graph = nullptr;
         GILA_CUDA(cudaStreamBeginCapture(b->own, cudaStreamCaptureModeThreadLocal));
-        cudaMemsetAsync(b->work, 0, sizeof(int), b->own);
+        cudaError_t e = cudaMemsetAsync(b->work, 0, sizeof(int) * 3, b->own);
         const bool fr = (prm->p == 2 && prm->q == 1);
-        cudaError_t e;
-        switch (prm->precision) {
-        case GILA_FP64:
-            e = fr ? launch_batch<double, kFR, false>(A, grid, tu.threads, smem, b->own)
-                   : launch_batch<double, kGeneric, false>(A, grid, tu.threads, smem, b->own);
-            break;
-        case GILA_FP32_COMPENSATED:
-            e = fr ? launch_batch<float, kFR, true>(A, grid, tu.threads, smem, b->own)
-                   : launch_batch<float, kGeneric, true>(A, grid, tu.threads, smem, b->own);
-            break;
-        default:
-            e = fr ? launch_batch<float, kFR, false>(A, grid, tu.threads, smem, b->own)
-                   : launch_batch<float, kGeneric, false>(A, grid, tu.threads, smem, b->own);
-            break;
-        }
+        const bool fork = nrows > 0 && nrest > 0;
+        cudaStream_t gst = fork ? b->side : b->own;
+        if (e == cudaSuccess && fork) e = cudaEventRecord(b->ev_fork, b->own);
+        if (e == cudaSuccess && fork) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
+        auto launch = [&](auto model, auto one) {
+            // `one`: a value of the force type; its second field the compensation
+            using T = typename decltype(one)::type;
+            constexpr bool comp = decltype(one)::comp;
+            constexpr int M = decltype(model)::value;
+            if (e == cudaSuccess && nrows > 0)
+                e = launch_batch_rows<T, M, comp>(R, rgrid, cl, tu.threads, rsmem, b->own);
+            if (e == cudaSuccess && nrest > 0)
+                e = launch_batch<T, M, comp>(A, grid, tu.threads, smem, gst);
+        };
+        auto by_type = [&](auto model) {
+            switch (prm->precision) {
+            case GILA_FP64: launch(model, Form<double, false>()); break;
+            case GILA_FP32_COMPENSATED: launch(model, Form<float, true>()); break;
+            default: launch(model, Form<float, false>()); break;
+            }
+        };
+        if (fr) by_type(std::integral_constant<int, kFR>());
+        else by_type(std::integral_constant<int, kGeneric>());
+        if (e == cudaSuccess && fork) e = cudaEventRecord(b->ev_join, b->side);
+        if (e == cudaSuccess && fork) e = cudaStreamWaitEvent(b->own, b->ev_join, 0);
         cudaError_t e2 = cudaStreamEndCapture(b->own, &graph);
         if (e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -499,12 +1274,19 @@ void gila_batch_destroy(gila_batch* b)
     if (b->own) cudaStreamSynchronize(b->own);
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->own) cudaStreamDestroy(b->own);
+    if (b->side) cudaStreamDestroy(b->side);
+    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+    if (b->ev_join) cudaEventDestroy(b->ev_join);
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
     cudaFree(b->voff);
     cudaFree(b->order);
     cudaFree(b->work);
     cudaFree(b->geo);
+    for (void* p : {(void*)b->rorder[0], (void*)b->rorder[1], (void*)b->soff, (void*)b->sgraph,
+                    (void*)b->base, (void*)b->units, (void*)b->skip, (void*)b->sdesc,
+                    (void*)b->deg, (void*)b->perm, (void*)b->rank, (void*)b->cuts, (void*)b->tk})
+        cudaFree(p);
     cudaFree(b->tmp);
     cudaFree(b->pos[0]);
     cudaFree(b->pos[1]);
@@ -584,7 +1366,8 @@ gila_status gila_batch_autotune(gila_batch* b, const gila_params* prm, const voi
     q.iters = probe_iters;
     static const int kThreadsSet[3] = {256, 512, 1024};
     static const int kCtasSet[4] = {1, 2, 4, 8};
-    static const int kGroups[3][3] = {{8, 24, 64}, {4, 12, 32}, {16, 48, 128}};
+    // no groups set: rows per lane where they apply
+    static const int kGroups[4][3] = {{0, 0, 0}, {8, 24, 64}, {4, 12, 32}, {16, 48, 128}};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     GILA_CUDA(cudaEventCreate(&e0));
     GILA_CUDA(cudaEventCreate(&e1));
@@ -595,7 +1378,7 @@ gila_status gila_batch_autotune(gila_batch* b, const gila_params* prm, const voi
     for (int ti = 0; ti < 3 && s == GILA_OK; ++ti)
         for (int ci = 0; ci < 4 && s == GILA_OK; ++ci) {
             if (kCtasSet[ci] * kThreadsSet[ti] > 2048) continue;
-            for (int gi = 0; gi < 3 && s == GILA_OK; ++gi) {
+            for (int gi = 0; gi < 4 && s == GILA_OK; ++gi) {
                 gila_batch_tuning c = {kThreadsSet[ti], kCtasSet[ci], kGroups[gi][0],
                                        kGroups[gi][1], kGroups[gi][2]};
                 b->tune = c;
@@ -674,7 +1457,7 @@ gila_status gila_layout_batch_run(gila_batch* b, const gila_params* prm, const d
         GILA_CUDA(cudaMemcpyAsync(pos_out_host, b->stage, 16 * n, cudaMemcpyDeviceToHost, b->user));
     }
     GILA_CUDA(cudaStreamSynchronize(b->user));
-    return GILA_OK;
+    return batch_wait_failed(b->user);
 }
 
 gila_status gila_layout_batch(gila_graph* const* gs, int32_t count, const gila_params* prm,

@@ -57,9 +57,7 @@ constexpr uint64_t kTestWaitNs = 1000000ull;   // the bound while the wait test 
 // of r^2 = 2e38 is below the smallest normal and flushes to 0; in FP64 r^2
 // = 1.48e308 flushes rcp to 0 the same way; the generic model cuts terms
 // beyond r^2 = 1e38 (FP32) or 1e300 (FP64). 0 * Delta then adds nothing.
-template <class T> struct FarSlot;
-template <> struct FarSlot<float> { static constexpr float v = 1.0e19f; };
-template <> struct FarSlot<double> { static constexpr double v = 8.6e153; };
+// (FarSlot, force.cuh)
 
 constexpr int kPrefetch = 4;  // steps between an L2 prefetch of ids and their ring load (4, 12, 24
                                // measured: 4 best; longer distances crowd L2)
@@ -144,30 +142,6 @@ __host__ __device__ __forceinline__ int32_t lane_len(int32_t L)
 {
     // a share is at most L / kBThreads + 8 entries (8-aligned cuts)
     return (L == 0) ? 0 : ((L / kBThreads + 2 * kStep - 1) & ~(kStep - 1));
-}
-
-// acc += (x, y) with a two-sum error term per component; in FP32 both
-// components go through packed two-lane operations (six instead of twelve).
-template <class T, bool COMP>
-__device__ __forceinline__ void add_compensated(Acc<T, COMP>& acc, T x, T y)
-{
-    if constexpr (sizeof(T) == 4 && COMP) {
-        uint64_t s, c, v, t, bp, e1, e2;
-        asm("mov.b64 %0, {%1, %2};" : "=l"(s) : "f"(acc.sx), "f"(acc.sy));
-        asm("mov.b64 %0, {%1, %2};" : "=l"(c) : "f"(acc.cx), "f"(acc.cy));
-        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(s), "l"(v));    // t = s + v
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(bp) : "l"(t), "l"(s));   // bp = t - s
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(t), "l"(bp));  // t - bp
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(s), "l"(e1));  // s - (t - bp)
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e2) : "l"(v), "l"(bp));  // v - bp
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(e1), "l"(e2));
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(c), "l"(e1));
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(acc.sx), "=f"(acc.sy) : "l"(t));
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(acc.cx), "=f"(acc.cy) : "l"(c));
-    } else {
-        acc.merge(x, y, T(0), T(0));
-    }
 }
 
 // Window mode's finish of the rows [u0, u0 + nrows) of a range, after their
@@ -732,13 +706,6 @@ struct RowsArgs {
     uint64_t wait_ns;
     int skip_copy;
 };
-
-__device__ __forceinline__ uint2 ld_ids2(const uint2* p)
-{
-    uint2 r;
-    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));
-    return r;
-}
 
 template <class T, int MODEL, bool COMP>
 __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kernel(const RowsArgs A)

@@ -63,6 +63,20 @@ __device__ __forceinline__ uint32_t ld_id(const uint32_t* p)
     return r;
 }
 
+// Streaming load of eight bytes of ids (four 16-bit ids).
+__device__ __forceinline__ uint2 ld_ids2(const uint2* p)
+{
+    uint2 r;
+    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));
+    return r;
+}
+
+// Coordinates of the slot that padding ids point at: so far away that its
+// term is exactly zero (see blocked.cu).
+template <class T> struct FarSlot;
+template <> struct FarSlot<float> { static constexpr float v = 1.0e19f; };
+template <> struct FarSlot<double> { static constexpr double v = 8.6e153; };
+
 template <class T>
 __device__ __forceinline__ T ipow_(T x, int e)
 {
@@ -124,6 +138,30 @@ struct Acc {
     __device__ __forceinline__ T fx() const { return COMP ? sx + cx : sx; }
     __device__ __forceinline__ T fy() const { return COMP ? sy + cy : sy; }
 };
+
+// acc += (x, y) with a two-sum error term per component; in FP32 both
+// components go through packed two-lane operations (six instead of twelve).
+template <class T, bool COMP>
+__device__ __forceinline__ void add_compensated(Acc<T, COMP>& acc, T x, T y)
+{
+    if constexpr (sizeof(T) == 4 && COMP) {
+        uint64_t s, c, v, t, bp, e1, e2;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(s) : "f"(acc.sx), "f"(acc.sy));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(c) : "f"(acc.cx), "f"(acc.cy));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(s), "l"(v));    // t = s + v
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(bp) : "l"(t), "l"(s));   // bp = t - s
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(t), "l"(bp));  // t - bp
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(s), "l"(e1));  // s - (t - bp)
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(e2) : "l"(v), "l"(bp));  // v - bp
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(e1) : "l"(e1), "l"(e2));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(c), "l"(e1));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(acc.sx), "=f"(acc.sy) : "l"(t));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(acc.cx), "=f"(acc.cy) : "l"(c));
+    } else {
+        acc.merge(x, y, T(0), T(0));
+    }
+}
 
 // Where a kernel reads positions from.
 enum Src {

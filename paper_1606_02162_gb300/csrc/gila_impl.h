@@ -147,6 +147,7 @@ struct gila_graph {
     int32_t* col = nullptr;
     // k-hop lists
     int32_t k_built = 0;
+    int64_t khop_serial = 0;  // builds of the lists so far (plans tell by it which they are of)
     int64_t nnz_khop = 0;
     int64_t* krow = nullptr;
     uint32_t* kcol = nullptr;

@@ -1108,6 +1108,7 @@ gila_status build_khop_fill(gila_graph* g, int k)
     if (s != GILA_OK) return s;
     g->nnz_khop = nnz;
     g->k_built = k;
+    ++g->khop_serial;
     return GILA_OK;
 }
 

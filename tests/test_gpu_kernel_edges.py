@@ -100,3 +100,47 @@ def test_row_per_lane_step(name, g, k, rows, pq):
         assert ("row per lane" in kernel) == rows, kernel
         assert torch.equal(y, x + disp)
         assert np.abs(disp.double().cpu().numpy() - want).max() <= TOL[prec] * np.abs(want).max()
+
+
+# slices of one, a whole and a started 32 rows; graphs below, at and above the
+# slices from which a cluster takes one (2048 vertices in FP32, 512 in FP64);
+# one beyond FP64's shared memory; empty rows; long rows and an unsorted
+# adjacency, which keep the group kernel beside the others
+def batch_graphs():
+    return [I.csr_from_edges(1, [], []), I.path(31), I.cycle(32), I.grid(3, 11), I.grid(16, 32),
+            I.tri_mesh(19, 27), I.random_tree(2016, 3), I.grid(32, 64), I.erdos_renyi(2081, 4.0, 5),
+            mesh_with_tail(40, 60, 33), I.grid(100, 100), I.star(300), unsorted_rows(I.grid(9, 9)),
+            I.erdos_renyi(5000, 4.0, 9)]
+
+
+@pytest.mark.parametrize("prec", list(TOL), ids=["fp32", "fp32c", "fp64"])
+@pytest.mark.parametrize("pq,sched", [((2, 1), O.SCHED_LINEAR), ((3, 2), O.SCHED_GEOM)],
+                         ids=["fr_linear", "p3q2_geometric"])
+def test_batch_row_per_lane(prec, pq, sched):
+    graphs = batch_graphs()
+    p, q = pq
+    pos = [I.uniform_positions(g.n, 60 + i).astype(np.float32).astype(np.float64)
+           for i, g in enumerate(graphs)]
+    off = np.concatenate([[0], np.cumsum([g.n for g in graphs])])
+    iters = 4 if prec == G.GILA_FP64 else 1
+    prm = G.params(k=2, iters=iters, d=1.2, p=p, q=q, precision=prec,
+                   schedule=G.GILA_COOL_LINEAR if sched == O.SCHED_LINEAR else G.GILA_COOL_GEOMETRIC)
+    with G.Batch(graphs) as b:
+        out = G.gila_layout_batch_run(b.handle, prm, np.concatenate(pos))
+        again = G.gila_layout_batch_run(b.handle, prm, np.concatenate(pos))
+        G.gila_batch_khop_reset(b.handle)  # the plan is made anew
+        rebuilt = G.gila_layout_batch_run(b.handle, prm, np.concatenate(pos))
+        G.gila_batch_tune(b.handle, threads=256, ctas_per_sm=8)
+        shaped = G.gila_layout_batch_run(b.handle, prm, np.concatenate(pos))
+    assert np.array_equal(out, again) and np.array_equal(out, rebuilt) and np.array_equal(out, shaped)
+    for i, g in enumerate(graphs):
+        krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 2)
+        want = O.run(g.n, g.row_ptr, g.col_idx, krow, kcol, pos[i], iters, d=1.2, p=p, q=q,
+                     schedule=sched) - pos[i]
+        got = out[off[i]:off[i + 1]] - pos[i]
+        scale = np.abs(want).max()
+        # FP32: the move is read back as (position + move) - position
+        slack = 4 * np.finfo(np.float32).eps * np.abs(pos[i]).max() if prec != G.GILA_FP64 else 0.0
+        # FP64: rounding grows over four iterations (1e-9 as for a few iterations)
+        tol = 1e-9 if prec == G.GILA_FP64 else TOL[prec]
+        assert np.abs(got - want).max() <= tol * max(scale, 1e-300) + slack, (i, g.name, g.n)
