@@ -305,10 +305,13 @@ struct Rep {
     {
         return rcp_fast(fmaf(dx, dx, fmaf(dy, dy, 0x1p-100f)));
     }
+    // FP64 likewise, with 2^-1000: no effect on an r^2 >= 2^-946, a finite
+    // factor at r^2 = 0, and no comparison (which takes the FP64 pipe, two
+    // lanes a clock per SM, like the ten operations that remain: 250 graphs
+    // of the batch 3.88 -> 3.68 ms)
     __device__ __forceinline__ static double rep_fr1(double dx, double dy)
     {
-        const double r2 = dx * dx + dy * dy;
-        return r2 > 0.0 ? rcp_newton(r2) : 0.0;
+        return rcp_newton(fma(dx, dx, fma(dy, dy, 0x1p-1000)));
     }
 };
 
