@@ -68,7 +68,7 @@ __device__ int g_tile_wait_failed = 0;
 
 struct BlockedArgs {
     const uint16_t* tk;        // tile-relative ids, block by block, in share storage order
-    const int64_t* toff;       // nt n: start of segment (tile j, row u) within its block
+    const int32_t* toff;       // nt n: start of segment (tile j, row u) within its block
     const int64_t* blk;        // 2 nb: first slot in tk and entry count of block b
     const int4* bdesc;         // nb: first row, end row and tile of block b
     int64_t n;
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
     // meanwhile: the row directory (segment starts within the block) and
     // zero partials for rows with no entries in this tile
     for (int i = threadIdx.x; i < nrows; i += kBThreads) {
-        D[i] = (int32_t)A.toff[(int64_t)j * A.n + u0 + i];
+        D[i] = A.toff[(int64_t)j * A.n + u0 + i];
         P2* c = cellp(i);
         P2 z;
         z.x = T(0);
@@ -1055,13 +1055,194 @@ __device__ __forceinline__ void seg_bounds(const int64_t* __restrict__ krow,
 
 __global__ void seglen_kernel(int64_t n, const int64_t* __restrict__ krow,
                               const uint32_t* __restrict__ kcol, int nt, int tv,
-                              int64_t* __restrict__ len)
+                              int32_t* __restrict__ len)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * nt) return;
     int64_t lo, hi;
     seg_bounds(krow, kcol, i % n, (int)(i / n), nt, tv, &lo, &hi);
-    len[i] = hi - lo;
+    len[i] = (int32_t)(hi - lo);
+}
+
+__global__ void rowlen_kernel(int64_t n, const int64_t* __restrict__ krow, int32_t* __restrict__ len)
+{
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < n) len[u] = (int32_t)(krow[u + 1] - krow[u]);
+}
+
+// ---- the plan's cut of every tile's rows into ranges, on the device: with
+// the segment lengths of n nt cells (4.3 million on BA n = 333,334, k = 2)
+// copied to the host, summed, searched and their offsets copied back, the
+// host took 19 of the 27.2 ms from reset to the first step, the GPU 8.6;
+// 8.2 ms with the plan here.
+
+// A segment's entries as stored, and the cost of its row in the block: the
+// padded entries and a per-row term where it has entries (directory, row
+// change, cell store), else only the zeroed cell.
+__host__ __device__ __forceinline__ int64_t seg_padded(int64_t len)
+{
+    return (len + kStep - 1) & ~int64_t(kStep - 1);
+}
+__host__ __device__ __forceinline__ int64_t row_cost(int64_t len)
+{
+    return len > 0 ? 8 + seg_padded(len) : 1;
+}
+
+constexpr int kCellThreads = 256;
+constexpr int kCellItems = 8;
+constexpr int kCellTile = kCellThreads * kCellItems;
+
+// Totals of padded lengths and costs of every kCellTile cells.
+__global__ void __launch_bounds__(kCellThreads)
+cell_sums_kernel(int64_t cells, const int32_t* __restrict__ len, int64_t* __restrict__ sums)
+{
+    __shared__ int64_t wt[kCellThreads / 32 + 1];
+    const int64_t base = (int64_t)blockIdx.x * kCellTile;
+    int64_t pad = 0, cost = 0;
+    for (int i = threadIdx.x; i < kCellTile && base + i < cells; i += kCellThreads) {
+        const int64_t l = len[base + i];
+        pad += seg_padded(l);
+        cost += row_cost(l);
+    }
+    int64_t tp, tc;
+    block_inclusive_scan<int64_t, kCellThreads>(pad, wt, &tp);
+    block_inclusive_scan<int64_t, kCellThreads>(cost, wt, &tc);
+    if (threadIdx.x == 0) {
+        sums[2 * blockIdx.x] = tp;
+        sums[2 * blockIdx.x + 1] = tc;
+    }
+}
+
+// Exclusive scan of both totals, in place, by one block.
+__global__ void __launch_bounds__(1024) cell_scan_sums_kernel(int64_t* __restrict__ sums, int64_t nb)
+{
+    __shared__ int64_t wt[1024 / 32 + 1];
+    int64_t cp = 0, cc = 0;
+    for (int64_t b0 = 0; b0 < nb; b0 += 1024) {
+        const int64_t i = b0 + threadIdx.x;
+        const int64_t p = i < nb ? sums[2 * i] : 0, c = i < nb ? sums[2 * i + 1] : 0;
+        int64_t tp, tc;
+        const int64_t ip = block_inclusive_scan<int64_t, 1024>(p, wt, &tp);
+        const int64_t ic = block_inclusive_scan<int64_t, 1024>(c, wt, &tc);
+        if (i < nb) {
+            sums[2 * i] = cp + ip - p;
+            sums[2 * i + 1] = cc + ic - c;
+        }
+        cp += tp;
+        cc += tc;
+    }
+}
+
+// Exclusive prefix sums of the cells (cells + 1 values each).
+__global__ void __launch_bounds__(kCellThreads)
+cell_prefix_kernel(int64_t cells, const int32_t* __restrict__ len, const int64_t* __restrict__ sums,
+                   int64_t* __restrict__ pre_pad, int64_t* __restrict__ pre_cost)
+{
+    __shared__ int64_t wt[kCellThreads / 32 + 1];
+    __shared__ int64_t sp[kCellTile], sc[kCellTile];
+    const int64_t base = (int64_t)blockIdx.x * kCellTile;
+    const int t0 = threadIdx.x * kCellItems;
+    int32_t l[kCellItems];
+    int64_t pad = 0, cost = 0;
+#pragma unroll
+    for (int i = 0; i < kCellItems; ++i) {
+        l[i] = base + t0 + i < cells ? len[base + t0 + i] : -1;
+        if (l[i] >= 0) {
+            pad += seg_padded(l[i]);
+            cost += row_cost(l[i]);
+        }
+    }
+    int64_t tp, tc;
+    int64_t rp = sums[2 * blockIdx.x] + block_inclusive_scan<int64_t, kCellThreads>(pad, wt, &tp) - pad;
+    int64_t rc = sums[2 * blockIdx.x + 1] + block_inclusive_scan<int64_t, kCellThreads>(cost, wt, &tc) - cost;
+#pragma unroll
+    for (int i = 0; i < kCellItems; ++i) {
+        sp[t0 + i] = rp;
+        sc[t0 + i] = rc;
+        if (l[i] >= 0) {
+            rp += seg_padded(l[i]);
+            rc += row_cost(l[i]);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kCellTile && base + i < cells; i += kCellThreads) {
+        pre_pad[base + i] = sp[i];
+        pre_cost[base + i] = sc[i];
+    }
+    if (base + t0 < cells && base + t0 + kCellItems >= cells) {  // the thread of the last cell
+        pre_pad[cells] = rp;
+        pre_cost[cells] = rc;
+    }
+}
+
+// Greedy cut of every tile's rows into ranges of cost at most caps[x] (a
+// range takes at least one row) and at most max_rows rows, for as many caps
+// as the grid is wide: a warp per (cap, tile) walks the tile, finding each
+// range's end by a 32-way search of the prefix costs. counts[x] receives the
+// ranges of all tiles; with cuts, tile j's bounds go to cuts[j stride ...]
+// and their number to tile_counts[j]. A tile stops once it exceeds limit.
+__global__ void __launch_bounds__(256)
+cut_kernel(int64_t n, int nt, const int64_t* __restrict__ pre, const int64_t* __restrict__ caps,
+           int64_t max_rows, int64_t limit, int* __restrict__ counts, int32_t* __restrict__ cuts,
+           int64_t stride, int* __restrict__ tile_counts)
+{
+    const int lane = threadIdx.x & 31;
+    const int j = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (j >= nt) return;
+    const int64_t cap = caps[blockIdx.x];
+    const int64_t* p = pre + (int64_t)j * n;
+    int64_t s = 0, count = 0;
+    if (cuts && lane == 0) cuts[j * stride] = 0;
+    while (s < n && count <= limit) {
+        const int64_t most = p[s] + cap;
+        int64_t lo = s + 1, hi = s + max_rows < n ? s + max_rows : n;
+        while (lo < hi) {  // the last e in [lo, hi] with p[e] <= most, lo if none
+            const int64_t step = (hi - lo + 31) >> 5;
+            const int64_t x = lo + step * (lane + 1) < hi ? lo + step * (lane + 1) : hi;
+            const int c = __popc(__ballot_sync(kFull, p[x] <= most));
+            const int64_t l0 = lo;
+            if (c > 0) lo = l0 + step * c < hi ? l0 + step * c : hi;
+            if (c < 32 && l0 + step * (c + 1) - 1 < hi) hi = l0 + step * (c + 1) - 1;
+        }
+        s = lo;
+        ++count;
+        if (cuts && lane == 0 && count < stride) cuts[j * stride + count] = (int32_t)s;
+    }
+    if (lane == 0) {
+        atomicAdd(&counts[blockIdx.x], (int)(count < INT32_MAX / 2 ? count : INT32_MAX / 2));
+        if (tile_counts) tile_counts[j] = (int)count;
+    }
+}
+
+// Padded entries and cost of blocks given as (first row, end row, tile, -).
+__global__ void block_sums_kernel(int64_t n, int64_t cells, int64_t nb, const int4* __restrict__ blocks,
+                                  const int64_t* __restrict__ pre, int64_t* __restrict__ out)
+{
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= nb) return;
+    const int4 x = blocks[b];
+    const int64_t lo = x.z * n + x.x, hi = x.z * n + x.y;
+    out[2 * b] = pre[hi] - pre[lo];
+    out[2 * b + 1] = pre[cells + 1 + hi] - pre[cells + 1 + lo];
+}
+
+// Starts of the segments within their blocks.
+__global__ void toff_kernel(int64_t n, const int4* __restrict__ bdesc,
+                            const int64_t* __restrict__ pre_pad, int32_t* __restrict__ toff)
+{
+    const int4 x = bdesc[blockIdx.x];
+    const int64_t* p = pre_pad + x.z * n;
+    const int64_t first = p[x.x];
+    for (int64_t u = x.x + threadIdx.x; u < x.y; u += blockDim.x)
+        toff[x.z * n + u] = (int32_t)(p[u] - first);
+}
+
+// Vertices of adjacency degree above kHubDeg, in any order.
+__global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t* __restrict__ hubs,
+                            int* __restrict__ count)
+{
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < n && row[u + 1] - row[u] > kHubDeg) hubs[atomicAdd(count, 1)] = (int32_t)u;
 }
 
 // Copy every (tile, row) segment into its block's share storage as 16-bit
@@ -1115,8 +1296,8 @@ __global__ void pad_fill_kernel(uint16_t* __restrict__ tk, const int64_t* __rest
 template <int G, bool SPREAD>
 __global__ void __launch_bounds__(kSpreadWarps * 32) block_layout_kernel(
     int64_t n, const int64_t* __restrict__ krow, const uint32_t* __restrict__ kcol, int nt,
-    int tv, const int64_t* __restrict__ wbase, const int64_t* __restrict__ toff,
-    const int64_t* __restrict__ blk, const int32_t* __restrict__ tfirst,
+    int tv, const int64_t* __restrict__ wbase, const int32_t* __restrict__ len,
+    const int32_t* __restrict__ toff, const int64_t* __restrict__ blk, const int32_t* __restrict__ tfirst,
     const int32_t* __restrict__ rstart, const int32_t* __restrict__ rblock,
     uint16_t* __restrict__ tk)
 {
@@ -1128,9 +1309,13 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) block_layout_kernel(
     if (i >= n * nt) return;  // warp-uniform
     const int j = (int)(i / n);
     const int64_t u = i % n;
-    int64_t lo, hi;
-    seg_bounds(krow, kcol, u, j, nt, tv, &lo, &hi);
-    if (hi == lo) return;
+    const int seglen = len[i];
+    if (seglen == 0) return;
+    // the segment starts after the row's segments in earlier tiles
+    int64_t lo = krow[u];
+    for (int jj = lane; jj - lane < j; jj += 32)
+        lo += __reduce_add_sync(kFull, jj < j ? (unsigned)len[(int64_t)jj * n + u] : 0u);
+    const int64_t hi = lo + seglen;
     // the range of tile j that holds row u (tile j's ranges: blocks
     // tfirst[j] .. tfirst[j + 1] - 1 in tile order, their row bounds at
     // rstart + tfirst[j] + j), and that range's block
@@ -1149,7 +1334,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) block_layout_kernel(
     const int64_t bsp = blk[2 * b];
     const int32_t L = (int32_t)blk[2 * b + 1];
     const int32_t m8 = lane_len(L);
-    const int32_t S0 = (int32_t)toff[i], S1 = S0 + (int32_t)(hi - lo);
+    const int32_t S0 = toff[i], S1 = S0 + (int32_t)(hi - lo);
     const int32_t S8 = S0 + (int32_t)((hi - lo + kStep - 1) & ~int64_t(kStep - 1));  // padded end
     // the share holding entry p (t follows p, which only grows) and the slot
     int t = (int)((int64_t)S0 * kBThreads / L);
@@ -1326,7 +1511,7 @@ constexpr int kMetSmemMax = kSmemCap - 12 * 1024;  // the tile's share of shared
 
 struct MetricArgs {
     const int64_t* krow;
-    const int64_t* len;    // tile mode: nt n segment lengths (row u's entries in tile j)
+    const int32_t* len;    // tile mode: nt n segment lengths (row u's entries in tile j)
     const uint32_t* kcol;
     const int4* bdesc;     // nb: first row, end row and tile of block b
     const int64_t* wbase;  // window mode: 2 nb (first id, length), else null
@@ -1583,28 +1768,30 @@ void free_tile_plans(gila_graph* g)
         cudaFree(P.tk);
         cudaFree(P.part);
         cudaFree(P.len);
+        cudaFree(P.pre);
+        cudaFree(P.cut);
         P = TilePlan();
     }
 }
 
 // First and last id of every k-hop row (rows are sorted); INT32_MAX and -1
-// for empty rows.
+// for empty rows. *widest receives the most ids a row spans.
 __global__ void rowspan_kernel(int64_t n, const int64_t* __restrict__ krow,
-                               const uint32_t* __restrict__ kcol, int32_t* __restrict__ span)
+                               const uint32_t* __restrict__ kcol, int32_t* __restrict__ span,
+                               int32_t* __restrict__ widest)
 {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= n) return;
-    const int64_t b = krow[u], e = krow[u + 1];
-    span[2 * u] = b < e ? (int32_t)kcol[b] : INT32_MAX;
-    span[2 * u + 1] = b < e ? (int32_t)kcol[e - 1] : -1;
-}
-
-// Cost of a row in one tile's (or window's) block: its padded entries and a
-// per-row term where it has entries (directory, row change, cell store),
-// else only the zeroed cell.
-inline int64_t row_cost(int64_t len)
-{
-    return len > 0 ? 8 + ((len + kStep - 1) & ~int64_t(kStep - 1)) : 1;
+    int32_t wide = 0;
+    if (u < n) {
+        const int64_t b = krow[u], e = krow[u + 1];
+        const int32_t first = b < e ? (int32_t)kcol[b] : INT32_MAX;
+        const int32_t last = b < e ? (int32_t)kcol[e - 1] : -1;
+        span[2 * u] = first;
+        span[2 * u + 1] = last;
+        if (b < e) wide = last - first + 1;
+    }
+    wide = __reduce_max_sync(kFull, wide);
+    if ((threadIdx.x & 31) == 0 && wide > 0) atomicMax(widest, wide);
 }
 
 // Greedy cut of one tile's rows into ranges of cost at most cap (a range
@@ -1683,25 +1870,123 @@ int64_t blocks_target(const gila_graph* g, bool window)
 }
 
 // The adjacency rows longer than kHubDeg, which the combine kernel gives a
-// block each.
+// block each (fewer than nnz / kHubDeg of them); synchronises.
 gila_status plan_hubs(gila_graph* g, TilePlan& P)
 {
-    const int64_t n = g->n;
-    std::vector<int64_t> arow((size_t)n + 1);
-    GILA_CUDA(cudaMemcpyAsync(arow.data(), g->row, sizeof(int64_t) * (n + 1),
+    const int64_t n = g->n, most = g->nnz_adj / kHubDeg + 1;
+    gila_status s = ensure((void**)&P.hubs, &P.hubs_cap, sizeof(int32_t) * ((size_t)most + 1));
+    if (s != GILA_OK) return s;
+    int* count = P.hubs + most;
+    GILA_CUDA(cudaMemsetAsync(count, 0, sizeof(int), g->stream));
+    hubs_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->row, P.hubs, count);
+    count_launch();
+    GILA_CUDA(cudaGetLastError());
+    GILA_CUDA(cudaMemcpyAsync(&P.nhub, count, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));
+    return GILA_OK;
+}
+
+// Prefix sums of the cells' padded lengths and costs (P.len, on the device)
+// into P.pre: cells + 1 values each.
+gila_status prefix_cells(gila_graph* g, TilePlan& P, int64_t cells)
+{
+    const int64_t nb = (cells + kCellTile - 1) / kCellTile;
+    gila_status s;
+    if ((s = ensure((void**)&P.pre, &P.pre_cap, sizeof(int64_t) * 2 * ((size_t)cells + 1))) != GILA_OK ||
+        (s = ensure(&P.cut, &P.cut_cap, sizeof(int64_t) * 2 * (size_t)nb)) != GILA_OK)
+        return s;
+    int64_t* sums = (int64_t*)P.cut;
+    cell_sums_kernel<<<(unsigned)nb, kCellThreads, 0, g->stream>>>(cells, P.len, sums);
+    count_launch();
+    cell_scan_sums_kernel<<<1, 1024, 0, g->stream>>>(sums, nb);
+    count_launch();
+    cell_prefix_kernel<<<(unsigned)nb, kCellThreads, 0, g->stream>>>(cells, P.len, sums, P.pre,
+                                                                    P.pre + cells + 1);
+    count_launch();
+    GILA_CUDA(cudaGetLastError());
+    return GILA_OK;
+}
+
+// Row ranges of every tile, all blocks with at most the same cost: about the
+// smallest for which the blocks number at most `target` (or the fewest the
+// row limit allows). A grid of about target equal CTAs then ends together,
+// where equal row ranges for all tiles left the hubs' tile with CTAs twice
+// the mean and one more range than the target sent a few CTAs into a second
+// wave (Barabasi-Albert n = 100,000, k = 2: 156 CTAs on 152 SMs, the SMs busy
+// 54% of the kernel's time). The cap is searched from below, the mean cost of
+// a block, 32 caps at a time: to within 1/512 of itself in two rounds.
+gila_status partition_tiles(gila_graph* g, TilePlan& P, int64_t n, int64_t nt, int64_t target,
+                            int64_t max_rows, std::vector<std::vector<int32_t>>& rs)
+{
+    constexpr int kCaps = 32;
+    const int64_t cells = n * nt;
+    const int64_t* pre = P.pre + cells + 1;
+    target = std::max<int64_t>(target, nt * ((n + max_rows - 1) / max_rows));
+    const int64_t stride = target + 2;
+    const size_t head = kCaps * 12 + sizeof(int) * (size_t)nt, at_cuts = (head + 15) & ~size_t(15);
+    gila_status s = ensure(&P.cut, &P.cut_cap, at_cuts + sizeof(int32_t) * (size_t)(nt * stride));
+    if (s != GILA_OK) return s;
+    int64_t* d_caps = (int64_t*)P.cut;
+    int* d_counts = (int*)(d_caps + kCaps);
+    int* d_tiles = d_counts + kCaps;
+    int32_t* d_cuts = (int32_t*)((char*)P.cut + at_cuts);
+    int64_t total = 0;
+    GILA_CUDA(cudaMemcpyAsync(&total, pre + cells, sizeof(int64_t), cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));
+    int64_t caps[kCaps];
+    int counts[kCaps];
+    auto count = [&](int used, bool write) -> gila_status {
+        GILA_CUDA(cudaMemcpyAsync(d_caps, caps, sizeof(int64_t) * (size_t)used,
+                                  cudaMemcpyHostToDevice, g->stream));
+        GILA_CUDA(cudaMemsetAsync(d_counts, 0, sizeof(int) * kCaps, g->stream));
+        cut_kernel<<<dim3((unsigned)used, (unsigned)((nt + 7) / 8)), 256, 0, g->stream>>>(
+            n, (int)nt, pre, d_caps, max_rows, target, d_counts, write ? d_cuts : nullptr, stride,
+            write ? d_tiles : nullptr);
+        count_launch();
+        GILA_CUDA(cudaGetLastError());
+        GILA_CUDA(cudaMemcpyAsync(counts, d_counts, sizeof(int) * (size_t)used,
+                                  cudaMemcpyDeviceToHost, g->stream));
+        GILA_CUDA(cudaStreamSynchronize(g->stream));
+        return GILA_OK;
+    };
+    // below `lo` no cut reaches the target; at total + 1 every one does
+    int64_t lo = std::max<int64_t>(1, total / target), hi = total + 1;
+    for (int64_t width = lo / 16 + 1; lo < total + 1; width *= 4) {
+        for (int i = 0; i < kCaps; ++i) caps[i] = std::min<int64_t>(lo + width * i, total + 1);
+        if ((s = count(kCaps, false)) != GILA_OK) return s;
+        int i = 0;
+        while (i < kCaps && counts[i] > target) ++i;
+        if (i < kCaps) {
+            hi = caps[i];
+            if (i > 0) lo = caps[i - 1];
+            else lo = hi - 1;
+            break;
+        }
+        lo = caps[kCaps - 1];
+    }
+    if (hi - lo > 1) {
+        const int64_t width = (hi - lo + kCaps - 1) / kCaps;
+        for (int i = 0; i < kCaps; ++i) caps[i] = std::min<int64_t>(lo + width * (i + 1), hi);
+        if ((s = count(kCaps, false)) != GILA_OK) return s;
+        for (int i = 0; i < kCaps; ++i)
+            if (counts[i] <= target) {
+                hi = caps[i];
+                break;
+            }
+    }
+    caps[0] = hi;
+    if ((s = count(1, true)) != GILA_OK) return s;
+    if (counts[0] > target) return fail(GILA_ESTATE, "block partition");  // cannot happen
+    std::vector<int> tiles((size_t)nt);
+    std::vector<int32_t> cuts((size_t)(nt * stride));
+    GILA_CUDA(cudaMemcpyAsync(tiles.data(), d_tiles, sizeof(int) * (size_t)nt,
+                              cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaMemcpyAsync(cuts.data(), d_cuts, sizeof(int32_t) * cuts.size(),
                               cudaMemcpyDeviceToHost, g->stream));
     GILA_CUDA(cudaStreamSynchronize(g->stream));
-    std::vector<int32_t> hubs;
-    for (int64_t u = 0; u < n; ++u)
-        if (arow[(size_t)u + 1] - arow[(size_t)u] > kHubDeg) hubs.push_back((int32_t)u);
-    if (!hubs.empty()) {
-        gila_status s = ensure((void**)&P.hubs, &P.hubs_cap, sizeof(int32_t) * hubs.size());
-        if (s != GILA_OK) return s;
-        GILA_CUDA(cudaMemcpyAsync(P.hubs, hubs.data(), sizeof(int32_t) * hubs.size(),
-                                  cudaMemcpyHostToDevice, g->stream));
-    }
-    GILA_CUDA(cudaStreamSynchronize(g->stream));  // the host vector goes out of scope
-    P.nhub = (int32_t)hubs.size();
+    rs.resize((size_t)nt);
+    for (int64_t j = 0; j < nt; ++j)
+        rs[(size_t)j].assign(cuts.begin() + j * stride, cuts.begin() + j * stride + tiles[(size_t)j] + 1);
     return GILA_OK;
 }
 
@@ -1845,15 +2130,23 @@ gila_status plan_window(gila_graph* g, size_t esz, TilePlan& P, bool* fits,
 {
     *fits = false;
     const int64_t n = g->n;
+    gila_status s = ensure((void**)&P.rowspan, &P.rowspan_cap, sizeof(int32_t) * (2 * (size_t)n + 1));
+    if (s != GILA_OK) return s;
+    int32_t* widest = P.rowspan + 2 * n;
+    GILA_CUDA(cudaMemsetAsync(widest, 0, sizeof(int32_t), g->stream));
+    rowspan_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, g->kcol,
+                                                                      P.rowspan, widest);
+    count_launch();
+    GILA_CUDA(cudaGetLastError());
+    // a window holds at least its widest row's ids: most graphs end here
+    int32_t span_max = 0;
+    GILA_CUDA(cudaMemcpyAsync(&span_max, widest, sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+    GILA_CUDA(cudaStreamSynchronize(g->stream));
+    if (span_max > kMaxTile || ((size_t)span_max + 1) * esz > (size_t)(kSmemCap - 4096))
+        return GILA_OK;
     std::vector<int64_t> krow((size_t)n + 1);
     GILA_CUDA(cudaMemcpyAsync(krow.data(), g->krow, sizeof(int64_t) * (n + 1),
                               cudaMemcpyDeviceToHost, g->stream));
-    gila_status s = ensure((void**)&P.rowspan, &P.rowspan_cap, sizeof(int32_t) * 2 * (size_t)n);
-    if (s != GILA_OK) return s;
-    rowspan_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, g->kcol,
-                                                                      P.rowspan);
-    count_launch();
-    GILA_CUDA(cudaGetLastError());
     std::vector<int32_t> span(2 * (size_t)n);
     GILA_CUDA(cudaMemcpyAsync(span.data(), P.rowspan, sizeof(int32_t) * 2 * n,
                               cudaMemcpyDeviceToHost, g->stream));
@@ -1913,18 +2206,17 @@ gila_status plan_window(gila_graph* g, size_t esz, TilePlan& P, bool* fits,
 // launched) costliest first, so that in a grid of several waves the CTAs
 // that start last are short ones.
 gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int64_t tv,
-                         const std::vector<int64_t>& len,
                          const std::vector<std::vector<int32_t>>& rs,
                          const std::vector<int64_t>* wb)
 {
     const int64_t n = g->n;
     const int64_t cells = n * nt;
+    gila_status s;
     struct Blk {
         int32_t j, r, u0, u1;
         int64_t L, cost;
     };
     std::vector<Blk> bl;
-    std::vector<int64_t> toff((size_t)cells);
     // directory for the layout kernel: tfirst (nt + 1), then each tile's
     // range bounds (nb + nt), then the block of each (tile, range) (nb)
     std::vector<int32_t> tfirst((size_t)nt + 1, 0), rstart;
@@ -1932,15 +2224,32 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
         tfirst[(size_t)j] = (int32_t)bl.size();
         const std::vector<int32_t>& c = rs[(size_t)j];
         rstart.insert(rstart.end(), c.begin(), c.end());
-        for (size_t r = 0; r + 1 < c.size(); ++r) {
-            int64_t off = 0, cost = 0;
-            for (int64_t u = c[r]; u < c[r + 1]; ++u) {
-                const int64_t l = len[(size_t)(j * n + u)];
-                toff[(size_t)(j * n + u)] = off;
-                off += (l + kStep - 1) & ~int64_t(kStep - 1);  // padded
-                cost += row_cost(l);
-            }
-            bl.push_back({(int32_t)j, (int32_t)r, c[r], c[r + 1], off, cost});
+        for (size_t r = 0; r + 1 < c.size(); ++r)
+            bl.push_back({(int32_t)j, (int32_t)r, c[r], c[r + 1], 0, 0});
+    }
+    {
+        // the blocks' entries and costs from the prefix sums
+        const size_t m = bl.size();
+        std::vector<int32_t> at(4 * m, 0);
+        for (size_t b = 0; b < m; ++b) {
+            at[4 * b] = bl[b].u0;
+            at[4 * b + 1] = bl[b].u1;
+            at[4 * b + 2] = bl[b].j;
+        }
+        std::vector<int64_t> sums(2 * m);
+        if ((s = ensure(&P.cut, &P.cut_cap, 32 * m + 32)) != GILA_OK) return s;
+        int4* d_at = (int4*)P.cut;
+        int64_t* d_sums = (int64_t*)(d_at + m);
+        GILA_CUDA(cudaMemcpyAsync(d_at, at.data(), 16 * m, cudaMemcpyHostToDevice, g->stream));
+        block_sums_kernel<<<(unsigned)((m + 127) / 128), 128, 0, g->stream>>>(n, cells, (int64_t)m, d_at,
+                                                                             P.pre, d_sums);
+        count_launch();
+        GILA_CUDA(cudaGetLastError());
+        GILA_CUDA(cudaMemcpyAsync(sums.data(), d_sums, 16 * m, cudaMemcpyDeviceToHost, g->stream));
+        GILA_CUDA(cudaStreamSynchronize(g->stream));
+        for (size_t b = 0; b < m; ++b) {
+            bl[b].L = sums[2 * b];
+            bl[b].cost = sums[2 * b + 1];
         }
     }
     tfirst[(size_t)nt] = (int32_t)bl.size();
@@ -1971,8 +2280,7 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
     dir.insert(dir.end(), rstart.begin(), rstart.end());
     dir.insert(dir.end(), rblock.begin(), rblock.end());
     const int64_t tk_len = slots + kStep + 256 * 4;  // slack: the kernel's ring reads ahead
-    gila_status s;
-    if ((s = ensure((void**)&P.toff, &P.toff_cap, sizeof(int64_t) * (size_t)cells)) != GILA_OK)
+    if ((s = ensure((void**)&P.toff, &P.toff_cap, sizeof(int32_t) * (size_t)cells)) != GILA_OK)
         return s;
     if ((s = ensure((void**)&P.blk, &P.blk_cap, sizeof(int64_t) * blk.size())) != GILA_OK) return s;
     if ((s = ensure((void**)&P.bdesc, &P.bdesc_cap, sizeof(int32_t) * bdesc.size())) != GILA_OK)
@@ -1989,8 +2297,6 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
     } else if ((s = ensure(&P.part, &P.part_cap, 2 * esz * (size_t)cells)) != GILA_OK) {
         return s;
     }
-    GILA_CUDA(cudaMemcpyAsync(P.toff, toff.data(), sizeof(int64_t) * cells, cudaMemcpyHostToDevice,
-                              g->stream));
     GILA_CUDA(cudaMemcpyAsync(P.blk, blk.data(), sizeof(int64_t) * blk.size(),
                               cudaMemcpyHostToDevice, g->stream));
     GILA_CUDA(cudaMemcpyAsync(P.bdesc, bdesc.data(), sizeof(int32_t) * bdesc.size(),
@@ -2004,6 +2310,9 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
     GILA_CUDA(cudaMemsetAsync(P.tk + slots, 0, sizeof(uint16_t) * (size_t)(tk_len - slots),
                               g->stream));
     if (nb > 0) {
+        toff_kernel<<<(unsigned)nb, 256, 0, g->stream>>>(n, reinterpret_cast<const int4*>(P.bdesc),
+                                                         P.pre, P.toff);
+        count_launch();
         pad_fill_kernel<<<(unsigned)std::min<int64_t>(nb, 4096), 256, 0, g->stream>>>(
             P.tk, P.blk, wdev, (int)tv, nb);
         count_launch();
@@ -2015,15 +2324,15 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
     const unsigned lay_blocks = (unsigned)((cells + kSpreadWarps - 1) / kSpreadWarps);
     if (g->tune.bank_spread >= 0 && esz == 8)
         block_layout_kernel<16, true><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.toff, P.blk, d_tfirst, d_rstart,
+            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
             d_rblock, P.tk);
     else if (g->tune.bank_spread >= 0)
         block_layout_kernel<8, true><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.toff, P.blk, d_tfirst, d_rstart,
+            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
             d_rblock, P.tk);
     else
         block_layout_kernel<16, false><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.toff, P.blk, d_tfirst, d_rstart,
+            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
             d_rblock, P.tk);
     count_launch();
     GILA_CUDA(cudaGetLastError());
@@ -2078,7 +2387,12 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
             gila_status s = plan_window(g, esz, P, &fits, len, rs, wb, &wmax, &rmax);
             if (s != GILA_OK || P.rows) return s;
             if (fits) {
-                if ((s = build_layout(g, esz, P, 1, 0, len, {rs}, &wb)) != GILA_OK) return s;
+                if ((s = ensure((void**)&P.len, &P.len_cap, sizeof(int32_t) * (size_t)n)) != GILA_OK)
+                    return s;
+                rowlen_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, P.len);
+                count_launch();
+                if ((s = prefix_cells(g, P, n)) != GILA_OK) return s;
+                if ((s = build_layout(g, esz, P, 1, 0, {rs}, &wb)) != GILA_OK) return s;
                 P.window = true;
                 P.tv = (int32_t)wmax;
                 P.rmax = (int32_t)rmax;
@@ -2107,23 +2421,15 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
         geometry(rmax);
     }
     const int64_t cells = n * nt;
-    gila_status s = ensure((void**)&P.len, &P.len_cap, sizeof(int64_t) * (size_t)cells);
+    gila_status s = ensure((void**)&P.len, &P.len_cap, sizeof(int32_t) * (size_t)cells);
     if (s != GILA_OK) return s;
     seglen_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, g->stream>>>(n, g->krow, g->kcol,
                                                                         (int)nt, (int)tv, P.len);
     count_launch();
     GILA_CUDA(cudaGetLastError());
-    std::vector<int64_t> len((size_t)cells);
-    GILA_CUDA(cudaMemcpyAsync(len.data(), P.len, sizeof(int64_t) * cells, cudaMemcpyDeviceToHost,
-                              g->stream));
-    GILA_CUDA(cudaStreamSynchronize(g->stream));
     // each tile's row ranges: blocks of about equal cost (padded entries +
     // a per-row term), at most rmax rows each, about ctas_per_sm per SM
-    std::vector<int64_t> pre((size_t)(nt * (n + 1)), 0);
-    for (int64_t j = 0; j < nt; ++j) {
-        int64_t* pj = pre.data() + j * (n + 1);
-        for (int64_t u = 0; u < n; ++u) pj[u + 1] = pj[u] + row_cost(len[(size_t)(j * n + u)]);
-    }
+    if ((s = prefix_cells(g, P, cells)) != GILA_OK) return s;
     // the block count: at least 5% above what the row limit alone makes,
     // so that a tile with more entries than the others (the hubs' ids) can
     // still be cut finer, and whole waves of one CTA per SM, since blocks of
@@ -2134,8 +2440,9 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
     const int64_t floor_blocks = (n + rmax - 1) / rmax * nt;
     const int64_t want = std::max<int64_t>(target, (floor_blocks * 21 + 19) / 20);
     const int64_t tgt = (want + sms - 1) / sms * sms;
-    const std::vector<std::vector<int32_t>> rs = partition_blocks(pre, n, nt, tgt, rmax);
-    if ((s = build_layout(g, esz, P, nt, tv, len, rs, nullptr)) != GILA_OK) return s;
+    std::vector<std::vector<int32_t>> rs;
+    if ((s = partition_tiles(g, P, n, nt, tgt, rmax, rs)) != GILA_OK) return s;
+    if ((s = build_layout(g, esz, P, nt, tv, rs, nullptr)) != GILA_OK) return s;
     P.tv = (int32_t)tv;
     P.rmax = (int32_t)rmax;
     return GILA_OK;

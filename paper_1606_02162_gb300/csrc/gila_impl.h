@@ -104,7 +104,7 @@ struct TilePlan {
     size_t rdir_cap = 0;
     int64_t* blk = nullptr;          // 2 nb: start in tk and entry count of block b
     size_t blk_cap = 0;
-    int64_t* toff = nullptr;         // nt n: start of (tile j, row u) in tk
+    int32_t* toff = nullptr;         // nt n: start of (tile j, row u) within its block
     size_t toff_cap = 0;
     uint16_t* tk = nullptr;          // tile-relative 16-bit ids in block order
     size_t tk_cap = 0;
@@ -113,8 +113,12 @@ struct TilePlan {
     int32_t* hubs = nullptr;         // vertices of adjacency degree > 64 (combine kernel)
     size_t hubs_cap = 0;
     int32_t nhub = 0;
-    int64_t* len = nullptr;          // nt n segment lengths (plan scratch)
+    int32_t* len = nullptr;          // nt n segment lengths (plan scratch, quality figures)
     size_t len_cap = 0;
+    int64_t* pre = nullptr;          // plan scratch: 2 (nt n + 1) prefix sums of the segments'
+    size_t pre_cap = 0;              // padded lengths, then of their costs
+    void* cut = nullptr;             // plan scratch: cuts of the tiles' rows and their counts
+    size_t cut_cap = 0;
     // window mode: one window of positions per row range, covering every id
     // its rows touch; rows are finished by their range's CTA
     bool window = false;

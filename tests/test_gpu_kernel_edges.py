@@ -144,3 +144,32 @@ def test_batch_row_per_lane(prec, pq, sched):
         # FP64: rounding grows over four iterations (1e-9 as for a few iterations)
         tol = 1e-9 if prec == G.GILA_FP64 else TOL[prec]
         assert np.abs(got - want).max() <= tol * max(scale, 1e-300) + slack, (i, g.name, g.n)
+
+
+# cells (tiles x rows) below, at and above a scan tile of 2048; one tile and
+# more tiles than the warps of a block; blocks of a single row (a target above
+# the rows) and of the most rows; a hub's tile beside nearly empty ones
+@pytest.mark.parametrize("g,k,tune", [
+    (I.barabasi_albert(511, 2, 4), 2, dict(tile_vertices=128)),
+    (I.barabasi_albert(512, 2, 4), 2, dict(tile_vertices=128)),
+    (I.barabasi_albert(4101, 2, 5), 2, dict(tile_vertices=100)),
+    (I.barabasi_albert(40, 2, 6), 2, dict(tile_vertices=8, ctas_per_sm=8)),
+    (I.random_tree(9001, 7), 1, dict(tile_vertices=9002)),
+    (hub_and_gaps(1000, 6000, 50), 2, dict(tile_vertices=512)),
+], ids=["511", "512", "42_tiles", "rows_as_blocks", "one_tile", "hub"])
+@pytest.mark.parametrize("prec", list(TOL), ids=["fp32", "fp32c", "fp64"])
+def test_tile_plan_step(g, k, tune, prec):
+    import torch
+    pos = I.uniform_positions(g.n, 31).astype(np.float32).astype(np.float64)
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, k)
+    _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, 0.4, d=1.1)
+    dt = torch.float64 if prec == G.GILA_FP64 else torch.float32
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, tiled=1, **tune)
+        G.gila_profile_enable(h.handle, 2)
+        x = torch.tensor(pos, dtype=dt, device="cuda")
+        y, disp = torch.empty_like(x), torch.empty_like(x)
+        G.gila_layout_step(h.handle, G.params(k=k, d=1.1, precision=prec), 0.4, x, y, disp)
+        torch.cuda.synchronize()
+        assert G.gila_profile_read_kernel(h.handle)["name"] == "blocked_kernel"
+    assert np.abs(disp.double().cpu().numpy() - want).max() <= TOL[prec] * np.abs(want).max()
