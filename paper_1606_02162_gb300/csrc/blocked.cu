@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
     if (live && gl == 0) finish_vertex<T, COMP>(A, u, pu.x, pu.y, rep, at);
 }
 
-// Length of row u's segment in tile j (binary search on the sorted row).
+// Bounds of row u's segment in tile j (binary search on the sorted row).
 __device__ __forceinline__ void seg_bounds(const int64_t* __restrict__ krow,
                                            const uint32_t* __restrict__ kcol, int64_t u, int j,
                                            int nt, int tv, int64_t* lo, int64_t* hi)
@@ -1055,19 +1055,23 @@ __device__ __forceinline__ void seg_bounds(const int64_t* __restrict__ krow,
 
 __global__ void seglen_kernel(int64_t n, const int64_t* __restrict__ krow,
                               const uint32_t* __restrict__ kcol, int nt, int tv,
-                              int32_t* __restrict__ len)
+                              int32_t* __restrict__ len, int32_t* __restrict__ start)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * nt) return;
     int64_t lo, hi;
     seg_bounds(krow, kcol, i % n, (int)(i / n), nt, tv, &lo, &hi);
     len[i] = (int32_t)(hi - lo);
+    start[i] = (int32_t)(lo - krow[i % n]);
 }
 
-__global__ void rowlen_kernel(int64_t n, const int64_t* __restrict__ krow, int32_t* __restrict__ len)
+__global__ void rowlen_kernel(int64_t n, const int64_t* __restrict__ krow, int32_t* __restrict__ len,
+                              int32_t* __restrict__ start)
 {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u < n) len[u] = (int32_t)(krow[u + 1] - krow[u]);
+    if (u >= n) return;
+    len[u] = (int32_t)(krow[u + 1] - krow[u]);
+    start[u] = 0;
 }
 
 // ---- the plan's cut of every tile's rows into ranges, on the device: with
@@ -1179,8 +1183,9 @@ cell_prefix_kernel(int64_t cells, const int32_t* __restrict__ len, const int64_t
 // range takes at least one row) and at most max_rows rows, for as many caps
 // as the grid is wide: a warp per (cap, tile) walks the tile, finding each
 // range's end by a 32-way search of the prefix costs. counts[x] receives the
-// ranges of all tiles; with cuts, tile j's bounds go to cuts[j stride ...]
-// and their number to tile_counts[j]. A tile stops once it exceeds limit.
+// ranges of all tiles; with cuts, tile j's bounds go to
+// cuts[(x nt + j) stride ...] and their number to tile_counts[x nt + j]. A
+// tile stops once it exceeds limit.
 __global__ void __launch_bounds__(256)
 cut_kernel(int64_t n, int nt, const int64_t* __restrict__ pre, const int64_t* __restrict__ caps,
            int64_t max_rows, int64_t limit, int* __restrict__ counts, int32_t* __restrict__ cuts,
@@ -1192,7 +1197,8 @@ cut_kernel(int64_t n, int nt, const int64_t* __restrict__ pre, const int64_t* __
     const int64_t cap = caps[blockIdx.x];
     const int64_t* p = pre + (int64_t)j * n;
     int64_t s = 0, count = 0;
-    if (cuts && lane == 0) cuts[j * stride] = 0;
+    if (cuts) cuts += ((int64_t)blockIdx.x * nt + j) * stride;
+    if (cuts && lane == 0) cuts[0] = 0;
     while (s < n && count <= limit) {
         const int64_t most = p[s] + cap;
         int64_t lo = s + 1, hi = s + max_rows < n ? s + max_rows : n;
@@ -1206,11 +1212,11 @@ cut_kernel(int64_t n, int nt, const int64_t* __restrict__ pre, const int64_t* __
         }
         s = lo;
         ++count;
-        if (cuts && lane == 0 && count < stride) cuts[j * stride + count] = (int32_t)s;
+        if (cuts && lane == 0 && count < stride) cuts[count] = (int32_t)s;
     }
     if (lane == 0) {
         atomicAdd(&counts[blockIdx.x], (int)(count < INT32_MAX / 2 ? count : INT32_MAX / 2));
-        if (tile_counts) tile_counts[j] = (int)count;
+        if (tile_counts) tile_counts[(int64_t)blockIdx.x * nt + j] = (int)count;
     }
 }
 
@@ -1248,7 +1254,8 @@ __global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t*
 // Copy every (tile, row) segment into its block's share storage as 16-bit
 // ids relative to the tile: entry p of the block, held by the share of
 // thread t (s = p - lane_start(L, t)), goes to slot
-// (t / 32) 32 lane_len(L) + 256 (s / 8) + 8 (t % 32) + s % 8.
+// (t / 32) 32 lane_len(L) + 256 (s / 8) + 8 (t % 32) + s % 8. The slots that
+// no entry takes hold the padding id already (pad_fill_kernel).
 //
 // With SPREAD each segment's ids are also ordered for blocked_kernel's
 // shared-memory gathers. A warp's gather is served in groups of G lanes
@@ -1260,19 +1267,42 @@ __global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t*
 // aims at residue (t + s) mod G, distinct across the group for every s. A
 // row's sum does not depend on the order of its entries (up to rounding)
 // and a segment is one row, so its ids are dealt to its entries: each entry
-// takes an id of its target residue while one is left (lanes in order),
-// else one of the nearest residue above it (cyclically) that has ids left.
-// One warp per segment, through shared memory by chunks of at most
-// kSpreadChunk entries: count the chunk's residues, group its ids by residue
-// (stable), deal them 32 entries at a time.
-// A larger chunk leaves fewer entries without their target residue (each
-// such entry costs its half-warp one more gather wavefront): 2048 entries
-// held as 16-bit relative ids (4 KB a warp) against 1024 as 32-bit ids took
-// Chung-Lu n = 250,000, k = 3 from 4.27 to 4.18 ms per launch, the plan
-// from 174 to 170 ms; 4096 gave 4.15 ms but a 229 ms plan (half the
-// occupancy).
-constexpr int kSpreadWarps = 4;
+// takes an id of its target residue while one is left, and the entries left
+// over take the ids left over.
+//
+// Blocks come from the grid, so that a warp looks its block up once and then
+// takes rows of it. Three forms by length:
+// - up to 32 entries (two rows of up to 16 at once): an id and an entry per
+//   lane, matched by (residue, rank) through a table in shared memory;
+// - longer: by chunks of at most kSpreadChunk entries; the ids grouped by
+//   residue with a counter per lane and residue (no atomics, no matching),
+//   then dealt 32 entries at a time; the targets of 32 entries of one share
+//   are consecutive residues, so that an entry's rank among the entries of
+//   its target is its lane / G and every residue gives 32 / G ids.
+// A larger chunk leaves fewer entries without their target residue (each such
+// entry costs its half-warp one more gather wavefront): 2048 against 1024
+// took Chung-Lu n = 250,000, k = 3 from 4.27 to 4.18 ms per launch, 4096 gave
+// 4.15 ms at half the occupancy here.
+// The layout of Chung-Lu n = 60,000, k = 3 took 7.85 ms with a warp per
+// (tile, row), atomics and a matching step per 32 entries, 3.74 now; BA
+// n = 333,334, k = 2 (segments of 12 entries) 3.78 -> 1.34 ms.
+constexpr int kSpreadWarps = 8;
 constexpr int kSpreadChunk = 2048;
+
+// Shared memory of one warp of the layout kernel.
+struct SpreadSmem {
+    uint16_t in[kSpreadChunk];            // the chunk's relative ids by residue
+    union {
+        uint32_t off[16][32];             // next place of (residue, lane) while grouping
+        struct {                          // short rows:
+            uint8_t slot[32 * 32];        // entry of (residue, rank)
+            uint8_t rest[32];             // entries left over
+            int32_t cnt[2][32];           // ids and entries of each residue
+        } s;
+    };
+    uint32_t left[kSpreadChunk / 32];     // entries without an id of their residue, a bit each
+    int32_t ask[32], base[32];            // counts and places by residue
+};
 
 // Every slot of block b's share storage set to the block's padding id (its
 // far slot) before the layout kernel writes the entries: the slots past
@@ -1293,148 +1323,304 @@ __global__ void pad_fill_kernel(uint16_t* __restrict__ tk, const int64_t* __rest
     }
 }
 
-template <int G, bool SPREAD>
-__global__ void __launch_bounds__(kSpreadWarps * 32) block_layout_kernel(
-    int64_t n, const int64_t* __restrict__ krow, const uint32_t* __restrict__ kcol, int nt,
-    int tv, const int64_t* __restrict__ wbase, const int32_t* __restrict__ len,
-    const int32_t* __restrict__ toff, const int64_t* __restrict__ blk, const int32_t* __restrict__ tfirst,
-    const int32_t* __restrict__ rstart, const int32_t* __restrict__ rblock,
-    uint16_t* __restrict__ tk)
+// The share (thread of blocked_kernel) that holds entry p of a block of L
+// entries; inv = kBThreads / L.
+__device__ __forceinline__ int share_of(int32_t L, int32_t p, float inv)
 {
-    __shared__ uint16_t s_in[kSpreadWarps][kSpreadChunk];  // the chunk's relative ids by residue
-    __shared__ int s_run[kSpreadWarps][G];
-    __shared__ int s_ask[kSpreadWarps][G];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n * nt) return;  // warp-uniform
-    const int j = (int)(i / n);
-    const int64_t u = i % n;
-    const int seglen = len[i];
-    if (seglen == 0) return;
-    // the segment starts after the row's segments in earlier tiles
-    int64_t lo = krow[u];
-    for (int jj = lane; jj - lane < j; jj += 32)
-        lo += __reduce_add_sync(kFull, jj < j ? (unsigned)len[(int64_t)jj * n + u] : 0u);
-    const int64_t hi = lo + seglen;
-    // the range of tile j that holds row u (tile j's ranges: blocks
-    // tfirst[j] .. tfirst[j + 1] - 1 in tile order, their row bounds at
-    // rstart + tfirst[j] + j), and that range's block
-    const int32_t f0 = tfirst[j];
-    const int32_t* st = rstart + f0 + j;
-    int ra = 0, rb = tfirst[j + 1] - f0 - 1;
-    while (ra < rb) {
-        const int mid = (ra + rb + 1) >> 1;
-        if (st[mid] <= u) ra = mid; else rb = mid - 1;
-    }
-    const int64_t b = rblock[f0 + ra];
-    // ids are relative to tile j, or in window mode to block b's window;
-    // the padding takes the far slot one past the tile or window
-    const uint32_t tb = wbase ? (uint32_t)wbase[2 * b] : (uint32_t)j * (uint32_t)tv;
-    const uint16_t pad = wbase ? (uint16_t)wbase[2 * b + 1] : (uint16_t)tv;
-    const int64_t bsp = blk[2 * b];
-    const int32_t L = (int32_t)blk[2 * b + 1];
-    const int32_t m8 = lane_len(L);
-    const int32_t S0 = toff[i], S1 = S0 + (int32_t)(hi - lo);
-    const int32_t S8 = S0 + (int32_t)((hi - lo + kStep - 1) & ~int64_t(kStep - 1));  // padded end
-    // the share holding entry p (t follows p, which only grows) and the slot
-    int t = (int)((int64_t)S0 * kBThreads / L);
-    int32_t sidx = 0;  // p's index in its share, set by place
-    auto place = [&](int32_t p) -> int64_t {
-        while (t > 0 && lane_start(L, t) > p) --t;
-        while (t < kBThreads - 1 && lane_start(L, t + 1) <= p) ++t;
-        sidx = p - lane_start(L, t);
-        return bsp + (int64_t)(t >> 5) * 32 * m8 + 256 * (sidx >> 3) + 8 * (t & 31) + (sidx & 7);
-    };
-    if (!SPREAD) {
-        for (int32_t p = S0 + lane; p < S8; p += 32)
-            tk[place(p)] = (p < S1) ? (uint16_t)(kcol[lo + (p - S0)] - tb) : pad;
-        return;
-    }
-    uint16_t* in = s_in[wl];
-    int* run = s_run[wl];
-    int* ask = s_ask[wl];
-    for (int32_t c0 = S0; c0 < S1; c0 += kSpreadChunk) {
-        const int len = (S1 - c0 < kSpreadChunk) ? S1 - c0 : kSpreadChunk;
-        const uint32_t* src = kcol + lo + (c0 - S0);
-        // residue counts of the chunk and their exclusive prefix (lane c: residue c)
-        if (lane < G) run[lane] = 0;
-        __syncwarp();
-        for (int e = lane; e < len; e += 32) atomicAdd(&run[(src[e] - tb) % G], 1);
-        __syncwarp();
-        const int cnt = (lane < G) ? run[lane] : 0;
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int cstart = incl - cnt;
-        __syncwarp();
-        if (lane < G) run[lane] = cstart;
-        __syncwarp();
-        // stable grouping by residue
-        for (int e0 = 0; e0 < len; e0 += 32) {
-            const int e = e0 + lane;
-            const bool act = e < len;
-            const uint32_t id = act ? src[e] : 0u;
-            const int c = act ? (int)((id - tb) % G) : G + lane;
-            const unsigned m = __match_any_sync(kFull, c);
-            const int o = act ? run[c] + __popc(m & ((1u << lane) - 1u)) : 0;
-            __syncwarp();
-            if (act && lane == 31 - __clz(m)) run[c] += __popc(m);
-            __syncwarp();
-            if (act) in[o] = (uint16_t)(id - tb);
-        }
-        __syncwarp();  // the grouped ids are visible to the whole warp
+    // the last t with L t / kBThreads below the end of p's group of eight
+    int t = (int)((float)((p & ~(kStep - 1)) + kStep) * inv);
+    t = t < kBThreads ? t : kBThreads - 1;
+    while (t > 0 && lane_start(L, t) > p) --t;
+    while (t < kBThreads - 1 && lane_start(L, t + 1) <= p) ++t;
+    return t;
+}
 
-        // deal: lane c < G keeps residue c's ids left and taken
-        int rem = cnt, used = 0;
-        for (int e0 = 0; e0 < len; e0 += 32) {
-            const int e = e0 + lane;
-            const bool act = e < len;
-            const int64_t d = act ? place(c0 + e) : 0;
-            const int want = act ? (int)(((t % G) + sidx) % G) : 0;
-            // the target residue for as many lanes as it has ids left, in lane order
-            const unsigned m = __match_any_sync(kFull, act ? want : G + lane);
-            const int rank = __popc(m & ((1u << lane) - 1u));
-            const int left = __shfl_sync(kFull, rem, want);
-            const int base = __shfl_sync(kFull, cstart + used, want);
-            const bool got = act && rank < left;
-            uint16_t id = got ? in[base + rank] : (uint16_t)0;
-            // residue c's lane takes off the lanes that asked for c (at most rem)
-            if (lane < G) ask[lane] = 0;
-            __syncwarp();
-            if (act && rank == 0) ask[want] = __popc(m);
-            __syncwarp();
-            if (lane < G) {
-                const int give = (ask[lane] < rem) ? ask[lane] : rem;
-                rem -= give;
-                used += give;
-            }
-            // the others in lane order: the nearest residue at or above the
-            // target (cyclically) that has ids left
-            unsigned pend = __ballot_sync(kFull, act && !got);
-            while (pend) {
-                const int l = __ffs(pend) - 1;
-                const int wt = __shfl_sync(kFull, want, l);
-                const unsigned av = __ballot_sync(kFull, lane < G && rem > 0) & ((1u << G) - 1u);
-                if (av == 0) break;  // cannot happen: ids left equal entries left
-                const unsigned rot = ((av >> wt) | (av << (G - wt))) & ((1u << G) - 1u);
-                const int c = (wt + __ffs(rot) - 1) % G;
-                const int at = __shfl_sync(kFull, cstart + used, c);
-                if (lane == c) {
-                    --rem;
-                    ++used;
-                }
-                if (lane == l) id = in[at];
-                pend &= pend - 1;
-            }
-            if (act) tk[d] = id;
-        }
-        __syncwarp();  // the next chunk reuses the buffers
+// Slot of entry number sidx of share t (see above), from the block's start.
+__device__ __forceinline__ int64_t share_slot(int t, int32_t sidx, int32_t m8)
+{
+    return (int64_t)(t >> 5) * 32 * m8 + 256 * (int64_t)(sidx >> 3) + 8 * (t & 31) + (sidx & 7);
+}
+
+// One entry and one id per lane (entry p of the block), of one row or, with
+// `second` telling their lanes apart, of two: dealt by residue within a row.
+template <int G>
+__device__ __forceinline__ void deal_short(SpreadSmem& S, bool act, int32_t p, uint32_t id,
+                                           bool second, int32_t L, int32_t m8, float inv,
+                                           uint16_t* tk, int lane)
+{
+    const int key = second ? 16 : 0;
+    int64_t at = 0;
+    int want = 0;
+    if (act) {
+        const int t = share_of(L, p, inv);
+        const int32_t sidx = p - lane_start(L, t);
+        at = share_slot(t, sidx, m8);
+        want = ((t + sidx) & (G - 1)) + key;
     }
-    // the padding (at most 7 entries, lanes 0-6)
-    if (S1 + lane < S8) tk[place(S1 + lane)] = pad;
+    const unsigned lt = lanemask_lt();
+    const int has = (int)(id & (G - 1)) + key;
+    const unsigned mw = __match_any_sync(kFull, act ? want : 64 + lane);
+    const unsigned mh = __match_any_sync(kFull, act ? has : 64 + lane);
+    const int rw = __popc(mw & lt), rh = __popc(mh & lt);
+    S.s.cnt[0][lane] = 0;
+    S.s.cnt[1][lane] = 0;
+    __syncwarp();
+    if (act) {
+        S.s.slot[want * 32 + rw] = (uint8_t)lane;
+        if (rw == 0) S.s.cnt[1][want] = __popc(mw);
+        if (rh == 0) S.s.cnt[0][has] = __popc(mh);
+    }
+    __syncwarp();
+    const bool served = act && rw < S.s.cnt[0][want];  // this lane's entry finds its residue
+    const bool placed = act && rh < S.s.cnt[1][has];   // this lane's id finds an entry
+    // the rest in lane order: a row has as many entries as ids left over, so
+    // that the k-th entry left of all the lanes and the k-th id left belong
+    // to the same row
+    const unsigned er = __ballot_sync(kFull, act && !served), ir = __ballot_sync(kFull, act && !placed);
+    if (act && !served) S.s.rest[__popc(er & lt)] = (uint8_t)lane;
+    __syncwarp();
+    int to = lane;
+    if (placed) to = S.s.slot[has * 32 + rh];
+    else if (act) to = S.s.rest[__popc(ir & lt)];
+    const int64_t dst = __shfl_sync(kFull, at, to);
+    if (act) tk[dst] = (uint16_t)id;
+    __syncwarp();  // the next rows reuse the tables
+}
+
+template <int G, bool SPREAD>
+__global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
+    int64_t n, const int64_t* __restrict__ krow, const uint32_t* __restrict__ kcol, int tv,
+    const int64_t* __restrict__ wbase, const int32_t* __restrict__ len,
+    const int32_t* __restrict__ start, const int32_t* __restrict__ toff,
+    const int64_t* __restrict__ blk, const int4* __restrict__ bdesc, uint16_t* __restrict__ tk_all)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SpreadSmem& S = reinterpret_cast<SpreadSmem*>(smem_raw)[warp];
+    const int64_t b = blockIdx.x;
+    const int4 bd = bdesc[b];
+    const int j = bd.z;
+    const int32_t L = (int32_t)blk[2 * b + 1];
+    if (L == 0) return;
+    // ids are relative to tile j, or in window mode to block b's window
+    const uint32_t tb = wbase ? (uint32_t)wbase[2 * b] : (uint32_t)j * (uint32_t)tv;
+    uint16_t* tk = tk_all + blk[2 * b];
+    const int32_t m8 = lane_len(L);
+    const float inv = (float)kBThreads / (float)L;
+    const int32_t* clen = len + (int64_t)j * n;
+    const int32_t* cstart = start + (int64_t)j * n;
+    const int32_t* coff = toff + (int64_t)j * n;
+
+    auto row = [&](int64_t u, int rl) {  // one row of rl entries by the whole warp
+        const uint32_t* src = kcol + krow[u] + cstart[u];
+        const int32_t S0 = coff[u];
+        if (!SPREAD) {
+            for (int e = lane; e < rl; e += 32) {
+                const int t = share_of(L, S0 + e, inv);
+                tk[share_slot(t, S0 + e - lane_start(L, t), m8)] = (uint16_t)(src[e] - tb);
+            }
+            return;
+        }
+        if (rl <= 32) {
+            const uint32_t id = lane < rl ? src[lane] - tb : 0u;
+            deal_short<G>(S, lane < rl, S0 + lane, id, false, L, m8, inv, tk, lane);
+            return;
+        }
+        for (int32_t c0 = 0; c0 < rl; c0 += kSpreadChunk) {
+            const int cl = rl - c0 < kSpreadChunk ? rl - c0 : kSpreadChunk;
+            const uint32_t* cs = src + c0;
+            // ids of each residue on this lane
+#pragma unroll
+            for (int c = 0; c < G; ++c) S.off[c][lane] = 0;
+#pragma unroll 1
+            for (int e0 = lane; e0 < cl; e0 += 256) {
+                uint32_t id[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) id[x] = e0 + 32 * x < cl ? cs[e0 + 32 * x] - tb : 0u;
+#pragma unroll
+                for (int x = 0; x < 8; ++x)
+                    if (e0 + 32 * x < cl) ++S.off[id[x] & (G - 1)][lane];
+            }
+            // counters to places: exclusive prefix over residues, then lanes
+            int cnt = 0, cst = 0;  // lane c: residue c's ids and where they start
+            {
+                int run = 0;
+#pragma unroll
+                for (int c = 0; c < G; ++c) {
+                    const int mine = (int)S.off[c][lane];
+                    const int incl = warp_inclusive_scan(mine, lane);
+                    S.off[c][lane] = (uint32_t)(run + incl - mine);
+                    const int tot = __shfl_sync(kFull, incl, 31);
+                    if (lane == c) {
+                        cnt = tot;
+                        cst = run;
+                    }
+                    run += tot;
+                }
+            }
+#pragma unroll 1
+            for (int e0 = lane; e0 < cl; e0 += 256) {
+                uint32_t id[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) id[x] = e0 + 32 * x < cl ? cs[e0 + 32 * x] - tb : 0u;
+#pragma unroll
+                for (int x = 0; x < 8; ++x)
+                    if (e0 + 32 * x < cl) S.in[S.off[id[x] & (G - 1)][lane]++] = (uint16_t)id[x];
+            }
+            __syncwarp();
+            // deal: lane c < G keeps residue c's next id and the ids left
+            constexpr int kPer = 32 / G;  // entries of one target in 32 consecutive ones
+            int rem = cnt, next = cst, nleft = 0;
+            int t = share_of(L, S0 + c0, inv);
+            int32_t sb = lane_start(L, t), se = lane_start(L, t + 1);
+            for (int e0 = 0; e0 < cl;) {
+                const int32_t p0 = S0 + c0 + e0;
+                while (se <= p0 && t < kBThreads - 1) {  // the share that holds the first entry
+                    ++t;
+                    sb = se;
+                    se = lane_start(L, t + 1);
+                }
+                const int32_t s0 = p0 - sb;  // a multiple of 8, like every bound here
+                const int same = (se - p0 < cl - e0 ? se - p0 : cl - e0) >> 5;
+                if (same > 0) {
+                    // whole groups of 32 entries of one share: a lane's target
+                    // is the same in all of them, and group i takes the ids
+                    // kPer i .. of every residue
+                    const int want = (t + s0 + lane) & (G - 1), rank = lane / G;
+                    const int have = __shfl_sync(kFull, rem, want);
+                    const uint16_t* from = S.in + __shfl_sync(kFull, next, want) + rank;
+                    uint16_t* to = tk + (int64_t)(t >> 5) * 32 * m8 + 8 * (t & 31) +
+                                   256 * ((s0 + lane) >> 3) + (lane & 7);
+                    if (__all_sync(kFull, rank + kPer * (same - 1) < have)) {
+#pragma unroll 4
+                        for (int i = 0; i < same; ++i) to[1024 * i] = from[kPer * i];
+                        for (int i = lane; i < same; i += 32) S.left[(e0 >> 5) + i] = 0u;
+                    } else {
+                        for (int i = 0; i < same; ++i) {
+                            const bool got = rank + kPer * i < have;
+                            if (got) to[1024 * i] = from[kPer * i];
+                            const unsigned lm = __ballot_sync(kFull, !got);
+                            if (lane == 0) S.left[(e0 >> 5) + i] = lm;
+                            nleft += __popc(lm);
+                        }
+                    }
+                    if (lane < G) {
+                        const int give = kPer * same < rem ? kPer * same : rem;
+                        rem -= give;
+                        next += give;
+                    }
+                    e0 += 32 * same;
+                    continue;
+                }
+                // 32 entries that reach into the next share, or the last ones
+                const int e = e0 + lane;
+                const bool act = e < cl;
+                int32_t sidx = s0 + lane;
+                int tl = t;
+                if (act && p0 + lane >= se) {
+                    tl = share_of(L, p0 + lane, inv);
+                    sidx = p0 + lane - lane_start(L, tl);
+                }
+                const int want = (tl + sidx) & (G - 1);
+                const unsigned m = __match_any_sync(kFull, act ? want : G + lane);
+                const int rank = __popc(m & lanemask_lt());
+                S.ask[lane] = 0;
+                __syncwarp();
+                if (act && rank == 0) S.ask[want] = __popc(m);
+                __syncwarp();
+                const int have = __shfl_sync(kFull, rem, want);
+                const int from = __shfl_sync(kFull, next, want);
+                const bool got = act && rank < have;
+                if (got) tk[share_slot(tl, sidx, m8)] = S.in[from + rank];
+                const unsigned lm = __ballot_sync(kFull, act && !got);
+                if (lane == 0) S.left[e0 >> 5] = lm;
+                nleft += __popc(lm);
+                if (lane < G) {
+                    const int give = S.ask[lane] < rem ? S.ask[lane] : rem;
+                    rem -= give;
+                    next += give;
+                }
+                __syncwarp();
+                e0 += 32;
+            }
+            // the entries left over take the ids left over, in order
+            if (nleft > 0) {
+                if (lane >= G) rem = 0;
+                int incl = rem;
+#pragma unroll
+                for (int o = 1; o < G; o <<= 1) {
+                    const int v = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                S.ask[lane] = lane < G ? incl : INT32_MAX;        // ids left up to residue c
+                S.base[lane] = next - (incl - rem);               // the k-th id left: in[this + k]
+                __syncwarp();
+                // listed first (the counters' place is free), then one a lane
+                uint16_t* list = reinterpret_cast<uint16_t*>(S.off);
+                constexpr int kList = (int)(sizeof(S.off) / 2);
+                for (int l0 = 0; l0 < nleft; l0 += kList) {
+                    int before = -l0;
+                    for (int w0 = 0; w0 * 32 < cl; w0 += 32) {  // a word of 32 entries per lane
+                        uint32_t m = (w0 + lane) * 32 < cl ? S.left[w0 + lane] : 0u;
+                        const int mine = __popc(m);
+                        const int upto = warp_inclusive_scan(mine, lane);
+                        for (int k = before + upto - mine; m; m &= m - 1, ++k)
+                            if (k >= 0 && k < kList)
+                                list[k] = (uint16_t)((w0 + lane) * 32 + __ffs(m) - 1);
+                        before += __shfl_sync(kFull, upto, 31);
+                    }
+                    __syncwarp();
+                    const int stop = nleft - l0 < kList ? nleft - l0 : kList;
+                    for (int x = lane; x < stop; x += 32) {
+                        const int k = l0 + x;
+                        int c = 0;  // the residue of the k-th id left
+#pragma unroll
+                        for (int o = G / 2; o > 0; o >>= 1)
+                            if (S.ask[c + o - 1] <= k) c += o;
+                        const int32_t p = S0 + c0 + list[x];
+                        const int ts = share_of(L, p, inv);
+                        tk[share_slot(ts, p - lane_start(L, ts), m8)] = S.in[S.base[c] + k];
+                    }
+                    __syncwarp();
+                }
+            }
+            __syncwarp();  // the next chunk reuses the buffers
+        }
+    };
+    // this CTA's part of the block's rows, taken in pairs by its warps
+    __shared__ int s_next;
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    const int64_t rows = bd.y - bd.x;
+    const int64_t u0 = bd.x + rows * blockIdx.y / gridDim.y;
+    const int64_t u1 = bd.x + rows * (blockIdx.y + 1) / gridDim.y;
+    for (;;) {
+        int64_t u = 0;
+        if (lane == 0) u = u0 + 2 * (int64_t)atomicAdd(&s_next, 1);
+        u = __shfl_sync(kFull, u, 0);
+        if (u >= u1) break;
+        const int l0 = clen[u], l1 = u + 1 < u1 ? clen[u + 1] : 0;
+        if (SPREAD && l0 <= 16 && l1 <= 16) {
+            if (l0 + l1 == 0) continue;
+            const bool second = lane >= 16;
+            const int64_t v = second ? u + 1 : u;
+            const int e = lane & 15;
+            const bool act = e < (second ? l1 : l0);
+            int32_t p = 0;
+            uint32_t id = 0;
+            if (act) {
+                p = coff[v] + e;
+                id = kcol[krow[v] + cstart[v] + e] - tb;
+            }
+            deal_short<G>(S, act, p, id, second, L, m8, inv, tk, lane);
+            continue;
+        }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int rl = h ? l1 : l0;
+            if (rl) row(u + h, rl);
+        }
+    }
 }
 
 template <class T, int MODEL, bool COMP, bool WIN>
@@ -1512,6 +1698,7 @@ constexpr int kMetSmemMax = kSmemCap - 12 * 1024;  // the tile's share of shared
 struct MetricArgs {
     const int64_t* krow;
     const int32_t* len;    // tile mode: nt n segment lengths (row u's entries in tile j)
+    const int32_t* start;  // ... and their starts within the rows
     const uint32_t* kcol;
     const int4* bdesc;     // nb: first row, end row and tile of block b
     const int64_t* wbase;  // window mode: 2 nb (first id, length), else null
@@ -1594,13 +1781,12 @@ __global__ void __launch_bounds__(kMetThreads, 1) khop_metric_kernel(const Metri
             int64_t lo = 0, hi = 0;
             if (threadIdx.x < kMetBatch && u < u1 && tb + tn > u + 1) {
                 // the row's entries in this tile: the whole row in window
-                // mode; in tile mode the segment after the row's segments in
-                // earlier tiles (their lengths, summed in order)
+                // mode, in tile mode its segment
                 lo = A.krow[u];
                 if (A.wbase) {
                     hi = A.krow[u + 1];
                 } else {
-                    for (int jj = 0; jj < j; ++jj) lo += A.len[(int64_t)jj * A.n + u];
+                    lo += A.start[(int64_t)j * A.n + u];
                     hi = lo + A.len[(int64_t)j * A.n + u];
                 }
                 if (tb <= u) {
@@ -1762,7 +1948,6 @@ void free_tile_plans(gila_graph* g)
         cudaFree(P.sdesc);
         cudaFree(P.deg);
         cudaFree(P.bdesc);
-        cudaFree(P.rdir);
         cudaFree(P.blk);
         cudaFree(P.toff);
         cudaFree(P.tk);
@@ -1914,17 +2099,25 @@ gila_status prefix_cells(gila_graph* g, TilePlan& P, int64_t cells)
 // the mean and one more range than the target sent a few CTAs into a second
 // wave (Barabasi-Albert n = 100,000, k = 2: 156 CTAs on 152 SMs, the SMs busy
 // 54% of the kernel's time). The cap is searched from below, the mean cost of
-// a block, 32 caps at a time: to within 1/512 of itself in two rounds.
+// a block, 256 caps at once in steps of 1/128 of it (a cap's walk is a chain
+// of dependent loads, 0.2 ms for 150 to 1200 blocks, so many caps at once
+// cost what one does). The cuts of every cap are written where they fit
+// kCutBytes, else those of the chosen one by another launch.
+constexpr size_t kCutBytes = (size_t)64 << 20;
+
 gila_status partition_tiles(gila_graph* g, TilePlan& P, int64_t n, int64_t nt, int64_t target,
                             int64_t max_rows, std::vector<std::vector<int32_t>>& rs)
 {
-    constexpr int kCaps = 32;
+    constexpr int kCaps = 256;
     const int64_t cells = n * nt;
     const int64_t* pre = P.pre + cells + 1;
     target = std::max<int64_t>(target, nt * ((n + max_rows - 1) / max_rows));
     const int64_t stride = target + 2;
-    const size_t head = kCaps * 12 + sizeof(int) * (size_t)nt, at_cuts = (head + 15) & ~size_t(15);
-    gila_status s = ensure(&P.cut, &P.cut_cap, at_cuts + sizeof(int32_t) * (size_t)(nt * stride));
+    const size_t per_cap = sizeof(int32_t) * (size_t)(nt * stride);
+    const bool every = per_cap * kCaps <= kCutBytes;
+    const size_t slots = every ? kCaps : 1;  // caps whose cuts are written
+    const size_t at_cuts = (kCaps * 12 + sizeof(int) * (size_t)nt * slots + 15) & ~size_t(15);
+    gila_status s = ensure(&P.cut, &P.cut_cap, at_cuts + per_cap * slots);
     if (s != GILA_OK) return s;
     int64_t* d_caps = (int64_t*)P.cut;
     int* d_counts = (int*)(d_caps + kCaps);
@@ -1933,10 +2126,10 @@ gila_status partition_tiles(gila_graph* g, TilePlan& P, int64_t n, int64_t nt, i
     int64_t total = 0;
     GILA_CUDA(cudaMemcpyAsync(&total, pre + cells, sizeof(int64_t), cudaMemcpyDeviceToHost, g->stream));
     GILA_CUDA(cudaStreamSynchronize(g->stream));
-    int64_t caps[kCaps];
-    int counts[kCaps];
+    std::vector<int64_t> caps(kCaps);
+    std::vector<int> counts(kCaps);
     auto count = [&](int used, bool write) -> gila_status {
-        GILA_CUDA(cudaMemcpyAsync(d_caps, caps, sizeof(int64_t) * (size_t)used,
+        GILA_CUDA(cudaMemcpyAsync(d_caps, caps.data(), sizeof(int64_t) * (size_t)used,
                                   cudaMemcpyHostToDevice, g->stream));
         GILA_CUDA(cudaMemsetAsync(d_counts, 0, sizeof(int) * kCaps, g->stream));
         cut_kernel<<<dim3((unsigned)used, (unsigned)((nt + 7) / 8)), 256, 0, g->stream>>>(
@@ -1944,44 +2137,34 @@ gila_status partition_tiles(gila_graph* g, TilePlan& P, int64_t n, int64_t nt, i
             write ? d_tiles : nullptr);
         count_launch();
         GILA_CUDA(cudaGetLastError());
-        GILA_CUDA(cudaMemcpyAsync(counts, d_counts, sizeof(int) * (size_t)used,
+        GILA_CUDA(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int) * (size_t)used,
                                   cudaMemcpyDeviceToHost, g->stream));
         GILA_CUDA(cudaStreamSynchronize(g->stream));
         return GILA_OK;
     };
-    // below `lo` no cut reaches the target; at total + 1 every one does
-    int64_t lo = std::max<int64_t>(1, total / target), hi = total + 1;
-    for (int64_t width = lo / 16 + 1; lo < total + 1; width *= 4) {
-        for (int i = 0; i < kCaps; ++i) caps[i] = std::min<int64_t>(lo + width * i, total + 1);
-        if ((s = count(kCaps, false)) != GILA_OK) return s;
-        int i = 0;
-        while (i < kCaps && counts[i] > target) ++i;
-        if (i < kCaps) {
-            hi = caps[i];
-            if (i > 0) lo = caps[i - 1];
-            else lo = hi - 1;
-            break;
-        }
-        lo = caps[kCaps - 1];
-    }
-    if (hi - lo > 1) {
-        const int64_t width = (hi - lo + kCaps - 1) / kCaps;
-        for (int i = 0; i < kCaps; ++i) caps[i] = std::min<int64_t>(lo + width * (i + 1), hi);
-        if ((s = count(kCaps, false)) != GILA_OK) return s;
+    // at total + 1 every cut reaches the target
+    int64_t lo = std::max<int64_t>(1, total / target);
+    int pick = kCaps;
+    for (int64_t width = lo / 128 + 1; pick == kCaps; width *= 16) {
         for (int i = 0; i < kCaps; ++i)
-            if (counts[i] <= target) {
-                hi = caps[i];
-                break;
-            }
+            caps[(size_t)i] = std::min<int64_t>(lo + width * i, total + 1);
+        if ((s = count(kCaps, every)) != GILA_OK) return s;
+        pick = 0;
+        while (pick < kCaps && counts[(size_t)pick] > target) ++pick;
+        lo = caps[kCaps - 1];
+        if (pick == kCaps && lo == total + 1) return fail(GILA_ESTATE, "block partition");  // cannot happen
     }
-    caps[0] = hi;
-    if ((s = count(1, true)) != GILA_OK) return s;
-    if (counts[0] > target) return fail(GILA_ESTATE, "block partition");  // cannot happen
+    size_t slot = (size_t)pick;
+    if (!every) {
+        caps[0] = caps[(size_t)pick];
+        if ((s = count(1, true)) != GILA_OK) return s;
+        slot = 0;
+    }
     std::vector<int> tiles((size_t)nt);
     std::vector<int32_t> cuts((size_t)(nt * stride));
-    GILA_CUDA(cudaMemcpyAsync(tiles.data(), d_tiles, sizeof(int) * (size_t)nt,
+    GILA_CUDA(cudaMemcpyAsync(tiles.data(), d_tiles + slot * (size_t)nt, sizeof(int) * (size_t)nt,
                               cudaMemcpyDeviceToHost, g->stream));
-    GILA_CUDA(cudaMemcpyAsync(cuts.data(), d_cuts, sizeof(int32_t) * cuts.size(),
+    GILA_CUDA(cudaMemcpyAsync(cuts.data(), d_cuts + slot * (size_t)(nt * stride), per_cap,
                               cudaMemcpyDeviceToHost, g->stream));
     GILA_CUDA(cudaStreamSynchronize(g->stream));
     rs.resize((size_t)nt);
@@ -2217,13 +2400,8 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
         int64_t L, cost;
     };
     std::vector<Blk> bl;
-    // directory for the layout kernel: tfirst (nt + 1), then each tile's
-    // range bounds (nb + nt), then the block of each (tile, range) (nb)
-    std::vector<int32_t> tfirst((size_t)nt + 1, 0), rstart;
     for (int64_t j = 0; j < nt; ++j) {
-        tfirst[(size_t)j] = (int32_t)bl.size();
         const std::vector<int32_t>& c = rs[(size_t)j];
-        rstart.insert(rstart.end(), c.begin(), c.end());
         for (size_t r = 0; r + 1 < c.size(); ++r)
             bl.push_back({(int32_t)j, (int32_t)r, c[r], c[r + 1], 0, 0});
     }
@@ -2252,14 +2430,13 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
             bl[b].cost = sums[2 * b + 1];
         }
     }
-    tfirst[(size_t)nt] = (int32_t)bl.size();
     const int64_t nb = (int64_t)bl.size();
     std::vector<int32_t> order((size_t)nb);
     for (int64_t b = 0; b < nb; ++b) order[(size_t)b] = (int32_t)b;
     std::stable_sort(order.begin(), order.end(),
                      [&](int32_t x, int32_t y) { return bl[(size_t)x].cost > bl[(size_t)y].cost; });
     std::vector<int64_t> blk(2 * (size_t)nb), wbb(wb ? 2 * (size_t)nb : 0);
-    std::vector<int32_t> bdesc(4 * (size_t)nb), rblock((size_t)nb);
+    std::vector<int32_t> bdesc(4 * (size_t)nb);
     int64_t slots = 0;
     for (int64_t b = 0; b < nb; ++b) {
         const Blk& x = bl[(size_t)order[(size_t)b]];
@@ -2270,22 +2447,16 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
         bdesc[4 * (size_t)b + 1] = x.u1;
         bdesc[4 * (size_t)b + 2] = x.j;
         bdesc[4 * (size_t)b + 3] = 0;
-        rblock[(size_t)(tfirst[(size_t)x.j] + x.r)] = (int32_t)b;
         if (wb) {
             wbb[2 * (size_t)b] = (*wb)[2 * (size_t)x.r];
             wbb[2 * (size_t)b + 1] = (*wb)[2 * (size_t)x.r + 1];
         }
     }
-    std::vector<int32_t> dir(tfirst);
-    dir.insert(dir.end(), rstart.begin(), rstart.end());
-    dir.insert(dir.end(), rblock.begin(), rblock.end());
     const int64_t tk_len = slots + kStep + 256 * 4;  // slack: the kernel's ring reads ahead
     if ((s = ensure((void**)&P.toff, &P.toff_cap, sizeof(int32_t) * (size_t)cells)) != GILA_OK)
         return s;
     if ((s = ensure((void**)&P.blk, &P.blk_cap, sizeof(int64_t) * blk.size())) != GILA_OK) return s;
     if ((s = ensure((void**)&P.bdesc, &P.bdesc_cap, sizeof(int32_t) * bdesc.size())) != GILA_OK)
-        return s;
-    if ((s = ensure((void**)&P.rdir, &P.rdir_cap, sizeof(int32_t) * dir.size())) != GILA_OK)
         return s;
     if ((s = ensure((void**)&P.tk, &P.tk_cap, sizeof(uint16_t) * (size_t)tk_len)) != GILA_OK)
         return s;
@@ -2300,8 +2471,6 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
     GILA_CUDA(cudaMemcpyAsync(P.blk, blk.data(), sizeof(int64_t) * blk.size(),
                               cudaMemcpyHostToDevice, g->stream));
     GILA_CUDA(cudaMemcpyAsync(P.bdesc, bdesc.data(), sizeof(int32_t) * bdesc.size(),
-                              cudaMemcpyHostToDevice, g->stream));
-    GILA_CUDA(cudaMemcpyAsync(P.rdir, dir.data(), sizeof(int32_t) * dir.size(),
                               cudaMemcpyHostToDevice, g->stream));
     // every block's slots set to its padding id, then the ids ordered for
     // conflict-free gathers, or in ascending order; the slack after the
@@ -2318,24 +2487,24 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
         count_launch();
         GILA_CUDA(cudaGetLastError());
     }
-    const int32_t* d_tfirst = P.rdir;
-    const int32_t* d_rstart = P.rdir + nt + 1;
-    const int32_t* d_rblock = P.rdir + nt + 1 + nb + nt;
-    const unsigned lay_blocks = (unsigned)((cells + kSpreadWarps - 1) / kSpreadWarps);
-    if (g->tune.bank_spread >= 0 && esz == 8)
-        block_layout_kernel<16, true><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
-            d_rblock, P.tk);
-    else if (g->tune.bank_spread >= 0)
-        block_layout_kernel<8, true><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
-            d_rblock, P.tk);
-    else
-        block_layout_kernel<16, false><<<lay_blocks, kSpreadWarps * 32, 0, g->stream>>>(
-            n, g->krow, g->kcol, (int)nt, (int)tv, wdev, P.len, P.toff, P.blk, d_tfirst, d_rstart,
-            d_rblock, P.tk);
-    count_launch();
-    GILA_CUDA(cudaGetLastError());
+    // CTAs per block, for about 48 per SM
+    constexpr int64_t kParts = 48;
+    const unsigned parts = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>(64, ((int64_t)sm_count(g->device) * kParts + nb - 1) / std::max<int64_t>(nb, 1)));
+    auto layout = [&](auto kernel) -> cudaError_t {
+        const size_t smem = sizeof(SpreadSmem) * kSpreadWarps;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<dim3((unsigned)nb, parts), kSpreadWarps * 32, smem, g->stream>>>(
+            n, g->krow, g->kcol, (int)tv, wdev, P.len, P.len + cells, P.toff, P.blk,
+            reinterpret_cast<const int4*>(P.bdesc), P.tk);
+        count_launch();
+        return cudaGetLastError();
+    };
+    if (nb > 0)
+        GILA_CUDA(g->tune.bank_spread < 0 ? layout(block_layout_kernel<16, false>)
+                  : esz == 8              ? layout(block_layout_kernel<16, true>)
+                                          : layout(block_layout_kernel<8, true>));
     if (!wb) {
         // hubs of the adjacency for the combine kernel (synchronises)
         if ((s = plan_hubs(g, P)) != GILA_OK) return s;
@@ -2387,9 +2556,10 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
             gila_status s = plan_window(g, esz, P, &fits, len, rs, wb, &wmax, &rmax);
             if (s != GILA_OK || P.rows) return s;
             if (fits) {
-                if ((s = ensure((void**)&P.len, &P.len_cap, sizeof(int32_t) * (size_t)n)) != GILA_OK)
+                if ((s = ensure((void**)&P.len, &P.len_cap, 2 * sizeof(int32_t) * (size_t)n)) != GILA_OK)
                     return s;
-                rowlen_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, P.len);
+                rowlen_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, P.len,
+                                                                                P.len + n);
                 count_launch();
                 if ((s = prefix_cells(g, P, n)) != GILA_OK) return s;
                 if ((s = build_layout(g, esz, P, 1, 0, {rs}, &wb)) != GILA_OK) return s;
@@ -2421,10 +2591,10 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
         geometry(rmax);
     }
     const int64_t cells = n * nt;
-    gila_status s = ensure((void**)&P.len, &P.len_cap, sizeof(int32_t) * (size_t)cells);
+    gila_status s = ensure((void**)&P.len, &P.len_cap, 2 * sizeof(int32_t) * (size_t)cells);
     if (s != GILA_OK) return s;
-    seglen_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, g->stream>>>(n, g->krow, g->kcol,
-                                                                        (int)nt, (int)tv, P.len);
+    seglen_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, g->stream>>>(
+        n, g->krow, g->kcol, (int)nt, (int)tv, P.len, P.len + cells);
     count_launch();
     GILA_CUDA(cudaGetLastError());
     // each tile's row ranges: blocks of about equal cost (padded entries +
@@ -2601,6 +2771,7 @@ gila_status blocked_khop_metric(gila_graph* g, const gila_params* prm, const voi
     MetricArgs M;
     M.krow = g->krow;
     M.len = P.window ? nullptr : P.len;
+    M.start = P.window ? nullptr : P.len + g->n * P.nt;
     M.kcol = g->kcol;
     M.bdesc = reinterpret_cast<const int4*>(P.bdesc);
     M.wbase = P.window ? P.wtile : nullptr;

@@ -100,8 +100,6 @@ struct TilePlan {
     int32_t rmax = 0;                // most rows of a range (window mode: cells per CTA)
     int32_t* bdesc = nullptr;        // 4 nb: first row, end row and tile of block b, 0
     size_t bdesc_cap = 0;
-    int32_t* rdir = nullptr;         // per tile its row ranges and their blocks (layout scratch)
-    size_t rdir_cap = 0;
     int64_t* blk = nullptr;          // 2 nb: start in tk and entry count of block b
     size_t blk_cap = 0;
     int32_t* toff = nullptr;         // nt n: start of (tile j, row u) within its block
@@ -113,7 +111,8 @@ struct TilePlan {
     int32_t* hubs = nullptr;         // vertices of adjacency degree > 64 (combine kernel)
     size_t hubs_cap = 0;
     int32_t nhub = 0;
-    int32_t* len = nullptr;          // nt n segment lengths (plan scratch, quality figures)
+    int32_t* len = nullptr;          // nt n segment lengths, then their starts within the rows
+                                     // (plan scratch, quality figures)
     size_t len_cap = 0;
     int64_t* pre = nullptr;          // plan scratch: 2 (nt n + 1) prefix sums of the segments'
     size_t pre_cap = 0;              // padded lengths, then of their costs
