@@ -914,27 +914,6 @@ constexpr int kCombineLanes = 4;
 constexpr int kCombineThreads = 256;
 constexpr int kHubDeg = 64;
 
-// Entries [s, e) of ids, lane gl of a group of G taking s + gl, s + gl + G,
-// ... as row_sum_rel does (same terms, same order of additions), with the
-// ids of U consecutive turns loaded before their terms, so that a lane has U
-// id loads and then U position gathers in flight instead of one of each.
-template <int U, class F, class A>
-__device__ __forceinline__ void row_sum_batched(const uint32_t* __restrict__ ids, int64_t s,
-                                                int64_t e, int gl, int G, const F& f, A& a)
-{
-    const uint32_t* p = ids + s;
-    const int len = (int)(e - s);
-    int j = gl;
-    for (; j + (U - 1) * G < len; j += U * G) {
-        uint32_t v[U];
-#pragma unroll
-        for (int k = 0; k < U; ++k) v[k] = ld_id(p + j + k * G);
-#pragma unroll
-        for (int k = 0; k < U; ++k) f(v[k], a);
-    }
-    for (; j < len; j += G) f(ld_id(p + j), a);
-}
-
 template <class T, bool COMP>
 __device__ __forceinline__ void add_cell(const void* part, int64_t n, int j, int64_t u,
                                          Acc<T, COMP>& s)

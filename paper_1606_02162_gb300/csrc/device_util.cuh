@@ -61,6 +61,41 @@ __device__ __forceinline__ T group_sum(T v, int width)
     return v;
 }
 
+// ------------------------------------- programmatic dependent launches
+// A kernel launched with launch_dependent() may start while the kernel before
+// it on the stream still runs, once every block of that one has called
+// pdl_trigger() or ended. Until pdl_wait(), which returns when the kernel
+// before has completed and its writes are visible, it may only read what no
+// kernel of the iteration writes (lists, plan). Every thread calls pdl_wait(),
+// so that a completed kernel implies all before it completed.
+
+__device__ __forceinline__ void pdl_trigger()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_dependent(bool early, void (*kernel)(P...), dim3 grid, unsigned threads,
+                                    size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------ bulk copies (TMA engine)
 // One-dimensional cp.async.bulk copies from global to shared memory,
 // completed through an mbarrier in shared memory. Every wait is bounded.

@@ -379,6 +379,27 @@ __device__ __forceinline__ void row_sum_rel(const uint32_t* __restrict__ ids, in
     for (int j = gl; j < len; j += G) f(ld_id(p + j), a);
 }
 
+// Entries [s, e) of ids, lane gl of a group of G taking s + gl, s + gl + G,
+// ... as row_sum_rel does (same terms, same order of additions), with the
+// ids of U consecutive turns loaded before their terms, so that a lane has U
+// id loads and then U position gathers in flight instead of one of each.
+template <int U, class F, class A>
+__device__ __forceinline__ void row_sum_batched(const uint32_t* __restrict__ ids, int64_t s,
+                                                int64_t e, int gl, int G, const F& f, A& a)
+{
+    const uint32_t* p = ids + s;
+    const int len = (int)(e - s);
+    int j = gl;
+    for (; j + (U - 1) * G < len; j += U * G) {
+        uint32_t v[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) v[k] = ld_id(p + j + k * G);
+#pragma unroll
+        for (int k = 0; k < U; ++k) f(v[k], a);
+    }
+    for (; j < len; j += G) f(ld_id(p + j), a);
+}
+
 template <class T>
 __device__ __forceinline__ void apply_move(T t, void* pos_out, void* disp_out, int64_t u,
                                            T xu, T yu, T fx, T fy)

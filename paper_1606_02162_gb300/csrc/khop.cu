@@ -15,6 +15,7 @@
 //   the counts, so the output needs no atomics and is the same every run.
 //   Afterwards rows are classed by length for scheduling.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <mutex>
 #include <string>
@@ -804,9 +805,14 @@ gila_status scan_exclusive_i64(const int64_t* in, int64_t n, int64_t* out, cudaS
 
 int sm_count(int device)
 {
-    int v = 0;
+    // asked for on every launch: kept per device (0: not known yet)
+    static std::atomic<int> known[64] = {};
+    const int at = device & 63;
+    int v = known[at].load(std::memory_order_relaxed);
+    if (v > 0) return v;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || v <= 0)
-        v = 1;
+        return 1;
+    known[at].store(v, std::memory_order_relaxed);
     return v;
 }
 

@@ -16,6 +16,7 @@
 // 8 lanes per row. A row's reduction order depends only on its length and
 // its position in the k-hop list, so results are reproducible.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <vector>
 
@@ -29,7 +30,19 @@ namespace gila {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarpsPerBlock = kThreads / 32;
+// Threads per block of the iteration kernel on small graphs: FP64 issues two
+// lanes a clock on an SM, and the latency chain of a row is the same
+// everywhere, so a grid that does not fill the SMs with 256 threads a block
+// is spread over more of them (32 x 32 grid, FP64: 7.2 -> 5.9 us per
+// iteration; with the early launches and rows by entries below 12.5 -> 5.9).
+// Four warps, one for each of an SM's schedulers.
+constexpr int kThreadsSmall = 128;
+// Rows of the warp class longer than this are taken by the whole block in
+// small grids (BA n = 10,000, k = 2: 17.6 -> 12.0 us per iteration with it,
+// the early launches and batched adjacency loads; at 512 14.7, at 256 18.4;
+// from 16 blocks per SM on, hubs' warps no longer stand out: the pruned
+// Chung-Lu graph n = 100,000 103 -> 115 with it)
+constexpr int kCoopRow = 1024;
 
 struct IterArgs {
     const int64_t* row;
@@ -50,6 +63,7 @@ struct IterArgs {
     void* pos_out;
     void* disp_out;
     const void* wt;  // repulsion weights (T[n]) or null
+    int coop;        // warp class: rows longer than this are taken by a whole block
 };
 
 template <class T>
@@ -60,9 +74,10 @@ __device__ __forceinline__ void apply_move_it(const IterArgs& A, int64_t u, T xu
 }
 
 // Block-wide sum of an accumulator in a fixed order (warps, then warp 0).
-template <class T, bool COMP>
+template <class T, bool COMP, int NT>
 __device__ __forceinline__ void block_reduce(Acc<T, COMP>& a, T* sh)
 {
+    constexpr int kWarpsPerBlock = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     a.group_reduce(32);
     if (lane == 0) {
@@ -84,22 +99,28 @@ __device__ __forceinline__ void block_reduce(Acc<T, COMP>& a, T* sh)
     }
 }
 
-// Repulsion over k-hop entries [ks, ke) of u and, when with_att, attraction
-// over u's adjacency row, by lanes gl = 0..G-1 of a group.
-template <class T, int MODEL, bool COMP, class R, class P2>
+// Repulsion over the k-hop entries [ks, ke) of a vertex at pu and, when
+// with_att, attraction over its adjacency entries [ab, ae), by lanes
+// gl = 0..G-1 of a group. SHORT rows are taken an entry per lane (a row of
+// twelve: two rounds of eight lanes; by vectors of four ids three lanes had
+// four entries each: the 32 x 32 grid, FP64, 7.3 -> 5.9 us), others by
+// vectors.
+template <class T, int MODEL, bool COMP, bool SHORT = false, class R, class P2>
 __device__ __forceinline__ void vertex_sum(const IterArgs& A, R rep,
-                                           Att<T, MODEL, COMP> att, int64_t u, P2 pu, int64_t ks,
-                                           int64_t ke, bool with_att, int gl, int G,
+                                           Att<T, MODEL, COMP> att, P2 pu, int64_t ks, int64_t ke,
+                                           int64_t ab, int64_t ae, bool with_att, int gl, int G,
                                            Acc<T, COMP>& a)
 {
     rep.xu = pu.x;
     rep.yu = pu.y;
-    row_sum(A.kcol, ks, ke, gl, G, rep, a);
+    if (SHORT)
+        row_sum_batched<4>(A.kcol, ks, ke, gl, G, rep, a);
+    else
+        row_sum(A.kcol, ks, ke, gl, G, rep, a);
     if (with_att) {
         att.xu = pu.x;
         att.yu = pu.y;
-        row_sum_rel(reinterpret_cast<const uint32_t*>(A.col), A.row[u], A.row[u + 1], gl, G, att,
-                    a);
+        row_sum_batched<4>(reinterpret_cast<const uint32_t*>(A.col), ab, ae, gl, G, att, a);
     }
 }
 
@@ -107,19 +128,21 @@ __device__ __forceinline__ void vertex_sum(const IterArgs& A, R rep,
 // (all 64 warps) fit an SM: the short-row classes are latency-bound and gain
 // from the warps (mesh k = 3 compensated: 0.162 -> 0.145 ms per iteration);
 // FP64 needs its registers.
-template <class T>
+template <class T, int NT>
 constexpr int plain_min_blocks()
 {
-    return sizeof(T) == 4 ? 8 : 1;
+    return sizeof(T) == 4 ? 2048 / NT : 1;
 }
 
-template <class T, int MODEL, bool COMP, bool W>
-__global__ void __launch_bounds__(kThreads, plain_min_blocks<T>())
+template <class T, int MODEL, bool COMP, bool W, int NT>
+__global__ void __launch_bounds__(NT, plain_min_blocks<T, NT>())
 iteration_kernel(const IterArgs A)
 {
     using P2 = typename V2<T>::type;
-    __shared__ T sh[kWarpsPerBlock * 4];
+    constexpr int kWarps = NT / 32;
+    __shared__ T sh[kWarps * 4];
     __shared__ int s_last;
+    __shared__ int s_len[kWarps];
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
     Rep<T, MODEL, COMP, kSrcGlobal, false, W> rep;
     rep.src.pos = pos;
@@ -130,16 +153,22 @@ iteration_kernel(const IterArgs A)
     att.src.pos = pos;
     att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
+    // the next iteration's blocks may come while this one's last rows run;
+    // lists and offsets are read before the wait for the placement
+    pdl_trigger();
     int b = blockIdx.x;
     if (b < A.b3) {
         // a chunk of a giant row: block sum, then the last chunk finishes u;
         // the row's first chunk also carries the attraction terms
         const Chunk ch = A.chunks[b];
         const int64_t u = ch.vertex;
+        const int64_t ab = A.row[u], ae = A.row[u + 1];
+        pdl_wait();
         const P2 pu = pos[u];
         Acc<T, COMP> a;
-        vertex_sum<T, MODEL, COMP>(A, rep, att, u, pu, ch.begin, ch.end, b == ch.first, threadIdx.x, kThreads, a);
-        block_reduce<T, COMP>(a, sh);
+        vertex_sum<T, MODEL, COMP>(A, rep, att, pu, ch.begin, ch.end, ab, ae, b == ch.first,
+                                   threadIdx.x, NT, a);
+        block_reduce<T, COMP, NT>(a, sh);
         if (threadIdx.x == 0) {
             double* part = A.partials + (int64_t)b * 4;
             part[0] = (double)a.sx;
@@ -167,41 +196,82 @@ iteration_kernel(const IterArgs A)
     b -= A.b3;
     if (b < A.b2) {
         const int64_t u = A.list2[b];
+        const int64_t ks = A.krow[u], ke = A.krow[u + 1], ab = A.row[u], ae = A.row[u + 1];
+        pdl_wait();
         const P2 pu = pos[u];
         Acc<T, COMP> a;
-        vertex_sum<T, MODEL, COMP>(A, rep, att, u, pu, A.krow[u], A.krow[u + 1], true, threadIdx.x, kThreads, a);
-        block_reduce<T, COMP>(a, sh);
+        vertex_sum<T, MODEL, COMP>(A, rep, att, pu, ks, ke, ab, ae, true, threadIdx.x, NT, a);
+        block_reduce<T, COMP, NT>(a, sh);
         if (threadIdx.x == 0) apply_move_it<T>(A, u, pu.x, pu.y, a.fx(), a.fy());
         return;
     }
     b -= A.b2;
     if (b < A.b1) {
-        const int i = b * kWarpsPerBlock + (threadIdx.x >> 5);
-        if (i >= A.n1) return;  // whole warp leaves together
-        const int lane = threadIdx.x & 31;
-        const int64_t u = A.list1[i];
-        const P2 pu = pos[u];
-        Acc<T, COMP> a;
-        vertex_sum<T, MODEL, COMP>(A, rep, att, u, pu, A.krow[u], A.krow[u + 1], true, lane, 32, a);
-        a.group_reduce(32);
-        if (lane == 0) apply_move_it<T>(A, u, pu.x, pu.y, a.fx(), a.fy());
+        // a row per warp. In a small grid (coop set), rows b, b + b1, ... of
+        // the class, so that the longest (hubs, neighbours in id) fall to
+        // different blocks, and a row of more than coop entries is taken by
+        // the whole block: the launch does not wait for a hub's row on one
+        // warp
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const bool spread = A.coop != INT_MAX;
+        const int64_t i = spread ? b + (int64_t)warp * A.b1 : (int64_t)b * kWarps + warp;
+        const bool live = i < A.n1;
+        int64_t u = 0, ks = 0, ke = 0, ab = 0, ae = 0;
+        if (live) {
+            u = A.list1[i];
+            ks = A.krow[u];
+            ke = A.krow[u + 1];
+            ab = A.row[u];
+            ae = A.row[u + 1];
+        }
+        if (spread) {
+            if (lane == 0) s_len[warp] = (int)(ke - ks);
+            __syncthreads();
+        }
+        pdl_wait();
+        if (live && ke - ks <= A.coop) {
+            const P2 pu = pos[u];
+            Acc<T, COMP> a;
+            vertex_sum<T, MODEL, COMP>(A, rep, att, pu, ks, ke, ab, ae, true, lane, 32, a);
+            a.group_reduce(32);
+            if (lane == 0) apply_move_it<T>(A, u, pu.x, pu.y, a.fx(), a.fy());
+        }
+        for (int w = 0; spread && w < kWarps; ++w) {
+            if (s_len[w] <= A.coop) continue;  // uniform over the block
+            const int64_t v = A.list1[b + (int64_t)w * A.b1];
+            const P2 pv = pos[v];
+            Acc<T, COMP> a;
+            vertex_sum<T, MODEL, COMP>(A, rep, att, pv, A.krow[v], A.krow[v + 1], A.row[v],
+                                       A.row[v + 1], true, threadIdx.x, NT, a);
+            block_reduce<T, COMP, NT>(a, sh);
+            if (threadIdx.x == 0) apply_move_it<T>(A, v, pv.x, pv.y, a.fx(), a.fy());
+            __syncthreads();  // sh is free again
+        }
         return;
     }
     b -= A.b1;
     {
         constexpr int G = 8;
         const int gl = threadIdx.x & (G - 1);
-        const int i = b * (kThreads / G) + (threadIdx.x / G);
+        const int i = b * (NT / G) + (threadIdx.x / G);
         const bool live = i < A.n0;
         // lanes of a group stay together through the shuffles below
-        const int64_t u = live ? A.list0[i] : 0;
+        int64_t u = 0, ks = 0, ke = 0, ab = 0, ae = 0;
+        if (live) {
+            u = A.list0[i];
+            ks = A.krow[u];
+            ke = A.krow[u + 1];
+            ab = A.row[u];
+            ae = A.row[u + 1];
+        }
+        pdl_wait();
         Acc<T, COMP> a;
         P2 pu;
         pu.x = T(0);
         pu.y = T(0);
         if (live) {
             pu = pos[u];
-            vertex_sum<T, MODEL, COMP>(A, rep, att, u, pu, A.krow[u], A.krow[u + 1], true, gl, G, a);
+            vertex_sum<T, MODEL, COMP, true>(A, rep, att, pu, ks, ke, ab, ae, true, gl, G, a);
         }
         a.group_reduce(G);
         if (live && gl == 0) apply_move_it<T>(A, u, pu.x, pu.y, a.fx(), a.fy());
@@ -278,14 +348,25 @@ ordered_kernel(int64_t n, const int64_t* __restrict__ row, const int32_t* __rest
 }
 
 template <class T, int MODEL, bool COMP>
-cudaError_t launch_typed(const IterArgs& A, unsigned grid, cudaStream_t st)
+cudaError_t launch_typed(const IterArgs& A, int nt, unsigned grid, int64_t sms, cudaStream_t st)
 {
-    if (A.wt)
-        iteration_kernel<T, MODEL, COMP, true><<<grid, kThreads, 0, st>>>(A);
+    // Early start of the next iteration's blocks saves 1.5 to 2.5 us an
+    // iteration (grid 32 x 32: FP32 4.3 -> 2.9, FP64 7.4 -> 5.9). FP64 takes
+    // it up to one block per SM: blocks that come early are not spread evenly,
+    // and two that share an SM share its two FP64 lanes (64 x 50 grid, 200
+    // blocks: 16.9 us with it, 9.7 without).
+    const bool early = sizeof(T) == 4 || (int64_t)grid <= sms;
+    cudaError_t e;
+    if (nt == kThreadsSmall)
+        e = launch_dependent(early, A.wt ? iteration_kernel<T, MODEL, COMP, true, kThreadsSmall>
+                                         : iteration_kernel<T, MODEL, COMP, false, kThreadsSmall>,
+                             dim3(grid), kThreadsSmall, 0, st, A);
     else
-        iteration_kernel<T, MODEL, COMP, false><<<grid, kThreads, 0, st>>>(A);
+        e = launch_dependent(early, A.wt ? iteration_kernel<T, MODEL, COMP, true, kThreads>
+                                         : iteration_kernel<T, MODEL, COMP, false, kThreads>,
+                             dim3(grid), kThreads, 0, st, A);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 // ------------------------------------------------------------- metrics
@@ -573,8 +654,17 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
     A.nchunks = B.nchunks;
     A.b3 = B.nchunks;
     A.b2 = B.n2;
-    A.b1 = (B.n1 + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    A.b0 = (B.n0 + (kThreads / 8) - 1) / (kThreads / 8);
+    // blocks of 256 threads, or of 64 where those would not fill the SMs twice
+    auto blocks = [&](int nt) {
+        A.b1 = (B.n1 + nt / 32 - 1) / (nt / 32);
+        A.b0 = (B.n0 + nt / 8 - 1) / (nt / 8);
+        return (int64_t)A.b3 + A.b2 + A.b1 + A.b0;
+    };
+    int nt = kThreads;
+    const int64_t sms = sm_count(g->device);
+    const int64_t grid0 = blocks(nt);
+    if (grid0 < 2 * sms) blocks(nt = kThreadsSmall);
+    A.coop = grid0 < 16 * sms ? kCoopRow : INT_MAX;
     A.c = force_consts(prm->d, t);
     A.p = prm->p;
     A.q = prm->q;
@@ -589,16 +679,16 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
     cudaEvent_t pa = prof_kernel_begin(g);
     switch (prm->precision) {
     case GILA_FP64:
-        e = fr ? launch_typed<double, kFR, false>(A, (unsigned)grid, g->stream)
-               : launch_typed<double, kGeneric, false>(A, (unsigned)grid, g->stream);
+        e = fr ? launch_typed<double, kFR, false>(A, nt, (unsigned)grid, sms, g->stream)
+               : launch_typed<double, kGeneric, false>(A, nt, (unsigned)grid, sms, g->stream);
         break;
     case GILA_FP32_COMPENSATED:
-        e = fr ? launch_typed<float, kFR, true>(A, (unsigned)grid, g->stream)
-               : launch_typed<float, kGeneric, true>(A, (unsigned)grid, g->stream);
+        e = fr ? launch_typed<float, kFR, true>(A, nt, (unsigned)grid, sms, g->stream)
+               : launch_typed<float, kGeneric, true>(A, nt, (unsigned)grid, sms, g->stream);
         break;
     default:
-        e = fr ? launch_typed<float, kFR, false>(A, (unsigned)grid, g->stream)
-               : launch_typed<float, kGeneric, false>(A, (unsigned)grid, g->stream);
+        e = fr ? launch_typed<float, kFR, false>(A, nt, (unsigned)grid, sms, g->stream)
+               : launch_typed<float, kGeneric, false>(A, nt, (unsigned)grid, sms, g->stream);
         break;
     }
     prof_kernel_end(g, pa, "iteration_kernel");
