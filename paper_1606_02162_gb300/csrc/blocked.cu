@@ -193,11 +193,16 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
     auto cellp = [&](int64_t i) -> P2* {
         return WIN ? cells + 2 * i : cell_ptr<T, COMP>(A.part, A.n, j, u0 + i);
     };
+    // Early start: the descriptors above and the row directory below are read
+    // while the iteration before still runs; the placement, and the partials
+    // that the kernel before reads, wait for it.
+    pdl_trigger();
     if (threadIdx.x == 0) {
         // tile j by the bulk-copy engine (tv is even and the placement is
         // 16-byte aligned, so the source is too); an odd float2 tail by hand
         const uint32_t bytes = (uint32_t)(((size_t)tn * sizeof(P2)) & ~size_t(15));
         mbar_init(&tile_bar, 1);
+        pdl_wait();
         mbar_arrive_expect_tx(&tile_bar, bytes);
         const unsigned char* src = reinterpret_cast<const unsigned char*>(pos + tb);
         for (uint32_t o = 0; o < bytes && !A.skip_copy; o += kBulkChunk)
@@ -209,6 +214,8 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
         far.y = FarSlot<T>::v;
         tile[WIN ? tn : (int64_t)A.tv] = far;
     }
+    for (int i = threadIdx.x; i < nrows; i += kBThreads) D[i] = A.toff[(int64_t)j * A.n + u0 + i];
+    pdl_wait();
     if (WIN && threadIdx.x == 32) {
         // the finish's adjacency (row offsets, neighbour ids) and the rows'
         // own positions, pulled into L2 while the window loads and the
@@ -218,10 +225,8 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
         prefetch_l2_range(A.col + ab, sizeof(int32_t) * (size_t)(ae - ab));
         prefetch_l2_range(pos + u0, sizeof(P2) * (size_t)(u1 - u0));
     }
-    // meanwhile: the row directory (segment starts within the block) and
     // zero partials for rows with no entries in this tile
     for (int i = threadIdx.x; i < nrows; i += kBThreads) {
-        D[i] = A.toff[(int64_t)j * A.n + u0 + i];
         P2* c = cellp(i);
         P2 z;
         z.x = T(0);
@@ -718,6 +723,22 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
     const int64_t tb = A.wbase[2 * blockIdx.x], tn = A.wbase[2 * blockIdx.x + 1];
+    pdl_trigger();
+    // this warp's slices and the first steps of their stream, read while the
+    // iteration before still runs
+    const int4 bd = A.bdesc[blockIdx.x];
+    const int s0 = bd.x >> 5, ns = ((bd.y + 31) >> 5) - s0;
+    const int sa = s0 + ns * warp / kRowWarps, sb = s0 + ns * (warp + 1) / kRowWarps;
+    int4 sd = make_int4(0, 0, 0, 0);
+    uint2 next[kRowAhead];
+    const uint2* ids = reinterpret_cast<const uint2*>(A.tk) + lane;
+    if (sa < sb) {
+        sd = A.sdesc[sa];
+#pragma unroll
+        for (int i = 0; i < kRowAhead; ++i)
+            if (i < sd.y) next[i] = ld_ids2(ids + 32 * ((int64_t)sd.x + i));
+    }
+    pdl_wait();
     if (threadIdx.x == 0) {
         // the window by the bulk-copy engine (its first id is even: 16-byte
         // aligned); an odd float2 tail by hand; the far slot after it
@@ -733,19 +754,6 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
         far.x = FarSlot<T>::v;
         far.y = FarSlot<T>::v;
         tile[tn] = far;
-    }
-    // this warp's slices and the first steps of their stream
-    const int4 bd = A.bdesc[blockIdx.x];
-    const int s0 = bd.x >> 5, ns = ((bd.y + 31) >> 5) - s0;
-    const int sa = s0 + ns * warp / kRowWarps, sb = s0 + ns * (warp + 1) / kRowWarps;
-    int4 sd = make_int4(0, 0, 0, 0);
-    uint2 next[kRowAhead];
-    const uint2* ids = reinterpret_cast<const uint2*>(A.tk) + lane;
-    if (sa < sb) {
-        sd = A.sdesc[sa];
-#pragma unroll
-        for (int i = 0; i < kRowAhead; ++i)
-            if (i < sd.y) next[i] = ld_ids2(ids + 32 * ((int64_t)sd.x + i));
     }
     if (threadIdx.x == 0) {
         bool ok = mbar_wait(&tile_bar, 0, A.wait_ns);
@@ -953,18 +961,20 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
     att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
     Acc<T, COMP> rep, at;
+    pdl_trigger();
     if ((int)blockIdx.x < A.nhub) {
         // one hub per block
         __shared__ T sh[kCombineThreads / 32][8];
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const int64_t u = A.hubs[blockIdx.x];
+        const int64_t rb = A.row[u], re = A.row[u + 1];
         const P2 pu = pos[u];
         for (int jj = threadIdx.x; jj < A.nt; jj += kCombineThreads)
             add_cell<T, COMP>(A.part, A.n, jj, u, rep);
         att.xu = pu.x;
         att.yu = pu.y;
-        row_sum_batched<4>(reinterpret_cast<const uint32_t*>(A.col), A.row[u], A.row[u + 1],
-                           (int)threadIdx.x, kCombineThreads, att, at);
+        row_sum_batched<4>(reinterpret_cast<const uint32_t*>(A.col), rb, re, (int)threadIdx.x,
+                           kCombineThreads, att, at);
         rep.group_reduce(32);
         at.group_reduce(32);
         if (lane == 0) {
@@ -997,6 +1007,15 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
         re = A.row[u + 1];
         live = re - rb <= kHubDeg;  // hubs are done by their own blocks
     }
+    // the neighbours' ids of a lane's first two turns are on their way before
+    // the cells (BA n = 100,000, k = 2: 33.5 -> 31.8 us an iteration)
+    const uint32_t* col = reinterpret_cast<const uint32_t*>(A.col);
+    uint32_t ahead[2] = {0u, 0u};
+    const int deg = (int)(re - rb);
+    if (live) {
+        if (gl < deg) ahead[0] = ld_id(col + rb + gl);
+        if (gl + kCombineLanes < deg) ahead[1] = ld_id(col + rb + gl + kCombineLanes);
+    }
     P2 pu;
     pu.x = T(0);
     pu.y = T(0);
@@ -1006,8 +1025,10 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
         pu = pos[u];
         att.xu = pu.x;
         att.yu = pu.y;
-        row_sum_batched<2>(reinterpret_cast<const uint32_t*>(A.col), rb, re, gl, kCombineLanes, att,
-                           at);
+        if (gl < deg) att(ahead[0], at);
+        if (gl + kCombineLanes < deg) att(ahead[1], at);
+        if (deg > 2 * kCombineLanes)
+            row_sum_batched<2>(col, rb + 2 * kCombineLanes, re, gl, kCombineLanes, att, at);
     }
     rep.group_reduce(kCombineLanes);
     at.group_reduce(kCombineLanes);
@@ -1616,11 +1637,17 @@ cudaError_t launch_blocked_typed(gila_graph* g, const BlockedArgs& B, const Comb
         configured.fetch_or(bit);
     }
     cudaEvent_t pa = prof_kernel_begin(g);
-    blocked_kernel<T, MODEL, COMP, WIN><<<grid, kBThreads, smem, st>>>(B);
+    cudaError_t e = launch_dependent(true, blocked_kernel<T, MODEL, COMP, WIN>, dim3((unsigned)grid),
+                                     kBThreads, smem, st, B);
     count_launch();
-    cudaError_t e = cudaGetLastError();
     prof_kernel_end(g, pa, WIN ? "blocked_kernel (window)" : "blocked_kernel");
     if (e != cudaSuccess || WIN) return e;
+    // Launched after blocked_kernel has ended: blocks that came early and
+    // waited on SMs that were done cost more than they hid (BA n = 100,000,
+    // k = 2: 35.9 us an iteration against 29.2). blocked_kernel itself comes
+    // early, while the combine before it ends: 31.8 -> 29.2 us, k = 3 155.3
+    // -> 153.3, BA n = 333,334, k = 2 136.5 -> 134.7; rows_kernel on the mesh
+    // 1000 x 1000, k = 3: 36.7 -> 34.2.
     combine_kernel<T, MODEL, COMP><<<(unsigned)(C.nreg + C.nhub), kCombineThreads, 0, st>>>(C);
     count_launch();
     return cudaGetLastError();
@@ -1639,10 +1666,9 @@ cudaError_t launch_rows(gila_graph* g, const RowsArgs& R, const TilePlan& P)
         configured.fetch_or(bit);
     }
     cudaEvent_t pa = prof_kernel_begin(g);
-    rows_kernel<T, MODEL, COMP>
-        <<<P.nb, kRowThreads, ((size_t)P.tv + 1) * 2 * sizeof(T), g->stream>>>(R);
+    cudaError_t e = launch_dependent(true, rows_kernel<T, MODEL, COMP>, dim3((unsigned)P.nb),
+                                     kRowThreads, ((size_t)P.tv + 1) * 2 * sizeof(T), g->stream, R);
     count_launch();
-    cudaError_t e = cudaGetLastError();
     prof_kernel_end(g, pa, "blocked_kernel (window, row per lane)");
     return e;
 }
