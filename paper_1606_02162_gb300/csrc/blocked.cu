@@ -49,6 +49,7 @@ constexpr int kTileBudget = kSmemCap - (kMaxRows + 1) * 4 - 4096;
 constexpr int64_t kMaxTile = 65534;  // tile-relative ids and the far slot's id fit 16 bits
 constexpr uint32_t kBulkChunk = 32768;      // bytes per bulk copy instruction
 constexpr int64_t kBlockedMinNnz = 4000000;  // automatic mode: k-hop entries needed (tiles)
+constexpr int kWeightedMinSeg = 8;  // automatic mode with weights: mean entries of a segment
 constexpr uint64_t kWaitNs = 1000000000ull;  // bound on a tile wait (1 s, far above any copy)
 constexpr uint64_t kTestWaitNs = 1000000ull;   // the bound while the wait test hook is on
 // Every (tile j, row) segment is padded to a multiple of 8 entries with the
@@ -90,6 +91,7 @@ struct BlockedArgs {
     void* pos_out;
     void* disp_out;
     int uniform;               // FP32 steps taken warp-uniformly (tuning step_schedule >= 0)
+    const void* wt;            // weighted tiles: repulsion weights (T[n])
 };
 
 template <class T, bool COMP>
@@ -160,9 +162,21 @@ __device__ __forceinline__ void window_finish(const struct BlockedArgs& A,
 // finished by a whole warp (a few per range), the others by one thread.
 constexpr int kFinishDeg = 32;
 
-template <class T, int MODEL, bool COMP, bool WIN>
+// Bytes of a weighted tile before its weights: positions, far slot, row
+// directory, rounded up to 16 for the bulk copy of the weights.
+__host__ __device__ __forceinline__ size_t weights_at(int64_t tv, int64_t rmax, size_t esz)
+{
+    return ((size_t)(tv + 1) * esz + (size_t)(rmax + 1) * 4 + 15) & ~size_t(15);
+}
+
+// W (tile mode): the tile's repulsion weights beside its positions, one more
+// shared-memory read and product per entry. (The plain kernel gathers a
+// position and a weight per entry through L2, 62% busy: the pruned Chung-Lu
+// graph of 100,000 vertices, k = 2, 2.2e7 entries, 104 -> 44 us an iteration.)
+template <class T, int MODEL, bool COMP, bool WIN, bool W>
 __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs A)
 {
+    static_assert(!(WIN && W), "weights come with tiles");
     using P2 = typename V2<T>::type;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // shared memory: the tile (or the range's window) with one more slot for
@@ -203,11 +217,23 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
         const uint32_t bytes = (uint32_t)(((size_t)tn * sizeof(P2)) & ~size_t(15));
         mbar_init(&tile_bar, 1);
         pdl_wait();
-        mbar_arrive_expect_tx(&tile_bar, bytes);
+        // (a weighted tile starts at a multiple of four vertices)
+        const uint32_t wbytes = W ? (uint32_t)(((size_t)tn * sizeof(T)) & ~size_t(15)) : 0u;
+        mbar_arrive_expect_tx(&tile_bar, bytes + wbytes);
         const unsigned char* src = reinterpret_cast<const unsigned char*>(pos + tb);
         for (uint32_t o = 0; o < bytes && !A.skip_copy; o += kBulkChunk)
             bulk_g2s(smem_raw + o, src + o, (bytes - o < kBulkChunk) ? bytes - o : kBulkChunk,
                      &tile_bar);
+        if constexpr (W) {
+            const T* wsrc = reinterpret_cast<const T*>(A.wt) + tb;
+            unsigned char* wdst = smem_raw + weights_at(A.tv, A.rmax, sizeof(P2));
+            for (uint32_t o = 0; o < wbytes && !A.skip_copy; o += kBulkChunk)
+                bulk_g2s(wdst + o, reinterpret_cast<const unsigned char*>(wsrc) + o,
+                         (wbytes - o < kBulkChunk) ? wbytes - o : kBulkChunk, &tile_bar);
+            T* w = reinterpret_cast<T*>(wdst);
+            for (int64_t i = wbytes / sizeof(T); i < tn; ++i) w[i] = wsrc[i];
+            w[A.tv] = T(1);  // the padding's
+        }
         if ((size_t)tn * sizeof(P2) != bytes) tile[tn - 1] = pos[tb + tn - 1];
         P2 far;  // the padding's slot, outside the copied range
         far.x = FarSlot<T>::v;
@@ -252,8 +278,11 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
     mbar_wait(&tile_bar, 0, A.wait_ns);  // completed: acquires the tile for this thread
 
     if (L > 0) {
-        Rep<T, MODEL, COMP, kSrcShared, true> f;  // d^2 is applied when the partials are added
+        // d^2 is applied when the partials are added
+        Rep<T, MODEL, COMP, kSrcShared, true, W> f;
         f.src.set_shared(tile, 0u);  // ids are relative to the tile
+        if constexpr (W)
+            f.wt = reinterpret_cast<const T*>(smem_raw + weights_at(A.tv, A.rmax, sizeof(P2)));
         f.d2 = T(1);
         f.q = A.q;
         // this thread's entries [a, b) (a < L), their storage, and the row of a
@@ -1623,21 +1652,21 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
     }
 }
 
-template <class T, int MODEL, bool COMP, bool WIN>
+template <class T, int MODEL, bool COMP, bool WIN, bool W>
 cudaError_t launch_blocked_typed(gila_graph* g, const BlockedArgs& B, const CombineArgs& C,
                                  int grid, size_t smem, cudaStream_t st, int device)
 {
     static std::atomic<uint64_t> configured{0};  // one bit per device; callers may race
     const uint64_t bit = 1ull << (device & 63);
     if (!(configured.load() & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(blocked_kernel<T, MODEL, COMP, WIN>,
+        cudaError_t e = cudaFuncSetAttribute(blocked_kernel<T, MODEL, COMP, WIN, W>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kSmemCap - 4096);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
     cudaEvent_t pa = prof_kernel_begin(g);
-    cudaError_t e = launch_dependent(true, blocked_kernel<T, MODEL, COMP, WIN>, dim3((unsigned)grid),
+    cudaError_t e = launch_dependent(true, blocked_kernel<T, MODEL, COMP, WIN, W>, dim3((unsigned)grid),
                                      kBThreads, smem, st, B);
     count_launch();
     prof_kernel_end(g, pa, WIN ? "blocked_kernel (window)" : "blocked_kernel");
@@ -1677,8 +1706,10 @@ template <class T, int MODEL, bool COMP>
 cudaError_t launch_pair(gila_graph* g, const BlockedArgs& B, const CombineArgs& C, int grid,
                         size_t smem, cudaStream_t st, int device, bool win)
 {
-    return win ? launch_blocked_typed<T, MODEL, COMP, true>(g, B, C, grid, smem, st, device)
-               : launch_blocked_typed<T, MODEL, COMP, false>(g, B, C, grid, smem, st, device);
+    if constexpr (MODEL == kFR)
+        if (B.wt) return launch_blocked_typed<T, MODEL, COMP, false, true>(g, B, C, grid, smem, st, device);
+    return win ? launch_blocked_typed<T, MODEL, COMP, true, false>(g, B, C, grid, smem, st, device)
+               : launch_blocked_typed<T, MODEL, COMP, false, false>(g, B, C, grid, smem, st, device);
 }
 
 // The k-hop term of the quality reductions, sum over unordered k-hop pairs
@@ -2536,12 +2567,17 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
     // tiles for a row directory of rmax entries: positions per tile (one
     // slot for the padding's position) and the number of tiles
     int64_t tv = 0, nt = 0;
+    const bool weighted = g->wt64 != nullptr;
     auto geometry = [&](int64_t rmax) {
-        int64_t tv_max = (kSmemCap - (rmax + 1) * 4 - 4096) / (int64_t)esz - 1;
+        // with weights: half a position more per vertex, tiles of a multiple
+        // of four vertices (their first weight on a 16-byte boundary)
+        const int64_t step = weighted ? 4 : 2;
+        const int64_t bytes = (int64_t)esz + (weighted ? (int64_t)esz / 2 : 0);
+        int64_t tv_max = (kSmemCap - (rmax + 1) * 4 - 4096) / bytes - 1 - (weighted ? 2 : 0);
         if (g->tune.tile_vertices > 0) tv_max = std::min<int64_t>(tv_max, g->tune.tile_vertices);
-        tv_max = std::max<int64_t>(2, std::min<int64_t>(tv_max, kMaxTile) & ~int64_t(1));
+        tv_max = std::max<int64_t>(step, std::min<int64_t>(tv_max, kMaxTile) & ~(step - 1));
         nt = (n + tv_max - 1) / tv_max;
-        tv = std::min<int64_t>(tv_max, (((n + nt - 1) / nt) + 1) & ~int64_t(1));
+        tv = std::min<int64_t>(tv_max, ((n + nt - 1) / nt + step - 1) & ~(step - 1));
     };
     geometry(kMaxRows);
     const int min_seg = g->tune.min_segment;  // 0: no limit
@@ -2553,7 +2589,8 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
         // spreads small graphs over more SMs (32 x 32 grid, FP64: 0.017 ms
         // plain, 0.105 ms in one window; triangulated 200 x 200 mesh, k = 3:
         // 0.015 against 0.021)
-        if (g->tune.tile_vertices <= 0 && (g->tune.tiled > 0 || g->nnz_khop >= kBlockedMinNnz)) {
+        if (!weighted && g->tune.tile_vertices <= 0 &&
+            (g->tune.tiled > 0 || g->nnz_khop >= kBlockedMinNnz)) {
             bool fits = false;
             std::vector<int64_t> len, wb;
             std::vector<int32_t> rs;
@@ -2580,7 +2617,9 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
     // against 0.0609 plain; BA n = 333,334, k = 2, segments of 12: 0.183
     // against 0.209). FP64 follows the same rule (its tiles hold half as
     // many positions): on BA k = 3 blocked 5.14 ms vs plain 6.03 ms
-    const bool tiles_pay = !(g->tune.tiled < 0 && avg_seg < min_seg);
+    // (weighted graphs, whose windows are not tried, stay with the plain
+    // kernel where most segments would be nearly empty)
+    const bool tiles_pay = !(g->tune.tiled < 0 && avg_seg < std::max(min_seg, weighted ? kWeightedMinSeg : 0));
     if (!tiles_pay || (g->tune.tiled < 0 && g->nnz_khop < kBlockedMinNnz)) return GILA_OK;
     // many rows: where 4096-row ranges alone make more blocks than the CTA
     // target, a larger directory (smaller tiles) gives fewer blocks, each
@@ -2635,9 +2674,16 @@ bool blocked_auto_applies(int64_t n, int64_t nnz_khop, size_t esz, const gila_tu
            (double)nnz_khop / ((double)n * (double)nt) >= (double)tune.min_segment;
 }
 
+// Repulsion weights with exponents other than Fruchterman-Reingold's are
+// applied by the plain kernel only.
+static bool plain_weights(const gila_graph* g, const gila_params* prm)
+{
+    return g->wt64 && !(prm->p == 2 && prm->q == 1);
+}
+
 gila_status prepare_iteration(gila_graph* g, const gila_params* prm)
 {
-    if (prm->precision == GILA_FP64_ORDERED || g->n == 0 || g->wt64) return GILA_OK;
+    if (prm->precision == GILA_FP64_ORDERED || g->n == 0 || plain_weights(g, prm)) return GILA_OK;
     TilePlan& P = g->tplan[is_f64(prm->precision) ? 1 : 0];
     return P.ready ? GILA_OK : plan_tiles(g, is_f64(prm->precision) ? 16 : 8, P);
 }
@@ -2646,8 +2692,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
                            void* pos_out, void* disp_out, bool* handled)
 {
     *handled = false;
-    // repulsion weights are applied by the plain kernel only
-    if (prm->precision == GILA_FP64_ORDERED || g->n == 0 || g->wt64) return GILA_OK;
+    if (prm->precision == GILA_FP64_ORDERED || g->n == 0 || plain_weights(g, prm)) return GILA_OK;
     const size_t esz = is_f64(prm->precision) ? 16 : 8;
     TilePlan& P = g->tplan[esz == 16 ? 1 : 0];
     if (!P.ready) {
@@ -2716,6 +2761,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     // keeps both schedules: with the divergent one compiled beside it the
     // uniform schedule itself measured faster (4.88 vs 5.08 ms on Chung-Lu)
     B.uniform = g->tune.step_schedule >= 0 ? 1 : 0;
+    B.wt = !g->wt64 ? nullptr : esz == 16 ? (const void*)g->wt64 : (const void*)g->wt32;
     CombineArgs C;
     C.row = g->row;
     C.col = g->col;
@@ -2732,6 +2778,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     C.nreg = (int32_t)((g->n * kCombineLanes + kCombineThreads - 1) / kCombineThreads);
     const int grid = P.nb;
     const size_t smem = P.window ? window_smem(P.tv, P.rmax, esz)
+                        : B.wt   ? weights_at(P.tv, P.rmax, esz) + (size_t)(P.tv + 1) * (esz / 2)
                                  : (size_t)(P.tv + 1) * esz + (size_t)(P.rmax + 1) * 4;
     const bool fr = (prm->p == 2 && prm->q == 1);
     const bool w = P.window;

@@ -235,7 +235,8 @@ struct PosSource {
 // rcp(r^2) unscaled: one MUFU, no divide. A pair at distance 0 adds nothing. With
 // UNSCALED the factor d^2 is left out (the caller multiplies the row's sum
 // by it once). With WEIGHTED the term is multiplied by wt[v], the repulsion
-// weight of the repelling vertex (Section 4.6).
+// weight of the repelling vertex (Section 4.6); wt is in shared memory where
+// the positions are.
 template <class T, int MODEL, bool COMP, int SRC = kSrcGlobal, bool UNSCALED = false,
           bool WEIGHTED = false>
 struct Rep {
@@ -248,7 +249,7 @@ struct Rep {
     template <bool C = COMP>
     __device__ __forceinline__ void operator()(uint32_t v, Acc<T, C>& a) const
     {
-        if constexpr (sizeof(T) == 4 && MODEL == kFR && UNSCALED && !WEIGHTED && SRC == kSrcShared) {
+        if constexpr (sizeof(T) == 4 && MODEL == kFR && UNSCALED && SRC == kSrcShared) {
             // the blocked kernel's FP32 term with packed two-lane FP32
             // arithmetic (sm_100 and later): one subtraction forms
             // (dx, dy) and one fused multiply-add accumulates c (dx, dy)
@@ -259,7 +260,8 @@ struct Rep {
             asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
             float dx, dy;
             asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
-            const float c = rep_fr1(dx, dy);
+            float c = rep_fr1(dx, dy);
+            if (WEIGHTED) c *= wt[v];
             asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
             asm("mov.b64 %0, {%1, %2};" : "=l"(ac) : "f"(a.sx), "f"(a.sy));
             asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
@@ -281,7 +283,7 @@ struct Rep {
                 c = (UNSCALED ? T(1) : d2) / (ipow_(dl, q) * dl);
             }
         }
-        if (WEIGHTED) c *= __ldg(wt + v);
+        if (WEIGHTED) c *= SRC == kSrcShared ? wt[v] : __ldg(wt + v);
         a.add(c * dx, c * dy);
     }
 

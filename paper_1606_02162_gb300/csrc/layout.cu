@@ -797,6 +797,8 @@ __global__ void weights_to_f32_kernel(int64_t n, const double* __restrict__ w,
 
 gila_status set_repulsion_weights(gila_graph* g, const double* w, bool w_on_device)
 {
+    // plans differ with and without weights (the values are read each time)
+    if ((w != nullptr) != (g->wt64 != nullptr)) invalidate_tile_plans(g);
     if (!w) {
         cudaFree(g->wt64);
         cudaFree(g->wt32);

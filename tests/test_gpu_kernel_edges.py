@@ -173,3 +173,35 @@ def test_tile_plan_step(g, k, tune, prec):
         torch.cuda.synchronize()
         assert G.gila_profile_read_kernel(h.handle)["name"] == "blocked_kernel"
     assert np.abs(disp.double().cpu().numpy() - want).max() <= TOL[prec] * np.abs(want).max()
+
+
+# weighted tiles: one tile and many, a last tile of one to three vertices (the
+# weights' tail behind the bulk copy), zero weights; other exponents stay with
+# the plain kernel; weights set, cleared and set again on one graph
+@pytest.mark.parametrize("n,tv", [(1001, 4), (1002, 100), (1003, 1000), (4097, 512), (900, 900)])
+@pytest.mark.parametrize("prec", list(TOL), ids=["fp32", "fp32c", "fp64"])
+def test_weighted_tiles(n, tv, prec):
+    import torch
+    g = I.barabasi_albert(n, 2, 8)
+    pos = I.uniform_positions(g.n, 41).astype(np.float32).astype(np.float64)
+    w = 1.0 + np.random.default_rng(n).integers(0, 5, g.n)
+    w[::7] = 0.0
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 2)
+    dt = torch.float64 if prec == G.GILA_FP64 else torch.float32
+    x = torch.tensor(pos, dtype=dt, device="cuda")
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, tiled=1, tile_vertices=tv)
+        G.gila_profile_enable(h.handle, 2)
+        for wt, p, q, kernel in ((w, 2, 1, "blocked_kernel"), (w, 3, 2, "iteration_kernel"),
+                                 (None, 2, 1, "blocked_kernel"), (w[::-1], 2, 1, "blocked_kernel"),
+                                 (w, 2, 1, "blocked_kernel")):
+            G.gila_graph_set_repulsion_weights(h.handle, wt)
+            _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, 0.4, d=1.1, p=p, q=q,
+                             wt=None if wt is None else np.ascontiguousarray(wt))
+            y, disp = torch.empty_like(x), torch.empty_like(x)
+            G.gila_layout_step(h.handle, G.params(k=2, d=1.1, p=p, q=q, precision=prec), 0.4, x, y,
+                               disp)
+            torch.cuda.synchronize()
+            assert G.gila_profile_read_kernel(h.handle)["name"].startswith(kernel)
+            got = disp.double().cpu().numpy()
+            assert np.abs(got - want).max() <= TOL[prec] * np.abs(want).max()
