@@ -1283,8 +1283,8 @@ __global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t*
 // Copy every (tile, row) segment into its block's share storage as 16-bit
 // ids relative to the tile: entry p of the block, held by the share of
 // thread t (s = p - lane_start(L, t)), goes to slot
-// (t / 32) 32 lane_len(L) + 256 (s / 8) + 8 (t % 32) + s % 8. The slots that
-// no entry takes hold the padding id already (pad_fill_kernel).
+// (t / 32) 32 lane_len(L) + 256 (s / 8) + 8 (t % 32) + s % 8; the entries up
+// to the segment's padded length take the block's padding id.
 //
 // With SPREAD each segment's ids are also ordered for blocked_kernel's
 // shared-memory gathers. A warp's gather is served in groups of G lanes
@@ -1300,7 +1300,8 @@ __global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t*
 // over take the ids left over.
 //
 // Blocks come from the grid, so that a warp looks its block up once and then
-// takes rows of it. Three forms by length:
+// takes rows of it: one at a time, or two where most segments are short
+// (SHORTS; the storage then holds the padding already). Three forms by length:
 // - up to 32 entries (two rows of up to 16 at once): an id and an entry per
 //   lane, matched by (residue, rank) through a table in shared memory;
 // - longer: by chunks of at most kSpreadChunk entries; the ids grouped by
@@ -1313,7 +1314,7 @@ __global__ void hubs_kernel(int64_t n, const int64_t* __restrict__ row, int32_t*
 // took Chung-Lu n = 250,000, k = 3 from 4.27 to 4.18 ms per launch, 4096 gave
 // 4.15 ms at half the occupancy here.
 // The layout of Chung-Lu n = 60,000, k = 3 took 7.85 ms with a warp per
-// (tile, row), atomics and a matching step per 32 entries, 3.74 now; BA
+// (tile, row), atomics and a matching step per 32 entries, 3.27 now; BA
 // n = 333,334, k = 2 (segments of 12 entries) 3.78 -> 1.34 ms.
 constexpr int kSpreadWarps = 8;
 constexpr int kSpreadChunk = 2048;
@@ -1333,23 +1334,27 @@ struct SpreadSmem {
     int32_t ask[32], base[32];            // counts and places by residue
 };
 
-// Every slot of block b's share storage set to the block's padding id (its
-// far slot) before the layout kernel writes the entries: the slots past
-// each thread's share keep it, so that the FP32 kernel takes a thread's
-// last steps like any other (their terms are exact zeros). Block starts are
-// multiples of 8 slots: whole 16-byte stores.
-__global__ void pad_fill_kernel(uint16_t* __restrict__ tk, const int64_t* __restrict__ blk,
-                                const int64_t* __restrict__ wbase, int tv, int64_t nb)
+// The slots past each thread's share set to the block's padding id (its far
+// slot), so that the FP32 kernel takes a thread's last steps like any other
+// (their terms are exact zeros). Shares and block starts are multiples of 8
+// slots: whole 16-byte stores. The segments' own padding is written by the
+// layout kernel, or, with `all`, here with every other slot: on short
+// segments, a third of whose slots are padding, that is cheaper (BA
+// n = 333,334, k = 2: 27 us here against 190 there), on long ones it writes
+// the whole storage once more (Chung-Lu n = 60,000, k = 3: 278 us, 8 now).
+__global__ void __launch_bounds__(kBThreads)
+pad_shares_kernel(uint16_t* __restrict__ tk, const int64_t* __restrict__ blk,
+                  const int64_t* __restrict__ wbase, int tv, int all)
 {
-    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int64_t bsp = blk[2 * b];
-        const int64_t words = (int64_t)kBThreads * lane_len((int32_t)blk[2 * b + 1]) / 8;
-        const uint32_t pad = wbase ? (uint32_t)wbase[2 * b + 1] : (uint32_t)tv;
-        const uint32_t pp = pad | (pad << 16);
-        const uint4 v = make_uint4(pp, pp, pp, pp);
-        uint4* dst = reinterpret_cast<uint4*>(tk + bsp);
-        for (int64_t i = threadIdx.x; i < words; i += blockDim.x) dst[i] = v;
-    }
+    const int64_t b = blockIdx.x;
+    const int32_t L = (int32_t)blk[2 * b + 1], m8 = lane_len(L);
+    const int t = threadIdx.x;
+    const uint32_t pad = wbase ? (uint32_t)wbase[2 * b + 1] : (uint32_t)tv;
+    const uint32_t pp = pad | (pad << 16);
+    uint4* dst = reinterpret_cast<uint4*>(tk + blk[2 * b] + (int64_t)(t >> 5) * 32 * m8) + (t & 31);
+    const int32_t own = (lane_start(L, t + 1) - lane_start(L, t)) / kStep;
+    for (int32_t k = all ? 0 : own; k < m8 / kStep; ++k)
+        dst[32 * (int64_t)k] = make_uint4(pp, pp, pp, pp);
 }
 
 // The share (thread of blocked_kernel) that holds entry p of a block of L
@@ -1372,19 +1377,21 @@ __device__ __forceinline__ int64_t share_slot(int t, int32_t sidx, int32_t m8)
 
 // One entry and one id per lane (entry p of the block), of one row or, with
 // `second` telling their lanes apart, of two: dealt by residue within a row.
+// Lanes with `tail` set store the padding of their row's end.
 template <int G>
-__device__ __forceinline__ void deal_short(SpreadSmem& S, bool act, int32_t p, uint32_t id,
-                                           bool second, int32_t L, int32_t m8, float inv,
-                                           uint16_t* tk, int lane)
+__device__ __forceinline__ void deal_short(SpreadSmem& S, bool act, bool tail, int32_t p, uint32_t id,
+                                           uint16_t pad, bool second, int32_t L, int32_t m8,
+                                           float inv, uint16_t* tk, int lane)
 {
     const int key = second ? 16 : 0;
     int64_t at = 0;
     int want = 0;
-    if (act) {
+    if (act || tail) {
         const int t = share_of(L, p, inv);
         const int32_t sidx = p - lane_start(L, t);
         at = share_slot(t, sidx, m8);
         want = ((t + sidx) & (G - 1)) + key;
+        if (tail) tk[at] = pad;
     }
     const unsigned lt = lanemask_lt();
     const int has = (int)(id & (G - 1)) + key;
@@ -1416,7 +1423,7 @@ __device__ __forceinline__ void deal_short(SpreadSmem& S, bool act, int32_t p, u
     __syncwarp();  // the next rows reuse the tables
 }
 
-template <int G, bool SPREAD>
+template <int G, bool SPREAD, bool SHORTS>
 __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
     int64_t n, const int64_t* __restrict__ krow, const uint32_t* __restrict__ kcol, int tv,
     const int64_t* __restrict__ wbase, const int32_t* __restrict__ len,
@@ -1440,9 +1447,17 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
     const int32_t* cstart = start + (int64_t)j * n;
     const int32_t* coff = toff + (int64_t)j * n;
 
+    const uint16_t pad = wbase ? (uint16_t)wbase[2 * b + 1] : (uint16_t)tv;
+    auto put_pad = [&](int32_t p) {
+        const int t = share_of(L, p, inv);
+        tk[share_slot(t, p - lane_start(L, t), m8)] = pad;
+    };
+
     auto row = [&](int64_t u, int rl) {  // one row of rl entries by the whole warp
         const uint32_t* src = kcol + krow[u] + cstart[u];
         const int32_t S0 = coff[u];
+        const int padded = (int)seg_padded(rl);
+        if (!SHORTS && (!SPREAD || rl > 32) && rl + lane < padded) put_pad(S0 + rl + lane);
         if (!SPREAD) {
             for (int e = lane; e < rl; e += 32) {
                 const int t = share_of(L, S0 + e, inv);
@@ -1452,7 +1467,8 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
         }
         if (rl <= 32) {
             const uint32_t id = lane < rl ? src[lane] - tb : 0u;
-            deal_short<G>(S, lane < rl, S0 + lane, id, false, L, m8, inv, tk, lane);
+            deal_short<G>(S, lane < rl, !SHORTS && lane >= rl && lane < padded, S0 + lane, id, pad, false, L, m8,
+                          inv, tk, lane);
             return;
         }
         for (int32_t c0 = 0; c0 < rl; c0 += kSpreadChunk) {
@@ -1616,7 +1632,9 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
             __syncwarp();  // the next chunk reuses the buffers
         }
     };
-    // this CTA's part of the block's rows, taken in pairs by its warps
+    // this CTA's part of the block's rows, taken by its warps one at a time,
+    // or in pairs where most rows are short
+    constexpr int unit = SHORTS ? 2 : 1;
     __shared__ int s_next;
     if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
@@ -1625,27 +1643,24 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
     const int64_t u1 = bd.x + rows * (blockIdx.y + 1) / gridDim.y;
     for (;;) {
         int64_t u = 0;
-        if (lane == 0) u = u0 + 2 * (int64_t)atomicAdd(&s_next, 1);
+        if (lane == 0) u = u0 + unit * (int64_t)atomicAdd(&s_next, 1);
         u = __shfl_sync(kFull, u, 0);
         if (u >= u1) break;
-        const int l0 = clen[u], l1 = u + 1 < u1 ? clen[u + 1] : 0;
-        if (SPREAD && l0 <= 16 && l1 <= 16) {
+        const int l0 = clen[u], l1 = unit == 2 && u + 1 < u1 ? clen[u + 1] : 0;
+        if (SPREAD && SHORTS && l0 <= 16 && l1 <= 16) {
             if (l0 + l1 == 0) continue;
             const bool second = lane >= 16;
             const int64_t v = second ? u + 1 : u;
             const int e = lane & 15;
-            const bool act = e < (second ? l1 : l0);
-            int32_t p = 0;
-            uint32_t id = 0;
-            if (act) {
-                p = coff[v] + e;
-                id = kcol[krow[v] + cstart[v] + e] - tb;
-            }
-            deal_short<G>(S, act, p, id, second, L, m8, inv, tk, lane);
+            const int lv = second ? l1 : l0;
+            const bool act = e < lv;
+            const int32_t p = act ? coff[v] + e : 0;
+            const uint32_t id = act ? kcol[krow[v] + cstart[v] + e] - tb : 0u;
+            deal_short<G>(S, act, false, p, id, pad, second, L, m8, inv, tk, lane);
             continue;
         }
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < unit; ++h) {
             const int rl = h ? l1 : l0;
             if (rl) row(u + h, rl);
         }
@@ -2508,18 +2523,18 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
                               cudaMemcpyHostToDevice, g->stream));
     GILA_CUDA(cudaMemcpyAsync(P.bdesc, bdesc.data(), sizeof(int32_t) * bdesc.size(),
                               cudaMemcpyHostToDevice, g->stream));
-    // every block's slots set to its padding id, then the ids ordered for
-    // conflict-free gathers, or in ascending order; the slack after the
-    // last block (read ahead by the kernel's ring, never used) is zeroed
+    // the slots past each share set to the block's padding id, then the ids
+    // ordered for conflict-free gathers, or in ascending order; the slack
+    // after the last block (read ahead by the kernel's ring, never used) is zeroed
     const int64_t* wdev = wb ? P.wtile : nullptr;
+    const int shorts = g->nnz_khop < 32 * cells ? 1 : 0;  // most segments short
     GILA_CUDA(cudaMemsetAsync(P.tk + slots, 0, sizeof(uint16_t) * (size_t)(tk_len - slots),
                               g->stream));
     if (nb > 0) {
         toff_kernel<<<(unsigned)nb, 256, 0, g->stream>>>(n, reinterpret_cast<const int4*>(P.bdesc),
                                                          P.pre, P.toff);
         count_launch();
-        pad_fill_kernel<<<(unsigned)std::min<int64_t>(nb, 4096), 256, 0, g->stream>>>(
-            P.tk, P.blk, wdev, (int)tv, nb);
+        pad_shares_kernel<<<(unsigned)nb, kBThreads, 0, g->stream>>>(P.tk, P.blk, wdev, (int)tv, shorts);
         count_launch();
         GILA_CUDA(cudaGetLastError());
     }
@@ -2538,9 +2553,13 @@ gila_status build_layout(gila_graph* g, size_t esz, TilePlan& P, int64_t nt, int
         return cudaGetLastError();
     };
     if (nb > 0)
-        GILA_CUDA(g->tune.bank_spread < 0 ? layout(block_layout_kernel<16, false>)
-                  : esz == 8              ? layout(block_layout_kernel<16, true>)
-                                          : layout(block_layout_kernel<8, true>));
+        GILA_CUDA(g->tune.bank_spread < 0
+                      ? layout(shorts ? block_layout_kernel<16, false, true>
+                                      : block_layout_kernel<16, false, false>)
+                  : esz == 8 ? layout(shorts ? block_layout_kernel<16, true, true>
+                                             : block_layout_kernel<16, true, false>)
+                             : layout(shorts ? block_layout_kernel<8, true, true>
+                                             : block_layout_kernel<8, true, false>));
     if (!wb) {
         // hubs of the adjacency for the combine kernel (synchronises)
         if ((s = plan_hubs(g, P)) != GILA_OK) return s;

@@ -416,10 +416,12 @@ ball2_kernel(int64_t n, const int64_t* __restrict__ row, const int32_t* __restri
             const int32_t u = col[e];
             atomicOr(&B[u >> 5], 1u << (u & 31));
         }
-        for (int64_t e = vb; e < ve; ++e) {
+        // a warp per neighbour (the block on one neighbour after another was
+        // a chain of dependent loads: Chung-Lu n = 60,000 510 -> 181 us)
+        for (int64_t e = vb + (tid >> 5); e < ve; e += kT2Threads / 32) {
             const int32_t u = col[e];
             const int64_t ub = row[u], ue = row[u + 1];
-            for (int64_t f = ub + tid; f < ue; f += kT2Threads) {
+            for (int64_t f = ub + (tid & 31); f < ue; f += 32) {
                 const int32_t x = col[f];
                 atomicOr(&B[x >> 5], 1u << (x & 31));
             }
@@ -435,13 +437,18 @@ ball2_kernel(int64_t n, const int64_t* __restrict__ row, const int32_t* __restri
     }
 }
 
-constexpr int kOrRegs = 8;  // uint4 words of the ball each thread keeps per pass
-
+// R uint4 words of the ball per thread and pass, so that 256 threads cover
+// the bitmap in one where they can, and 8 / R neighbours' words read before
+// the first is OR-ed in: eight loads in flight whatever the bitmap's size
+// (with eight words and one neighbour at a time a bitmap of 469 uint4 had
+// two: Chung-Lu n = 60,000 1572 -> 814 us).
+template <int R>
 __global__ void __launch_bounds__(kT2Threads)
 ball3_or_kernel(const int32_t* __restrict__ queue, int nq, const int64_t* __restrict__ row,
                 const int32_t* __restrict__ col, int64_t nwords, const uint32_t* __restrict__ b2,
                 int64_t* __restrict__ counts, uint32_t* __restrict__ store)
 {
+    constexpr int U = 8 / R;
     __shared__ int64_t s_wt[kT2Threads / 32 + 1];
     const int tid = threadIdx.x;
     const int64_t n4 = nwords / 4;  // nwords is a multiple of 4
@@ -450,30 +457,39 @@ ball3_or_kernel(const int32_t* __restrict__ queue, int nq, const int64_t* __rest
         const int64_t sb = row[src], se = row[src + 1];
         int64_t cnt = 0;
         uint4* dst = reinterpret_cast<uint4*>(store + (int64_t)qi * nwords);
-        for (int64_t c0 = 0; c0 < n4; c0 += (int64_t)kT2Threads * kOrRegs) {
-            uint4 acc[kOrRegs];
+        for (int64_t c0 = 0; c0 < n4; c0 += (int64_t)kT2Threads * R) {
+            uint4 acc[R];
             const uint4* own = reinterpret_cast<const uint4*>(b2 + (int64_t)src * nwords);
 #pragma unroll
-            for (int r = 0; r < kOrRegs; ++r) {
+            for (int r = 0; r < R; ++r) {
                 const int64_t i = c0 + (int64_t)r * kT2Threads + tid;
                 acc[r] = i < n4 ? own[i] : make_uint4(0u, 0u, 0u, 0u);
             }
-            for (int64_t e = sb; e < se; ++e) {
-                const uint4* nb = reinterpret_cast<const uint4*>(b2 + (int64_t)col[e] * nwords);
+            for (int64_t e = sb; e < se; e += U) {
+                uint4 w[U][R];
 #pragma unroll
-                for (int r = 0; r < kOrRegs; ++r) {
-                    const int64_t i = c0 + (int64_t)r * kT2Threads + tid;
-                    if (i < n4) {
-                        const uint4 w = __ldg(nb + i);
-                        acc[r].x |= w.x;
-                        acc[r].y |= w.y;
-                        acc[r].z |= w.z;
-                        acc[r].w |= w.w;
+                for (int u = 0; u < U; ++u) {
+                    // past the last neighbour the last one again (OR is idempotent)
+                    const int64_t at = e + u < se ? e + u : se - 1;
+                    const uint4* nb = reinterpret_cast<const uint4*>(b2 + (int64_t)col[at] * nwords);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int64_t i = c0 + (int64_t)r * kT2Threads + tid;
+                        w[u][r] = i < n4 ? __ldg(nb + i) : make_uint4(0u, 0u, 0u, 0u);
                     }
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        acc[r].x |= w[u][r].x;
+                        acc[r].y |= w[u][r].y;
+                        acc[r].z |= w[u][r].z;
+                        acc[r].w |= w[u][r].w;
+                    }
             }
 #pragma unroll
-            for (int r = 0; r < kOrRegs; ++r) {
+            for (int r = 0; r < R; ++r) {
                 const int64_t i = c0 + (int64_t)r * kT2Threads + tid;
                 if (i < n4) {
                     dst[i] = acc[r];
@@ -490,41 +506,64 @@ ball3_or_kernel(const int32_t* __restrict__ queue, int nq, const int64_t* __rest
 }
 
 // Fill from the balls the count pass stored: each block writes the sorted
-// rows of its sources straight from their bitmaps (no second search). A
-// chunk of 256 words is expanded into shared memory at the offsets a block
-// scan of their popcounts gives, then copied out with coalesced stores.
-constexpr int kFillStage = kT2Threads * 32;  // ids a chunk of 256 words can hold
+// rows of its sources straight from their bitmaps (no second search). A warp
+// takes an eighth of the bitmap: it counts its bits, finds its place behind
+// the warps before it (the one barrier of a source, with the one that frees
+// the counts), then expands 64 words at a time into its own shared memory and
+// copies the ids out with coalesced stores. (256 words at a time by the whole
+// block, four barriers each: BA n = 333,334, k = 2, a ball's 10,420 words,
+// 1.60 -> 0.93 ms; Chung-Lu n = 60,000, k = 3 1.75 -> 1.35.)
+constexpr int kFillWords = 64;  // words of a warp's turn, two per lane
 
 __global__ void __launch_bounds__(kT2Threads)
 t2_fill_stored_kernel(const int32_t* __restrict__ queue, int nq, int64_t nwords,
                       const uint32_t* __restrict__ store, const int64_t* __restrict__ krow,
                       uint32_t* __restrict__ kcol)
 {
-    __shared__ int64_t s_wt[kT2Threads / 32 + 1];
-    __shared__ uint32_t s_ids[kFillStage];
-    const int tid = threadIdx.x;
+    constexpr int kWarps = kT2Threads / 32;
+    __shared__ uint16_t s_ids[kWarps][kFillWords * 32];
+    __shared__ int s_cnt[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t* ids = s_ids[warp];
+    const int64_t turns = (nwords + kFillWords - 1) / kFillWords;
+    const int64_t t0 = turns * warp / kWarps, t1 = turns * (warp + 1) / kWarps;
     for (int qi = blockIdx.x; qi < nq; qi += gridDim.x) {
         const int32_t src = queue[qi];
-        const uint32_t* B = store + (int64_t)qi * nwords;
+        const uint2* B = reinterpret_cast<const uint2*>(store + (int64_t)qi * nwords);
+        // (nwords is even)
+        auto words = [&](int64_t t) {
+            const int64_t wi = t * kFillWords + 2 * lane;
+            uint2 w = wi < nwords ? B[wi >> 1] : make_uint2(0u, 0u);
+            if ((src >> 5) == wi) w.x &= ~(1u << (src & 31));
+            if ((src >> 5) == wi + 1) w.y &= ~(1u << (src & 31));
+            return w;
+        };
+        int cnt = 0;
+#pragma unroll 4
+        for (int64_t t = t0; t < t1; ++t) {
+            const uint2 w = words(t);
+            cnt += __popc(w.x) + __popc(w.y);
+        }
+        cnt = __reduce_add_sync(kFull, cnt);
+        if (lane == 0) s_cnt[warp] = cnt;
+        __syncthreads();
         uint32_t* out = kcol + krow[src];
-        int64_t base = 0;
-        for (int64_t w0 = 0; w0 < nwords; w0 += kT2Threads) {
-            const int64_t wi = w0 + tid;
-            uint32_t w = (wi < nwords) ? B[wi] : 0u;
-            if (wi == (src >> 5)) w &= ~(1u << (src & 31));
-            int64_t total;
-            const int64_t incl =
-                block_inclusive_scan<int64_t, kT2Threads>((int64_t)__popc(w), s_wt, &total);
-            int o = (int)(incl - __popc(w));
-            while (w) {
-                const int b = __ffs(w) - 1;
-                s_ids[o++] = (uint32_t)(wi * 32 + b);
-                w &= w - 1;
-            }
-            __syncthreads();
-            for (int i = tid; i < (int)total; i += kT2Threads) out[base + i] = s_ids[i];
-            __syncthreads();
-            base += total;
+        for (int w = 0; w < warp; ++w) out += s_cnt[w];
+        __syncthreads();  // s_cnt is free for the next source
+        for (int64_t t = t0; t < t1; ++t) {
+            const uint2 w = words(t);
+            const int c = __popc(w.x) + __popc(w.y);
+            const int incl = warp_inclusive_scan(c, lane);
+            const int total = __shfl_sync(kFull, incl, 31);
+            if (total == 0) continue;
+            int o = incl - c;
+            for (uint32_t m = w.x; m; m &= m - 1) ids[o++] = (uint16_t)(64 * lane + __ffs(m) - 1);
+            for (uint32_t m = w.y; m; m &= m - 1) ids[o++] = (uint16_t)(64 * lane + 31 + __ffs(m));
+            __syncwarp();
+            const uint32_t first = (uint32_t)(t * kFillWords * 32);
+            for (int i = lane; i < total; i += 32) out[i] = first + ids[i];
+            out += total;
+            __syncwarp();
         }
     }
 }
@@ -1009,9 +1048,13 @@ gila_status build_khop_count_impl(gila_graph* g, int k)
                 ball2_kernel<<<(unsigned)std::min<int64_t>(n, (int64_t)sms * 8), kT2Threads, smem,
                                st>>>(n, g->row, g->col, nwords, b2);
                 count_launch();
-                ball3_or_kernel<<<(unsigned)std::min<int64_t>(nq, (int64_t)sms * 8), kT2Threads, 0,
-                                  st>>>(S.queue, nq, g->row, g->col, nwords, b2, S.counts,
-                                        store);
+                const int64_t per = (nwords / 4 + kT2Threads - 1) / kT2Threads;
+                auto* or_kernel = per <= 1   ? ball3_or_kernel<1>
+                                  : per <= 2 ? ball3_or_kernel<2>
+                                  : per <= 4 ? ball3_or_kernel<4>
+                                             : ball3_or_kernel<8>;
+                or_kernel<<<(unsigned)std::min<int64_t>(nq, (int64_t)sms * 8), kT2Threads, 0, st>>>(
+                    S.queue, nq, g->row, g->col, nwords, b2, S.counts, store);
                 count_launch();
                 cudaError_t e = cudaStreamSynchronize(st);
                 if (e != cudaSuccess) return cuda_fail(e, "radius-3 balls");

@@ -205,3 +205,21 @@ def test_weighted_tiles(n, tv, prec):
             assert G.gila_profile_read_kernel(h.handle)["name"].startswith(kernel)
             got = disp.double().cpu().numpy()
             assert np.abs(got - want).max() <= TOL[prec] * np.abs(want).max()
+
+
+# balls stored as bitmaps: words below and above a warp's turn of 64, a last
+# turn of one word, one to four 16-byte words a thread in the radius-3 unions
+# (dense Chung-Lu), and sparse balls of many words (Barabasi-Albert)
+@pytest.mark.parametrize("g,k", [
+    (I.chung_lu(2049, 2.3, 8.0, 8196, 1), 3), (I.chung_lu(6001, 2.3, 8.0, 24004, 2), 3),
+    (I.chung_lu(33000, 2.3, 8.0, 132000, 3), 3), (I.chung_lu(70001, 2.3, 8.0, 280004, 4), 3),
+    (I.barabasi_albert_fast(40000, 3, 5), 2), (I.star(3000), 2),
+], ids=["cl2049", "cl6001", "cl33000", "cl70001", "ba40000", "star"])
+def test_khop_rows_from_bitmaps(g, k):
+    deg = np.diff(g.row_ptr)
+    sel = np.unique(np.concatenate([np.argsort(-deg)[:20], np.linspace(0, g.n - 1, 150).astype(int)]))
+    want_counts, want = O.khop_rows(g.n, g.row_ptr, g.col_idx, k, sel)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_build_khop(h.handle, k)
+        counts, cols = G.gila_khop_export_rows(h.handle, sel)
+    assert np.array_equal(counts, want_counts) and np.array_equal(cols, want)
