@@ -223,3 +223,30 @@ def test_khop_rows_from_bitmaps(g, k):
         G.gila_build_khop(h.handle, k)
         counts, cols = G.gila_khop_export_rows(h.handle, sel)
     assert np.array_equal(counts, want_counts) and np.array_equal(cols, want)
+
+
+@pytest.mark.parametrize("name,g,tune", [
+    ("plain", I.grid(20, 21), {}), ("tiles", I.barabasi_albert(3000, 2, 3), dict(tiled=1, tile_vertices=500)),
+    ("rows", I.tri_mesh(40, 50), dict(tiled=1)),
+], ids=["plain", "tiles", "rows"])
+def test_stream_capture(name, g, tune):
+    """Iterations captured into a CUDA graph replay to the same placement."""
+    import torch
+    x0 = torch.tensor(I.uniform_positions(g.n, 51), dtype=torch.float32, device="cuda")
+    prm = G.params(k=2, iters=6, t0=0.3)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, **tune) if tune else None
+        x = x0.clone()
+        G.gila_layout_run_device(h.handle, prm, x)  # lists and plan
+        torch.cuda.synchronize()
+        want = x.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            G.gila_graph_set_stream(h.handle)
+            G.gila_layout_run_device(h.handle, prm, x)
+        for _ in range(2):
+            x.copy_(x0)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(x, want)
+        G.gila_graph_set_stream(h.handle)
