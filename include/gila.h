@@ -252,7 +252,9 @@ gila_status gila_layout_metrics(gila_graph* g, const gila_params* prm, const voi
  * rows) in which a CTA or a cluster of CTAs takes one graph at a time and
  * carries it through all iterations with its placement staged in shared
  * memory. The launch is captured in a CUDA graph and replayed while the
- * arguments stay the same. Every graph follows its own temperature schedule
+ * arguments stay the same. CTAs of a cluster bound their waits for each
+ * other's positions; one that gives up is reported as GILA_ECUDA by the next
+ * gila_layout_batch_run in the process. Every graph follows its own temperature schedule
  * (default t0 from its own n and initial bounding box). A graph's result
  * depends only on the graph, its placement, the parameters and the batch
  * tuning, not on the other graphs of the batch. Precisions: GILA_FP32,

@@ -916,17 +916,22 @@ gila_status batch_plan(gila_batch* b)
         for (int32_t i = 0; i < count; ++i)
             std::fill(sg.begin() + soff[(size_t)i], sg.begin() + soff[(size_t)i + 1], i);
         const size_t n1 = (size_t)std::max<int64_t>(g->n, 1), s1 = (size_t)std::max<int64_t>(nsl, 1);
-        GILA_CUDA(cudaMalloc(&b->sgraph, sizeof(int32_t) * s1));
-        GILA_CUDA(cudaMalloc(&b->sdesc, sizeof(int2) * s1));
-        GILA_CUDA(cudaMalloc(&b->base, sizeof(int32_t) * (size_t)count));
-        GILA_CUDA(cudaMalloc(&b->units, sizeof(int32_t) * (size_t)count));
-        GILA_CUDA(cudaMalloc(&b->skip, 2 * (size_t)count));
-        GILA_CUDA(cudaMalloc(&b->deg, sizeof(uint16_t) * n1));
-        GILA_CUDA(cudaMalloc(&b->perm, sizeof(uint16_t) * n1));
-        GILA_CUDA(cudaMalloc(&b->rank, sizeof(uint16_t) * n1));
-        GILA_CUDA(cudaMalloc(&b->cuts, sizeof(uint16_t) * (kBrCluster + 1) * (size_t)count));
-        for (int w = 0; w < 2; ++w)
-            GILA_CUDA(cudaMalloc(&b->rorder[w], sizeof(int32_t) * (size_t)count));
+        // (what an earlier call that ran out of memory left is kept)
+        auto need = [](auto** p, size_t bytes) -> gila_status {
+            if (!*p) GILA_CUDA(cudaMalloc(p, bytes));
+            return GILA_OK;
+        };
+        gila_status s;
+        if ((s = need(&b->sgraph, sizeof(int32_t) * s1)) || (s = need(&b->sdesc, sizeof(int2) * s1)) ||
+            (s = need(&b->base, sizeof(int32_t) * (size_t)count)) ||
+            (s = need(&b->units, sizeof(int32_t) * (size_t)count)) ||
+            (s = need(&b->skip, 2 * (size_t)count)) || (s = need(&b->deg, sizeof(uint16_t) * n1)) ||
+            (s = need(&b->perm, sizeof(uint16_t) * n1)) ||
+            (s = need(&b->rank, sizeof(uint16_t) * n1)) ||
+            (s = need(&b->cuts, sizeof(uint16_t) * (kBrCluster + 1) * (size_t)count)) ||
+            (s = need(&b->rorder[0], sizeof(int32_t) * (size_t)count)) ||
+            (s = need(&b->rorder[1], sizeof(int32_t) * (size_t)count)))
+            return s;
         GILA_CUDA(cudaMemcpyAsync(b->sgraph, sg.data(), sizeof(int32_t) * (size_t)nsl,
                                   cudaMemcpyHostToDevice, st));
         int32_t* so = nullptr;
@@ -1074,12 +1079,15 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
         GILA_CUDA(cudaMemcpy(b->geo, geo.data(), sizeof(double) * geo.size(),
                              cudaMemcpyHostToDevice));
     }
-    if ((s = batch_plan(b)) != GILA_OK) return s;
+    // without memory for the plan every graph keeps the group kernel
+    s = batch_plan(b);
+    if (s != GILA_OK && s != GILA_ENOMEM) return s;
+    const bool planned = s == GILA_OK;
     const int sms = sm_count(g->device);
     const gila_batch_tuning tu = resolved(b, esz, sms);
     // lane groups set by the tuning ask for the group kernel on every graph
     const int w = esz == 16 ? 1 : 0;
-    const bool groups = b->tune.group4_max > 0 || b->tune.group8_max > 0 || b->tune.group16_max > 0;
+    const bool groups = !planned || b->tune.group4_max > 0 || b->tune.group8_max > 0 || b->tune.group16_max > 0;
     const int nbig = groups ? 0 : (int)b->big[w].size();
     const int nrows = groups ? 0 : nbig + (int)b->small[w].size();
     const int nrest = b->count - nrows;

@@ -2004,7 +2004,7 @@ void free_tile_plans(gila_graph* g)
         cudaFree(P.tk);
         cudaFree(P.part);
         cudaFree(P.len);
-        cudaFree(P.pre);
+        cudaFree(P.pre_buf);
         cudaFree(P.cut);
         P = TilePlan();
     }
@@ -2124,12 +2124,15 @@ gila_status plan_hubs(gila_graph* g, TilePlan& P)
 
 // Prefix sums of the cells' padded lengths and costs (P.len, on the device)
 // into P.pre: cells + 1 values each.
-gila_status prefix_cells(gila_graph* g, TilePlan& P, int64_t cells)
+gila_status prefix_cells(gila_graph* g, TilePlan& P, int64_t cells, size_t esz, bool tiles)
 {
     const int64_t nb = (cells + kCellTile - 1) / kCellTile;
     gila_status s;
-    if ((s = ensure((void**)&P.pre, &P.pre_cap, sizeof(int64_t) * 2 * ((size_t)cells + 1))) != GILA_OK ||
-        (s = ensure(&P.cut, &P.cut_cap, sizeof(int64_t) * 2 * (size_t)nb)) != GILA_OK)
+    if ((s = tiles ? ensure(&P.part, &P.part_cap, 2 * esz * (size_t)cells + 16)
+                   : ensure(&P.pre_buf, &P.pre_cap, 16 * ((size_t)cells + 1))) != GILA_OK)
+        return s;
+    P.pre = (int64_t*)(tiles ? P.part : P.pre_buf);
+    if ((s = ensure(&P.cut, &P.cut_cap, sizeof(int64_t) * 2 * (size_t)nb)) != GILA_OK)
         return s;
     int64_t* sums = (int64_t*)P.cut;
     cell_sums_kernel<<<(unsigned)nb, kCellThreads, 0, g->stream>>>(cells, P.len, sums);
@@ -2165,11 +2168,17 @@ gila_status partition_tiles(gila_graph* g, TilePlan& P, int64_t n, int64_t nt, i
     target = std::max<int64_t>(target, nt * ((n + max_rows - 1) / max_rows));
     const int64_t stride = target + 2;
     const size_t per_cap = sizeof(int32_t) * (size_t)(nt * stride);
-    const bool every = per_cap * kCaps <= kCutBytes;
-    const size_t slots = every ? kCaps : 1;  // caps whose cuts are written
-    const size_t at_cuts = (kCaps * 12 + sizeof(int) * (size_t)nt * slots + 15) & ~size_t(15);
-    gila_status s = ensure(&P.cut, &P.cut_cap, at_cuts + per_cap * slots);
-    if (s != GILA_OK) return s;
+    bool every = per_cap * kCaps <= kCutBytes;
+    size_t slots = 0, at_cuts = 0;  // caps whose cuts are written
+    gila_status s;
+    for (;;) {
+        slots = every ? kCaps : 1;
+        at_cuts = (kCaps * 12 + sizeof(int) * (size_t)nt * slots + 15) & ~size_t(15);
+        s = ensure(&P.cut, &P.cut_cap, at_cuts + per_cap * slots);
+        if (s == GILA_OK) break;
+        if (!every) return s;
+        every = false;
+    }
     int64_t* d_caps = (int64_t*)P.cut;
     int* d_counts = (int*)(d_caps + kCaps);
     int* d_tiles = d_counts + kCaps;
@@ -2622,7 +2631,7 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
                 rowlen_kernel<<<(unsigned)((n + 255) / 256), 256, 0, g->stream>>>(n, g->krow, P.len,
                                                                                 P.len + n);
                 count_launch();
-                if ((s = prefix_cells(g, P, n)) != GILA_OK) return s;
+                if ((s = prefix_cells(g, P, n, esz, false)) != GILA_OK) return s;
                 if ((s = build_layout(g, esz, P, 1, 0, {rs}, &wb)) != GILA_OK) return s;
                 P.window = true;
                 P.tv = (int32_t)wmax;
@@ -2662,7 +2671,7 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
     GILA_CUDA(cudaGetLastError());
     // each tile's row ranges: blocks of about equal cost (padded entries +
     // a per-row term), at most rmax rows each, about ctas_per_sm per SM
-    if ((s = prefix_cells(g, P, cells)) != GILA_OK) return s;
+    if ((s = prefix_cells(g, P, cells, esz, true)) != GILA_OK) return s;
     // the block count: at least 5% above what the row limit alone makes,
     // so that a tile with more entries than the others (the hubs' ids) can
     // still be cut finer, and whole waves of one CTA per SM, since blocks of

@@ -115,7 +115,10 @@ struct TilePlan {
                                      // (plan scratch, quality figures)
     size_t len_cap = 0;
     int64_t* pre = nullptr;          // plan scratch: 2 (nt n + 1) prefix sums of the segments'
-    size_t pre_cap = 0;              // padded lengths, then of their costs
+                                     // padded lengths, then of their costs (in part, which
+                                     // only iterations use, or in pre_buf: window mode)
+    void* pre_buf = nullptr;
+    size_t pre_cap = 0;
     void* cut = nullptr;             // plan scratch: cuts of the tiles' rows and their counts
     size_t cut_cap = 0;
     // window mode: one window of positions per row range, covering every id
