@@ -87,10 +87,10 @@ KERNEL_SOURCES = ("paper_1606_02162_gb300/csrc/blocked.cu",
                   "paper_1606_02162_gb300/csrc/force.cuh",
                   "paper_1606_02162_gb300/csrc/device_util.cuh")
 NCU_TRAFFIC = {
-    "chunglu250k_k3": {"bytes": 22770000000 + 96030000 + 52050000 + 512,
+    "chunglu250k_k3": {"bytes": 22759501312 + 96195328 + 52051712,
                        "kernels": "blocked_kernel + combine_kernel (one iteration)",
                        "profile": "profiles/launches_chunglu250k_k3.md",
-                       "sources_sha256": "ef1358f5c4f89edf74c85712a3ee31cc3b3757f3ada5517093e71b6c4fcefe66"},
+                       "sources_sha256": "c3aacda95e9249d69edcad81ad61fbf0c14ab3afedfd8d3a7157c38ed3ede079"},
 }
 
 
