@@ -90,7 +90,7 @@ NCU_TRAFFIC = {
     "chunglu250k_k3": {"bytes": 22759501312 + 96195328 + 52051712,
                        "kernels": "blocked_kernel + combine_kernel (one iteration)",
                        "profile": "profiles/launches_chunglu250k_k3.md",
-                       "sources_sha256": "c3aacda95e9249d69edcad81ad61fbf0c14ab3afedfd8d3a7157c38ed3ede079"},
+                       "sources_sha256": "f85466d58189c5fd5548795362a2dd88806883d3f2db912247d029f844a202ac"},
 }
 
 

@@ -2050,14 +2050,10 @@ int64_t cut_rows(const int64_t* pre, int64_t n, int64_t cap, int64_t limit, int6
     return count;
 }
 
-// Row ranges of every tile (window mode: one), all blocks with at most the
-// same cost, the smallest for which the blocks number at most `target` (or
-// the fewest the row limit allows). pre: nt prefix-sum arrays of n + 1
-// costs, tile after tile. A grid of about target equal CTAs then ends
-// together, where equal row ranges for all tiles left the hubs' tile with
-// CTAs twice the mean and one more range than the target sent a few CTAs
-// into a second wave (Barabasi-Albert n = 100,000, k = 2: 156 CTAs on 152
-// SMs, the SMs busy 54% of the kernel's time).
+// The same on the host, for window mode (its rows, or slices of rows, as one
+// tile): the smallest block cost for which the greedy cut gives at most
+// `target` ranges (or the fewest the row limit allows). pre: nt prefix-sum
+// arrays of n + 1 costs, tile after tile.
 std::vector<std::vector<int32_t>> partition_blocks(const std::vector<int64_t>& pre, int64_t n,
                                                    int64_t nt, int64_t target, int64_t max_rows)
 {
