@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 // keep), whose bound was the latency of one group's chain (offsets, ids,
 // positions, reduction) and, in FP64, lanes without work on the two FP64
 // operations a clock of an SM: 500 graphs of 50..5000 vertices, k = 2, 50
-// iterations in FP32 6.5 -> 0.60 ms, 3000 graphs 9.2 -> 1.6 ms (30
+// iterations in FP32 6.5 -> 0.58 ms, 3000 graphs 9.2 -> 1.6 ms (30
 // iterations), 250 graphs in FP64 20.8 -> 3.9 ms (20 iterations; its FP64
 // pipe is 63% busy, the FP32 form issues in 52% of the cycles, the rest mostly
 // the barrier between iterations).
@@ -501,6 +501,19 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                         if (k0 + x >= steps) break;
                         const uint32_t i0 = c4[x].x & 0xffffu, i1 = c4[x].x >> 16;
                         const uint32_t i2 = c4[x].y & 0xffffu, i3 = c4[x].y >> 16;
+                        const int e = 4 * (k0 + x);
+                        if constexpr (sizeof(T) == 4 && MODEL == kFR) {
+                            if (e < dmax) {  // the rows' first ids are their neighbours
+                                auto both = [&](auto& to) {
+                                    fr_entry(cur[i0], pu.x, pu.y, att.inv_d, e < deg, to, at);
+                                    fr_entry(cur[i1], pu.x, pu.y, att.inv_d, e + 1 < deg, to, at);
+                                    fr_entry(cur[i2], pu.x, pu.y, att.inv_d, e + 2 < deg, to, at);
+                                    fr_entry(cur[i3], pu.x, pu.y, att.inv_d, e + 3 < deg, to, at);
+                                };
+                                if constexpr (COMP) both(pend); else both(acc);
+                                continue;
+                            }
+                        }
                         if constexpr (COMP) {
                             f(i0, pend);
                             f(i1, pend);
@@ -512,8 +525,7 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                             f(i2, acc);
                             f(i3, acc);
                         }
-                        const int e = 4 * (k0 + x);
-                        if (e < dmax) {  // the rows' first ids are their neighbours
+                        if (e < dmax) {
                             if (e < deg) att(i0, at);
                             if (e + 1 < deg) att(i1, at);
                             if (e + 2 < deg) att(i2, at);

@@ -699,7 +699,8 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
 // keeps their gathers free of bank conflicts without any reordering. 512
 // threads at 64 registers put two CTAs on an SM, one loading its window
 // while the other computes.
-// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration
+// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration (29.7
+// since, with early launches and fr_entry)
 // against the shares of blocked_kernel; 700 x 700, FP32: 35.3 -> 17.6.
 //
 // Automatic mode takes it where (us per iteration, FP32, before -> this):
@@ -839,6 +840,19 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
                 if (k0 + i >= steps) break;
                 const uint32_t v0 = cur[i].x & 0xffffu, v1 = cur[i].x >> 16;
                 const uint32_t v2 = cur[i].y & 0xffffu, v3 = cur[i].y >> 16;
+                const int e = 4 * (k0 + i);
+                if constexpr (sizeof(T) == 4 && MODEL == kFR) {
+                    if (e < dmax) {  // the rows' first ids are their neighbours
+                        auto both = [&](auto& to) {
+                            fr_entry(tile[v0], pu.x, pu.y, att.inv_d, e < deg, to, at);
+                            fr_entry(tile[v1], pu.x, pu.y, att.inv_d, e + 1 < deg, to, at);
+                            fr_entry(tile[v2], pu.x, pu.y, att.inv_d, e + 2 < deg, to, at);
+                            fr_entry(tile[v3], pu.x, pu.y, att.inv_d, e + 3 < deg, to, at);
+                        };
+                        if constexpr (COMP) both(pend); else both(acc);
+                        continue;
+                    }
+                }
                 if constexpr (COMP) {
                     f(v0, pend);
                     f(v1, pend);
@@ -850,8 +864,7 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
                     f(v2, acc);
                     f(v3, acc);
                 }
-                const int e = 4 * (k0 + i);
-                if (e < dmax) {  // the rows' first ids are their neighbours
+                if (e < dmax) {
                     if (e < deg) att(v0, at);
                     if (e + 1 < deg) att(v1, at);
                     if (e + 2 < deg) att(v2, at);

@@ -344,6 +344,40 @@ struct Att {
     }
 };
 
+// A k-hop entry at pv that may be a neighbour as well (FP32,
+// Fruchterman-Reingold): the repulsion as Rep forms it, into `rep` without the
+// factor d^2, and with `edge` the attraction from the same difference and
+// r^2 (with the 2^-100, which keeps the square root finite at distance 0,
+// where it multiplies zero). One subtraction and one r^2 serve both: the mesh
+// 1000 x 1000, k = 3, 33.1 -> 29.7 us an iteration, 500 graphs of the batch
+// 634 -> 583 us a pass.
+template <bool CR, bool CA>
+__device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float inv_d, bool edge,
+                                         Acc<float, CR>& rep, Acc<float, CA>& at)
+{
+    uint64_t pu, pp, dd, cc, ac;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(pu) : "f"(xu), "f"(yu));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(pp) : "f"(pv.x), "f"(pv.y));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
+    float dx, dy;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, 0x1p-100f));
+    const float c = rcp_fast(r2);
+    asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(ac) : "f"(rep.sx), "f"(rep.sy));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(rep.sx), "=f"(rep.sy) : "l"(ac));
+    if (edge) {
+        const float s = -(r2 * rsqrt_fast(r2)) * inv_d;
+        if constexpr (CA) {
+            add_compensated(at, s * dx, s * dy);
+        } else {
+            at.sx = fmaf(s, dx, at.sx);
+            at.sy = fmaf(s, dy, at.sy);
+        }
+    }
+}
+
 // Entries [s, e) of kcol, lanes gl = 0..G-1 of a group (G >= 4): an
 // unaligned head of at most 3 entries, 16-byte vector loads of 4 ids,
 // then a tail of at most 3 entries. Which lane takes which entry depends on
