@@ -268,8 +268,17 @@ struct Rep {
             asm("mov.b64 {%0, %1}, %2;" : "=f"(a.sx), "=f"(a.sy) : "l"(ac));
             return;
         }
+        T dx, dy;
+        const T c = term(v, dx, dy);
+        a.add(c * dx, c * dy);
+    }
+
+    // The difference x_u - x_v and its factor c.
+    __device__ __forceinline__ T term(uint32_t v, T& dx, T& dy) const
+    {
         const P2 pv = src(v);
-        const T dx = xu - pv.x, dy = yu - pv.y;
+        dx = xu - pv.x;
+        dy = yu - pv.y;
         T c;
         if (MODEL == kFR) {
             c = UNSCALED ? rep_fr1(dx, dy) : rep_fr(d2, dx * dx + dy * dy);
@@ -284,7 +293,7 @@ struct Rep {
             }
         }
         if (WEIGHTED) c *= SRC == kSrcShared ? wt[v] : __ldg(wt + v);
-        a.add(c * dx, c * dy);
+        return c;
     }
 
     // (the plain kernels: rsqrt squared measured 4% faster there than rcp)

@@ -13,8 +13,11 @@
 // Work is split by row length into four classes, each a range of blocks
 // of the same launch (heaviest first): rows split into chunks summed by the
 // last chunk to finish, one block per row, one warp per row, and groups of
-// 8 lanes per row. A row's reduction order depends only on its length and
-// its position in the k-hop list, so results are reproducible.
+// 8 lanes per row. In FP64 the order of a row's additions depends only on its
+// length and its position in the k-hop list: an iteration's last bits are
+// amplified by those that follow (two vertices passing close by turn a
+// direction), so that a run of a hundred repeats to FP64 accuracy only if every
+// sum keeps its order. In FP32 it depends on the grid's size too (kCoopRow).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -34,10 +37,10 @@ constexpr int kThreads = 256;
 // lanes a clock on an SM, and the latency chain of a row is the same
 // everywhere, so a grid that does not fill the SMs with 256 threads a block
 // is spread over more of them (32 x 32 grid, FP64: 7.2 -> 5.9 us per
-// iteration; with the early launches and rows by entries below 12.5 -> 5.9).
+// iteration; with the early launches and staged rows below 12.5 -> 5.9).
 // Four warps, one for each of an SM's schedulers.
 constexpr int kThreadsSmall = 128;
-// Rows of the warp class longer than this are taken by the whole block in
+// FP32: rows of the warp class longer than this are taken by the whole block in
 // small grids (BA n = 10,000, k = 2: 17.6 -> 12.0 us per iteration with it,
 // the early launches and batched adjacency loads; at 512 14.7, at 256 18.4;
 // from 16 blocks per SM on, hubs' warps no longer stand out: the pruned
@@ -99,22 +102,74 @@ __device__ __forceinline__ void block_reduce(Acc<T, COMP>& a, T* sh)
     }
 }
 
+// Entries of a stage of row_sum_staged: a head and a tail of up to three and
+// eight vectors of four.
+constexpr int kStage = 40;
+
+template <class T>
+struct StageTerm {
+    T c, dx, dy;
+};
+
+// row_sum's sum of a short row by a group of eight lanes, the same additions
+// by the same lanes in the same order, with the terms formed an entry per lane
+// and passed to the lane that adds them through shared memory. An FP64 term
+// takes a dozen operations on a pipe of two lanes a clock, its addition two:
+// with row_sum the group forms four terms one after the other on the few lanes
+// that have a vector (32 x 32 grid, rows of twelve: 7.2 us an iteration with
+// it, 5.9 here). Every lane of the warp calls it; chunks of 32 aligned entries at a time.
+template <class T, class R, class A>
+__device__ __forceinline__ void row_sum_staged(const uint32_t* __restrict__ kcol, int64_t s,
+                                               int64_t e, int gl, const R& rep,
+                                               StageTerm<T>* stage, A& a)
+{
+    int64_t s4 = (s + 3) & ~int64_t(3);
+    if (s4 > e) s4 = e;
+    int64_t e4 = e & ~int64_t(3);
+    if (e4 < s4) e4 = s4;
+    const int head = (int)(s4 - s), body = (int)(e4 - s4), len = (int)(e - s);
+    const int chunks = __reduce_max_sync(kFull, (body + 31) >> 5);
+    auto add = [&](int at) {
+        const StageTerm<T> t = stage[at];
+        a.add(t.c * t.dx, t.c * t.dy);
+    };
+    for (int b = 0; b < chunks || b == 0; ++b) {
+        const bool last = 32 * (b + 1) >= body;
+        const int lo = b == 0 ? 0 : head + 32 * b;
+        const int hi = 32 * b >= body && b > 0 ? lo : last ? len : head + 32 * (b + 1);
+        for (int j = lo + gl; j < hi; j += 8) {
+            StageTerm<T> t;
+            t.c = rep.term(ld_id(kcol + s + j), t.dx, t.dy);
+            stage[j - lo] = t;
+        }
+        __syncwarp();
+        if (b == 0 && gl < head) add(gl);
+        if (32 * b + 4 * gl < body) {
+            const int at = head + 32 * b + 4 * gl - lo;
+            add(at);
+            add(at + 1);
+            add(at + 2);
+            add(at + 3);
+        }
+        if (hi == len && hi > lo && head + body + gl < len) add(head + body + gl - lo);
+        __syncwarp();
+    }
+}
+
 // Repulsion over the k-hop entries [ks, ke) of a vertex at pu and, when
 // with_att, attraction over its adjacency entries [ab, ae), by lanes
-// gl = 0..G-1 of a group. SHORT rows are taken an entry per lane (a row of
-// twelve: two rounds of eight lanes; by vectors of four ids three lanes had
-// four entries each: the 32 x 32 grid, FP64, 7.3 -> 5.9 us), others by
-// vectors.
-template <class T, int MODEL, bool COMP, bool SHORT = false, class R, class P2>
+// gl = 0..G-1 of a group. With a stage (short rows in FP64, whole warps) the
+// terms go through it.
+template <class T, int MODEL, bool COMP, bool STAGED = false, class R, class P2>
 __device__ __forceinline__ void vertex_sum(const IterArgs& A, R rep,
                                            Att<T, MODEL, COMP> att, P2 pu, int64_t ks, int64_t ke,
                                            int64_t ab, int64_t ae, bool with_att, int gl, int G,
-                                           Acc<T, COMP>& a)
+                                           Acc<T, COMP>& a, StageTerm<T>* stage = nullptr)
 {
     rep.xu = pu.x;
     rep.yu = pu.y;
-    if (SHORT)
-        row_sum_batched<4>(A.kcol, ks, ke, gl, G, rep, a);
+    if constexpr (STAGED)
+        row_sum_staged<T>(A.kcol, ks, ke, gl, rep, stage, a);
     else
         row_sum(A.kcol, ks, ke, gl, G, rep, a);
     if (with_att) {
@@ -143,6 +198,8 @@ iteration_kernel(const IterArgs A)
     __shared__ T sh[kWarps * 4];
     __shared__ int s_last;
     __shared__ int s_len[kWarps];
+    constexpr bool STAGED = sizeof(T) == 8;
+    __shared__ StageTerm<T> s_stage[STAGED ? NT / 8 : 1][kStage];
     const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
     Rep<T, MODEL, COMP, kSrcGlobal, false, W> rep;
     rep.src.pos = pos;
@@ -269,10 +326,10 @@ iteration_kernel(const IterArgs A)
         P2 pu;
         pu.x = T(0);
         pu.y = T(0);
-        if (live) {
-            pu = pos[u];
-            vertex_sum<T, MODEL, COMP, true>(A, rep, att, pu, ks, ke, ab, ae, true, gl, G, a);
-        }
+        if (live) pu = pos[u];
+        if (STAGED || live)
+            vertex_sum<T, MODEL, COMP, STAGED>(A, rep, att, pu, ks, ke, ab, ae, true, gl, G, a,
+                                               s_stage[STAGED ? threadIdx.x / G : 0]);
         a.group_reduce(G);
         if (live && gl == 0) apply_move_it<T>(A, u, pu.x, pu.y, a.fx(), a.fy());
     }
@@ -654,7 +711,8 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
     A.nchunks = B.nchunks;
     A.b3 = B.nchunks;
     A.b2 = B.n2;
-    // blocks of 256 threads, or of 64 where those would not fill the SMs twice
+    // blocks of 256 threads, or of 128 where those would not fill the SMs twice
+    // (FP64 rows summed by a whole block keep theirs: their order of additions)
     auto blocks = [&](int nt) {
         A.b1 = (B.n1 + nt / 32 - 1) / (nt / 32);
         A.b0 = (B.n0 + nt / 8 - 1) / (nt / 8);
@@ -663,15 +721,16 @@ gila_status launch_iteration(gila_graph* g, const gila_params* prm, double t, co
     int nt = kThreads;
     const int64_t sms = sm_count(g->device);
     const int64_t grid0 = blocks(nt);
-    if (grid0 < 2 * sms) blocks(nt = kThreadsSmall);
-    A.coop = grid0 < 16 * sms ? kCoopRow : INT_MAX;
+    const bool f64 = is_f64(prm->precision);
+    if (grid0 < 2 * sms && !(f64 && A.b3 + A.b2 > 0)) blocks(nt = kThreadsSmall);
+    A.coop = !f64 && grid0 < 16 * sms ? kCoopRow : INT_MAX;
     A.c = force_consts(prm->d, t);
     A.p = prm->p;
     A.q = prm->q;
     A.pos_in = pos_in;
     A.pos_out = pos_out;
     A.disp_out = disp_out;
-    A.wt = is_f64(prm->precision) ? (const void*)g->wt64 : (const void*)g->wt32;
+    A.wt = f64 ? (const void*)g->wt64 : (const void*)g->wt32;
     const int64_t grid = (int64_t)A.b3 + A.b2 + A.b1 + A.b0;
     if (grid == 0) return GILA_OK;
     const bool fr = (prm->p == 2 && prm->q == 1);

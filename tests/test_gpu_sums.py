@@ -1,0 +1,65 @@
+"""The sums of the force kernels: orders of additions that results rely on,
+and the accuracy each mode promises."""
+import os
+
+import numpy as np
+import pytest
+
+import __graft_entry__
+import oracle as O
+from paper_1606_02162_gb300 import gila as G
+from paper_1606_02162_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+GOLD = os.path.join(os.path.dirname(__file__), "golden")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+    import torch
+    torch.cuda.set_device(0)
+
+
+def test_fp64_run_keeps_its_order_of_additions():
+    """A hundred FP64 iterations in which two vertices pass close by: short
+    rows added in another order (an entry per lane) end 3e-5 away, by a CPU
+    restatement of both orders; the recorded order repeats exactly."""
+    import torch
+    want = np.loadtxt(os.path.join(GOLD, "grid_fp64_run.txt"))
+    g = I.grid(12, 12)
+    x = torch.tensor(I.uniform_positions(g.n, 5), dtype=torch.float64, device="cuda")
+    with G.Graph.from_inputs(g) as h:
+        G.gila_layout_run_device(h.handle, G.params(k=2, iters=100, t0=0.02, precision=G.GILA_FP64), x)
+    assert np.abs(x.cpu().numpy() - want).max() <= 1e-12 * np.abs(want).max()
+
+
+# FP64 rows that go through the stage: empty, below and above a vector, heads
+# and tails of every length, one and more chunks of 32 entries, the last with
+# and without a tail; with weights and other exponents
+@pytest.mark.parametrize("pq,weighted", [((2, 1), False), ((2, 1), True), ((3, 2), False)],
+                         ids=["fr", "weighted", "p3q2"])
+def test_staged_rows_fp64(pq, weighted):
+    import torch
+    p, q = pq
+    rng = np.random.default_rng(3)
+    sizes = list(range(1, 75)) + [96, 97, 98, 99, 127, 128, 129, 200]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    # cliques: rows of every length and, in turn, every alignment
+    a = np.concatenate([o + np.triu_indices(s, 1)[0] for o, s in zip(off, sizes)])
+    b = np.concatenate([o + np.triu_indices(s, 1)[1] for o, s in zip(off, sizes)])
+    g = I.csr_from_edges(int(off[-1]) + 5, a, b)
+    pos = I.uniform_positions(g.n, 9)
+    w = 1.0 + rng.integers(0, 4, g.n) if weighted else None
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 1)
+    _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, 0.4, d=1.1, p=p, q=q, wt=w)
+    x = torch.tensor(pos, device="cuda")
+    y, disp = torch.empty_like(x), torch.empty_like(x)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, tiled=0, small_max=256)  # every row by a group of eight
+        if weighted:
+            G.gila_graph_set_repulsion_weights(h.handle, w)
+        G.gila_layout_step(h.handle, G.params(k=1, d=1.1, p=p, q=q, precision=G.GILA_FP64), 0.4, x, y,
+                           disp)
+    assert np.abs(disp.cpu().numpy() - want).max() <= 1e-12 * np.abs(want).max()
