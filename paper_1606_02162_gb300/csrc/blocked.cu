@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
     const int64_t bsp = A.blk[2 * (int64_t)blockIdx.x];  // the block's first slot in tk
     // a block holds at most kMaxRows segments of at most tv entries: < 2^31
     const int32_t L = (int32_t)A.blk[2 * (int64_t)blockIdx.x + 1];
-    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
+    const P2* pos = reinterpret_cast<const P2*>(A.pos);
     const int64_t tb = WIN ? A.wbase[2 * blockIdx.x] : (int64_t)j * A.tv;
     const int64_t tn = WIN ? A.wbase[2 * blockIdx.x + 1]
                            : ((A.n - tb < A.tv) ? A.n - tb : (int64_t)A.tv);
@@ -640,7 +640,7 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
 {
     using P2 = typename V2<T>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
+    const P2* pos = reinterpret_cast<const P2*>(A.pos);
     Att<T, MODEL, COMP, kSrcShared> att;
     att.src.set_shared(tile, (uint32_t)tb);
     att.inv_d = const_inv_d<T>(A.c);
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
     __shared__ __align__(8) uint64_t tile_bar;
     __shared__ int tile_ok;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos);
+    const P2* pos = reinterpret_cast<const P2*>(A.pos);
     const int64_t tb = A.wbase[2 * blockIdx.x], tn = A.wbase[2 * blockIdx.x + 1];
     pdl_trigger();
     // this warp's slices and the first steps of their stream, read while the
@@ -997,9 +997,10 @@ template <class T, int MODEL, bool COMP>
 __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineArgs A)
 {
     using P2 = typename V2<T>::type;
-    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
-    Att<T, MODEL, COMP> att;
-    att.src.pos = pos;
+    // (launched after the kernel before has ended: nothing writes this placement)
+    const P2* __restrict__ pos_in = reinterpret_cast<const P2*>(A.pos_in);
+    Att<T, MODEL, COMP, kSrcConst> att;
+    att.src.pos = pos_in;
     att.inv_d = const_inv_d<T>(A.c);
     att.p = A.p;
     Acc<T, COMP> rep, at;
@@ -1010,7 +1011,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const int64_t u = A.hubs[blockIdx.x];
         const int64_t rb = A.row[u], re = A.row[u + 1];
-        const P2 pu = pos[u];
+        const P2 pu = pos_in[u];
         for (int jj = threadIdx.x; jj < A.nt; jj += kCombineThreads)
             add_cell<T, COMP>(A.part, A.n, jj, u, rep);
         att.xu = pu.x;
@@ -1064,7 +1065,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
     if (live) {
         // tile partials first (independent loads), lane gl takes tiles gl, gl + 8, ...
         for (int jj = gl; jj < A.nt; jj += kCombineLanes) add_cell<T, COMP>(A.part, A.n, jj, u, rep);
-        pu = pos[u];
+        pu = pos_in[u];
         att.xu = pu.x;
         att.yu = pu.y;
         if (gl < deg) att(ahead[0], at);

@@ -66,8 +66,12 @@ __device__ __forceinline__ T group_sum(T v, int width)
 // it on the stream still runs, once every block of that one has called
 // pdl_trigger() or ended. Until pdl_wait(), which returns when the kernel
 // before has completed and its writes are visible, it may only read what no
-// kernel of the iteration writes (lists, plan). Every thread calls pdl_wait(),
-// so that a completed kernel implies all before it completed.
+// kernel of the iteration writes (lists, plan). What such a kernel does write
+// (placements, partials) is read by ordinary loads after pdl_wait(), through
+// pointers without __restrict__: the compiler may turn a load through a
+// restricted pointer to const into ld.global.nc, which is not ordered by the
+// wait. Every thread calls pdl_wait(), so that a completed kernel implies all
+// before it completed.
 
 __device__ __forceinline__ void pdl_trigger()
 {

@@ -165,7 +165,11 @@ __device__ __forceinline__ void add_compensated(Acc<T, COMP>& acc, T x, T y)
 
 // Where a kernel reads positions from.
 enum Src {
-    kSrcGlobal = 0,   // the whole placement, read-only for the launch (ld.global.nc)
+    kSrcGlobal = 0,   // the whole placement in global memory, by ordinary loads: a kernel that
+                      // starts early is resident while the one before still writes it, so
+                      // that ld.global.nc, whose data must not change while a kernel runs, is
+                      // for lists, offsets and weights only
+    kSrcConst = 3,    // the same by ld.global.nc, in a kernel launched after all that write it
     kSrcShared = 1,   // a shared-memory tile of ids [base, base + size), 32-bit addresses
     kSrcGeneric = 2   // a buffer of ids [base, base + size) in shared or global memory
 };
@@ -210,7 +214,7 @@ __device__ __forceinline__ float rcp_fast(float x)
 template <class T, int SRC>
 struct PosSource {
     using P2 = typename V2<T>::type;
-    const P2* __restrict__ pos = nullptr;  // kSrcGlobal / kSrcGeneric
+    const P2* pos = nullptr;               // kSrcGlobal / kSrcConst / kSrcGeneric
     uint32_t base = 0;                     // first id held (kSrcShared / kSrcGeneric)
     const P2* shp = nullptr;               // kSrcShared: tile shifted so that shp[v] is id v
 
@@ -225,7 +229,8 @@ struct PosSource {
     {
         if (SRC == kSrcShared) return shp[v];
         if (SRC == kSrcGeneric) return pos[v - base];
-        return __ldg(pos + v);
+        if (SRC == kSrcConst) return __ldg(&pos[v]);
+        return pos[v];
     }
 };
 

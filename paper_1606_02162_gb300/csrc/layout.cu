@@ -200,7 +200,7 @@ iteration_kernel(const IterArgs A)
     __shared__ int s_len[kWarps];
     constexpr bool STAGED = sizeof(T) == 8;
     __shared__ StageTerm<T> s_stage[STAGED ? NT / 8 : 1][kStage];
-    const P2* __restrict__ pos = reinterpret_cast<const P2*>(A.pos_in);
+    const P2* pos = reinterpret_cast<const P2*>(A.pos_in);
     Rep<T, MODEL, COMP, kSrcGlobal, false, W> rep;
     rep.src.pos = pos;
     rep.d2 = const_d2<T>(A.c);
