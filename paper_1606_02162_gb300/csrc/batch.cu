@@ -256,11 +256,15 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 //
 // CTAs come in clusters of 1, 2, 4 or 8. A graph that would keep one CTA busy
 // for longer than its share of the batch is taken by a whole cluster: every
-// CTA holds the placement, computes a contiguous part of the slices (equal
-// steps), and pushes its new positions into the other CTAs' shared memory
+// CTA with slices holds the placement, computes a contiguous part of the slices
+// (equal steps), and pushes its new positions into the others' shared memory
 // with bulk copies that complete on their mbarriers, one mbarrier per parity
-// of the iteration (a CTA can be at most one iteration ahead of another: it
-// needs the other's positions to go on). After the large graphs each CTA
+// of the iteration. A CTA needs the positions of every other one to go on, so
+// that it is at most one iteration ahead of any: two mbarriers suffice, and a
+// buffer is overwritten only after its last reader. A CTA whose part is empty
+// (fewer slices than CTAs, or one slice that outweighs several shares) pushes
+// nothing, so that nobody would wait for it: it takes no part in the graph and
+// nothing is pushed to it. After the large graphs each CTA
 // takes small ones on its own. The order of a row's additions is the same in
 // every case and depends on the graph alone.
 //
@@ -367,7 +371,7 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
         mbar_init(&s_bar[0], 1);
         mbar_init(&s_bar[1], 1);
     }
-    uint32_t done_iters = 0;  // iterations exchanged so far: parity and phase of the mbarriers
+    uint32_t phase = 0;  // bit i: parity of the phase of s_bar[i] that this CTA waits for next
     bool failed = false;
 
     // one graph, its slices [s0 + ca, s0 + cb) on this CTA
@@ -381,6 +385,10 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
         const int part = kBrCluster / (int)csize;  // eighths of the graph per CTA
         const int ca = big ? cuts[rank * part] : 0;
         const int cb = big ? cuts[(rank + 1) * part] : ns;
+        if (ca == cb) return;  // no slices: no part in the exchange below
+        uint32_t peers = 0;    // the other CTAs of the cluster that have slices, a bit each
+        for (uint32_t r = 0; big && r < csize; ++r)
+            if (r != rank && cuts[(r + 1) * part] > cuts[r * part]) peers |= 1u << r;
         const uint16_t* perm = A.perm + v0;
         for (int i = threadIdx.x; i < n; i += blockDim.x) buf0[i] = gpos[v0 + perm[i]];
         if (threadIdx.x == 0) {
@@ -551,25 +559,27 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                 // push this CTA's new positions to its peers and wait for theirs
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncthreads();
-                uint64_t* bar = &s_bar[done_iters & 1];
+                uint64_t* bar = &s_bar[it & 1];
+                const uint32_t parity = (phase >> (it & 1)) & 1;
                 const uint32_t mine = (uint32_t)(cb - ca) * 32u * (uint32_t)sizeof(P2);
                 if (threadIdx.x == 0)
                     mbar_arrive_expect_tx(bar, (uint32_t)npad * (uint32_t)sizeof(P2) - mine);
-                if (threadIdx.x == 0 && mine > 0 && !failed) {
+                if (threadIdx.x == 0 && !failed) {
                     const uint32_t src = smem_addr(nxt + ca * 32), b = smem_addr(bar);
                     for (uint32_t r = 1; r < csize; ++r) {
                         const uint32_t to = (rank + r) & (csize - 1);
-                        bulk_s2s(cluster_map(src, to), src, mine, cluster_map(b, to));
+                        if ((peers >> to) & 1)
+                            bulk_s2s(cluster_map(src, to), src, mine, cluster_map(b, to));
                     }
                 }
-                if (!failed && !mbar_wait(bar, (done_iters >> 1) & 1, A.wait_ns)) {
+                if (!failed && !mbar_wait(bar, parity, A.wait_ns)) {
                     // give up: flag it, let what is in flight land (bounded),
                     // push and wait no more; the cluster leaves together
                     failed = true;
                     atomicExch(&g_batch_wait_failed, 1);
-                    mbar_wait(bar, (done_iters >> 1) & 1, A.wait_ns);
+                    mbar_wait(bar, parity, A.wait_ns);
                 }
-                ++done_iters;
+                phase ^= 1u << (it & 1);
                 // s_t of the next iteration is visible: written before the
                 // __syncthreads above
             } else {
