@@ -254,6 +254,9 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 // which a group of eight lanes issued for four vertices at a time), and ids
 // that arrive as 16-byte-aligned streams ahead of their use.
 //
+// In the compensated mode every term goes through a two-sum, as in the group
+// kernel (sixteen terms summed plainly before each had three times its error).
+//
 // CTAs come in clusters of 1, 2, 4 or 8. A graph that would keep one CTA busy
 // for longer than its share of the batch is taken by a whole cluster: every
 // CTA with slices holds the placement, computes a contiguous part of the slices
@@ -503,7 +506,6 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
 #pragma unroll
                     for (int x = 0; x < kBrAhead; ++x)
                         if (x < left) next[x] = ld_ids2(ids + 32 * (from + x));
-                    Acc<T, false> pend;
 #pragma unroll
                     for (int x = 0; x < kBrAhead; ++x) {
                         if (k0 + x >= steps) break;
@@ -512,27 +514,17 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                         const int e = 4 * (k0 + x);
                         if constexpr (sizeof(T) == 4 && MODEL == kFR) {
                             if (e < dmax) {  // the rows' first ids are their neighbours
-                                auto both = [&](auto& to) {
-                                    fr_entry(cur[i0], pu.x, pu.y, att.inv_d, e < deg, to, at);
-                                    fr_entry(cur[i1], pu.x, pu.y, att.inv_d, e + 1 < deg, to, at);
-                                    fr_entry(cur[i2], pu.x, pu.y, att.inv_d, e + 2 < deg, to, at);
-                                    fr_entry(cur[i3], pu.x, pu.y, att.inv_d, e + 3 < deg, to, at);
-                                };
-                                if constexpr (COMP) both(pend); else both(acc);
+                                fr_entry(cur[i0], pu.x, pu.y, att.inv_d, e < deg, acc, at);
+                                fr_entry(cur[i1], pu.x, pu.y, att.inv_d, e + 1 < deg, acc, at);
+                                fr_entry(cur[i2], pu.x, pu.y, att.inv_d, e + 2 < deg, acc, at);
+                                fr_entry(cur[i3], pu.x, pu.y, att.inv_d, e + 3 < deg, acc, at);
                                 continue;
                             }
                         }
-                        if constexpr (COMP) {
-                            f(i0, pend);
-                            f(i1, pend);
-                            f(i2, pend);
-                            f(i3, pend);
-                        } else {
-                            f(i0, acc);
-                            f(i1, acc);
-                            f(i2, acc);
-                            f(i3, acc);
-                        }
+                        f(i0, acc);
+                        f(i1, acc);
+                        f(i2, acc);
+                        f(i3, acc);
                         if (e < dmax) {
                             if (e < deg) att(i0, at);
                             if (e + 1 < deg) att(i1, at);
@@ -540,12 +532,8 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                             if (e + 3 < deg) att(i3, at);
                         }
                     }
-                    if constexpr (COMP) add_compensated(acc, pend.sx, pend.sy);
                 }
-                acc.sx *= d2;
-                acc.sy *= d2;
-                acc.cx *= d2;
-                acc.cy *= d2;
+                scale(acc, d2);
                 acc.merge(at.sx, at.sy, at.cx, at.cy);
                 T mx, my;
                 capped<T>(t, acc.fx(), acc.fy(), mx, my);

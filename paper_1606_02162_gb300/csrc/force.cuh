@@ -163,6 +163,23 @@ __device__ __forceinline__ void add_compensated(Acc<T, COMP>& acc, T x, T y)
     }
 }
 
+// acc *= f; in the compensated mode the rounding of the sum's product goes to
+// its error term.
+template <class T, bool COMP>
+__device__ __forceinline__ void scale(Acc<T, COMP>& acc, T f)
+{
+    if constexpr (COMP) {
+        const T x = acc.sx * f, y = acc.sy * f;
+        acc.cx = fma(acc.cx, f, fma(acc.sx, f, -x));
+        acc.cy = fma(acc.cy, f, fma(acc.sy, f, -y));
+        acc.sx = x;
+        acc.sy = y;
+    } else {
+        acc.sx *= f;
+        acc.sy *= f;
+    }
+}
+
 // Where a kernel reads positions from.
 enum Src {
     kSrcGlobal = 0,   // the whole placement in global memory, by ordinary loads: a kernel that
@@ -267,6 +284,10 @@ struct Rep {
             asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
             float c = rep_fr1(dx, dy);
             if (WEIGHTED) c *= wt[v];
+            if constexpr (C) {
+                add_compensated(a, c * dx, c * dy);
+                return;
+            }
             asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
             asm("mov.b64 %0, {%1, %2};" : "=l"(ac) : "f"(a.sx), "f"(a.sy));
             asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
@@ -377,10 +398,14 @@ __device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float in
     asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, 0x1p-100f));
     const float c = rcp_fast(r2);
-    asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ac) : "f"(rep.sx), "f"(rep.sy));
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(rep.sx), "=f"(rep.sy) : "l"(ac));
+    if constexpr (CR) {
+        add_compensated(rep, c * dx, c * dy);
+    } else {
+        asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(ac) : "f"(rep.sx), "f"(rep.sy));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(rep.sx), "=f"(rep.sy) : "l"(ac));
+    }
     if (edge) {
         const float s = -(r2 * rsqrt_fast(r2)) * inv_d;
         if constexpr (CA) {

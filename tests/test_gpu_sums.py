@@ -63,3 +63,31 @@ def test_staged_rows_fp64(pq, weighted):
         G.gila_layout_step(h.handle, G.params(k=1, d=1.1, p=p, q=q, precision=G.GILA_FP64), 0.4, x, y,
                            disp)
     assert np.abs(disp.cpu().numpy() - want).max() <= 1e-12 * np.abs(want).max()
+
+
+def wheel(near, ones, far):
+    """Vertex 0 at the origin; vertex 1, its only neighbour, joins it to all
+    the others, so that its k = 2 row is every other vertex. Along x, repulsion
+    1 / distance: `near` from vertex 1, 1 from each of `ones` vertices, and,
+    with `far`, -near from the last. All terms are powers of two."""
+    n = 2 + ones + (1 if far else 0)
+    g = I.csr_from_edges(n, [0] + [1] * (n - 2), [1] + list(range(2, n)))
+    pos = np.zeros((n, 2))
+    pos[1, 0] = -1.0 / near
+    pos[2:2 + ones, 0] = -1.0
+    if far:
+        pos[n - 1, 0] = 1.0 / near
+    return g, pos
+
+
+# 2^24 + 1 + ... + 1 - 2^24 in the compensated mode: every one is below the
+# last place of the plain sum, so that terms added plainly before the two-sum
+# lose them; with a two-sum per term the result is exact but for the
+# attraction (2^-48)
+@pytest.mark.parametrize("ones", [5, 14, 31, 60])
+def test_compensated_batch_sums_every_term(ones):
+    g, pos = wheel(2.0 ** 24, ones, True)
+    with G.Batch([g]) as b:
+        prm = G.params(k=2, iters=1, t0=1e9, precision=G.GILA_FP32_COMPENSATED)
+        out = G.gila_layout_batch_run(b.handle, prm, pos)
+    assert abs(out[0, 0] - ones) <= 1e-6 * ones
