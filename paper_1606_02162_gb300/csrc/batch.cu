@@ -256,6 +256,9 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 //
 // In the compensated mode every term goes through a two-sum, as in the group
 // kernel (sixteen terms summed plainly before each had three times its error).
+// In FP32 a row is added in four sums that are joined after sixteen ids, as many
+// partial sums as the group kernel's lanes keep: one sum over a row loses more
+// (a row of 2^24 and 63 ones loses 63 with one sum, 3 here, at 0.6% of the time).
 //
 // CTAs come in clusters of 1, 2, 4 or 8. A graph that would keep one CTA busy
 // for longer than its share of the batch is taken by a whole cluster: every
@@ -495,7 +498,10 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                 // the slice after this one: the warp's next, or its first
                 // again for the next iteration
                 const int2 sn = A.sdesc[s0 + (s + nwarps < cb ? s + nwarps : first)];
-                Acc<T, COMP> acc, at;
+                // FP32: four sums, one of each id of a step, added after sixteen ids
+                constexpr bool FOUR = sizeof(T) == 4 && !COMP;
+                constexpr int M = FOUR ? 3 : 0;
+                Acc<T, COMP> acc, at, part[M + 1];
                 for (int k0 = 0; k0 < steps || k0 == 0; k0 += kBrAhead) {
                     uint2 c4[kBrAhead];
 #pragma unroll
@@ -514,17 +520,17 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                         const int e = 4 * (k0 + x);
                         if constexpr (sizeof(T) == 4 && MODEL == kFR) {
                             if (e < dmax) {  // the rows' first ids are their neighbours
-                                fr_entry(cur[i0], pu.x, pu.y, att.inv_d, e < deg, acc, at);
-                                fr_entry(cur[i1], pu.x, pu.y, att.inv_d, e + 1 < deg, acc, at);
-                                fr_entry(cur[i2], pu.x, pu.y, att.inv_d, e + 2 < deg, acc, at);
-                                fr_entry(cur[i3], pu.x, pu.y, att.inv_d, e + 3 < deg, acc, at);
+                                fr_entry(cur[i0], pu.x, pu.y, att.inv_d, e < deg, part[0], at);
+                                fr_entry(cur[i1], pu.x, pu.y, att.inv_d, e + 1 < deg, part[1 & M], at);
+                                fr_entry(cur[i2], pu.x, pu.y, att.inv_d, e + 2 < deg, part[2 & M], at);
+                                fr_entry(cur[i3], pu.x, pu.y, att.inv_d, e + 3 < deg, part[3 & M], at);
                                 continue;
                             }
                         }
-                        f(i0, acc);
-                        f(i1, acc);
-                        f(i2, acc);
-                        f(i3, acc);
+                        f(i0, part[0]);
+                        f(i1, part[1 & M]);
+                        f(i2, part[2 & M]);
+                        f(i3, part[3 & M]);
                         if (e < dmax) {
                             if (e < deg) att(i0, at);
                             if (e + 1 < deg) att(i1, at);
@@ -532,7 +538,16 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                             if (e + 3 < deg) att(i3, at);
                         }
                     }
+                    if constexpr (FOUR) {
+                        part[0].merge(part[1].sx, part[1].sy, T(0), T(0));
+                        part[2].merge(part[3].sx, part[3].sy, T(0), T(0));
+                        part[0].merge(part[2].sx, part[2].sy, T(0), T(0));
+                        acc.merge(part[0].sx, part[0].sy, T(0), T(0));
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) part[i] = Acc<T, COMP>();
+                    }
                 }
+                if constexpr (!FOUR) acc = part[0];
                 scale(acc, d2);
                 acc.merge(at.sx, at.sy, at.cx, at.cy);
                 T mx, my;

@@ -91,3 +91,16 @@ def test_compensated_batch_sums_every_term(ones):
         prm = G.params(k=2, iters=1, t0=1e9, precision=G.GILA_FP32_COMPENSATED)
         out = G.gila_layout_batch_run(b.handle, prm, pos)
     assert abs(out[0, 0] - ones) <= 1e-6 * ones
+
+
+# 2^24 + 1 + ... + 1 in FP32: only ones added to the large term are lost. The
+# lanes of the group form (sixteen at rows of 25 to 64, eight at 9 to 24) add at
+# most four entries each, so that three ones are lost, and each of at most
+# seven joins of partial sums rounds a sum of at most 2^25 (unit 2) by 1
+@pytest.mark.parametrize("ones", [11, 22, 40, 61])
+def test_fp32_batch_keeps_partial_sums(ones):
+    g, pos = wheel(2.0 ** 24, ones, False)
+    with G.Batch([g]) as b:
+        prm = G.params(k=2, iters=1, t0=1e9, precision=G.GILA_FP32)
+        out = G.gila_layout_batch_run(b.handle, prm, pos)
+    assert abs(out[0, 0] - (2.0 ** 24 + ones)) <= 3 + 7
