@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                              : t0 * (double)A.iters / (double)A.iters);
         }
         __syncthreads();
-        Rep<T, MODEL, COMP, kSrcShared, true> f;
+        Rep<T, MODEL, COMP, kSrcShared, true, false, true> f;  // right at the smallest distances too
         f.d2 = T(1);
         f.q = A.q;
         Att<T, MODEL, COMP, kSrcShared> att;

@@ -251,16 +251,32 @@ struct PosSource {
     }
 };
 
+// 1 / r^2 at every distance whose square is a normal number (FP32 from 1.1e-19,
+// FP64 from 1.5e-154), and finite at distance 0, where it multiplies
+// dx = dy = 0: the pair adds nothing. FP64 bounds r^2 by its high word, off the
+// FP64 pipe.
+__device__ __forceinline__ float rcp_r2(float dx, float dy)
+{
+    return rcp_fast(fmaxf(fmaf(dx, dx, dy * dy), 0x1p-126f));
+}
+__device__ __forceinline__ double rcp_r2(double dx, double dy)
+{
+    const double r2 = fma(dx, dx, dy * dy);
+    const unsigned hi = (unsigned)__double2hiint(r2);
+    return rcp_newton(__hiloint2double((int)(hi > 0x00100000u ? hi : 0x00100000u), __double2loint(r2)));
+}
+
 // Repulsion of one k-hop entry v on u (Section 3.1 with the repelling set
 // of Section 4.5): adds c (x_u - x_v) with c = d^2 / delta^(q+1). For
 // Fruchterman-Reingold (q = 1) in FP32 that is d^2 * rsqrt(r^2)^2, or
 // rcp(r^2) unscaled: one MUFU, no divide. A pair at distance 0 adds nothing. With
 // UNSCALED the factor d^2 is left out (the caller multiplies the row's sum
-// by it once). With WEIGHTED the term is multiplied by wt[v], the repulsion
+// by it once). With NEAR the shared-memory forms take 1 / r^2 by rcp_r2,
+// otherwise by rep_fr1, one operation shorter in FP32. With WEIGHTED the term is multiplied by wt[v], the repulsion
 // weight of the repelling vertex (Section 4.6); wt is in shared memory where
 // the positions are.
 template <class T, int MODEL, bool COMP, int SRC = kSrcGlobal, bool UNSCALED = false,
-          bool WEIGHTED = false>
+          bool WEIGHTED = false, bool NEAR = false>
 struct Rep {
     using P2 = typename V2<T>::type;
     PosSource<T, SRC> src;
@@ -282,7 +298,7 @@ struct Rep {
             asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
             float dx, dy;
             asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
-            float c = rep_fr1(dx, dy);
+            float c = NEAR ? rcp_r2(dx, dy) : rep_fr1(dx, dy);
             if (WEIGHTED) c *= wt[v];
             if constexpr (C) {
                 add_compensated(a, c * dx, c * dy);
@@ -307,7 +323,7 @@ struct Rep {
         dy = yu - pv.y;
         T c;
         if (MODEL == kFR) {
-            c = UNSCALED ? rep_fr1(dx, dy) : rep_fr(d2, dx * dx + dy * dy);
+            c = !UNSCALED ? rep_fr(d2, dx * dx + dy * dy) : NEAR ? rcp_r2(dx, dy) : rep_fr1(dx, dy);
         } else {
             const T r2 = dx * dx + dy * dy;
             c = T(0);
@@ -342,13 +358,12 @@ struct Rep {
     {
         return rcp_fast(fmaf(dx, dx, fmaf(dy, dy, 0x1p-100f)));
     }
-    // FP64 likewise, with 2^-1000: no effect on an r^2 >= 2^-946, a finite
-    // factor at r^2 = 0, and no comparison (which takes the FP64 pipe, two
-    // lanes a clock per SM, like the ten operations that remain: 250 graphs
-    // of the batch 3.88 -> 3.68 ms)
+    // (no comparison in either width: it would take the FP64 pipe, two lanes a
+    // clock per SM, like the ten operations that remain; 250 graphs of the batch
+    // 3.88 -> 3.63 ms)
     __device__ __forceinline__ static double rep_fr1(double dx, double dy)
     {
-        return rcp_newton(fma(dx, dx, fma(dy, dy, 0x1p-1000)));
+        return rcp_r2(dx, dy);
     }
 };
 
@@ -382,8 +397,8 @@ struct Att {
 // A k-hop entry at pv that may be a neighbour as well (FP32,
 // Fruchterman-Reingold): the repulsion as Rep forms it, into `rep` without the
 // factor d^2, and with `edge` the attraction from the same difference and
-// r^2 (with the 2^-100, which keeps the square root finite at distance 0,
-// where it multiplies zero). One subtraction and one r^2 serve both: the mesh
+// r^2 (at least the smallest normal number, as in rcp_r2; at distance 0 the
+// square root multiplies zero). One subtraction and one r^2 serve both: the mesh
 // 1000 x 1000, k = 3, 33.1 -> 29.7 us an iteration, 500 graphs of the batch
 // 634 -> 583 us a pass.
 template <bool CR, bool CA>
@@ -396,7 +411,7 @@ __device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float in
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
     float dx, dy;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
-    const float r2 = fmaf(dx, dx, fmaf(dy, dy, 0x1p-100f));
+    const float r2 = fmaxf(fmaf(dx, dx, dy * dy), 0x1p-126f);
     const float c = rcp_fast(r2);
     if constexpr (CR) {
         add_compensated(rep, c * dx, c * dy);

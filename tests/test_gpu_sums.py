@@ -104,3 +104,57 @@ def test_fp32_batch_keeps_partial_sums(ones):
         prm = G.params(k=2, iters=1, t0=1e9, precision=G.GILA_FP32)
         out = G.gila_layout_batch_run(b.handle, prm, pos)
     assert abs(out[0, 0] - (2.0 ** 24 + ones)) <= 3 + 7
+
+
+# a whole batch drawn at a tiny scale: d and the distances scaled by 2^-e. FP32
+# squares stay normal numbers down to distances of 2^-63 and FP64 ones to
+# 2^-511. Scaled by a power of two a layout is the same layout, so that the
+# move is held to the FP32 and FP64 bounds of a move at scale 1 (FP32: the
+# approximate reciprocal and root keep their relative errors)
+@pytest.mark.parametrize("prec,e", [("FP32", 30), ("FP32", 45), ("FP32", 55), ("FP32_COMPENSATED", 55),
+                                    ("FP64", 300), ("FP64", 490)])
+def test_batch_at_small_distances(prec, e):
+    prec = getattr(G, "GILA_" + prec)
+    graphs = [I.grid(9, 13), I.tri_mesh(12, 12), I.random_tree(200, 3), I.erdos_renyi(700, 4.0, 5)]
+    pos = [I.uniform_positions(g.n, 80 + i).astype(np.float32).astype(np.float64)
+           for i, g in enumerate(graphs)]
+    s = 2.0 ** -e
+    prm = G.params(k=2, iters=1, d=s, t0=s, precision=prec)
+    with G.Batch(graphs) as b:
+        out = G.gila_layout_batch_run(b.handle, prm, s * np.concatenate(pos)) / s
+    at = 0
+    for g, x in zip(graphs, pos):
+        krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 2)
+        _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, x, 1.0)
+        got = out[at:at + g.n] - x
+        at += g.n
+        slack = 4 * np.finfo(np.float32).eps * np.abs(x).max() if prec != G.GILA_FP64 else 0.0
+        tol = 1e-12 if prec == G.GILA_FP64 else 1e-4
+        assert np.abs(got - want).max() <= tol * np.abs(want).max() + slack, g.name
+
+
+# the same for the single-graph kernels that keep to it: every FP64 form, and
+# the FP32 row-per-lane form where all of a row's ids are its neighbours
+@pytest.mark.parametrize("prec,e,k,tune,kernel", [
+    ("FP64", 490, 2, dict(tiled=1), "row per lane"), ("FP64", 490, 2, dict(tiled=1, tile_vertices=100), "blocked"),
+    ("FP64", 490, 2, dict(tiled=0), "iteration"), ("FP32", 55, 1, dict(tiled=1), "row per lane"),
+    ("FP32", 55, 2, dict(tiled=0), "iteration"), ("FP32_COMPENSATED", 55, 1, dict(tiled=1), "row per lane"),
+])
+def test_step_at_small_distances(prec, e, k, tune, kernel):
+    import torch
+    prec = getattr(G, "GILA_" + prec)
+    g = I.grid(40, 41)
+    pos = I.uniform_positions(g.n, 90).astype(np.float32).astype(np.float64)
+    s = 2.0 ** -e
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, k)
+    _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, 1.0)
+    x = torch.tensor(s * pos, dtype=torch.float64 if prec == G.GILA_FP64 else torch.float32, device="cuda")
+    y, disp = torch.empty_like(x), torch.empty_like(x)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, **tune)
+        G.gila_profile_enable(h.handle, 2)
+        G.gila_layout_step(h.handle, G.params(k=k, d=s, precision=prec), s, x, y, disp)
+        torch.cuda.synchronize()
+        assert kernel in G.gila_profile_read_kernel(h.handle)["name"]
+    tol = 1e-12 if prec == G.GILA_FP64 else 1e-4
+    assert np.abs(disp.double().cpu().numpy() / s - want).max() <= tol * np.abs(want).max()
