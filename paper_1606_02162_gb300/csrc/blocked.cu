@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
                          (wbytes - o < kBulkChunk) ? wbytes - o : kBulkChunk, &tile_bar);
             T* w = reinterpret_cast<T*>(wdst);
             for (int64_t i = wbytes / sizeof(T); i < tn; ++i) w[i] = wsrc[i];
-            w[A.tv] = T(1);  // the padding's
+            w[A.tv] = T(0);  // the padding's
         }
         if ((size_t)tn * sizeof(P2) != bytes) tile[tn - 1] = pos[tb + tn - 1];
         P2 far;  // the padding's slot, outside the copied range
@@ -278,12 +278,14 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
     mbar_wait(&tile_bar, 0, A.wait_ns);  // completed: acquires the tile for this thread
 
     if (L > 0) {
-        // d^2 is applied when the partials are added
-        Rep<T, MODEL, COMP, kSrcShared, true, W> f;
+        // d^2 is applied when the partials are added, with weights to each
+        // term (the plain kernel's form: a weight's product with an unscaled
+        // 1 / r^2 overflows earlier)
+        Rep<T, MODEL, COMP, kSrcShared, !W, W> f;
         f.src.set_shared(tile, 0u);  // ids are relative to the tile
         if constexpr (W)
             f.wt = reinterpret_cast<const T*>(smem_raw + weights_at(A.tv, A.rmax, sizeof(P2)));
-        f.d2 = T(1);
+        f.d2 = W ? const_d2<T>(A.c) : T(1);
         f.q = A.q;
         // this thread's entries [a, b) (a < L), their storage, and the row of a
         const int32_t a = lane_start(L, threadIdx.x), b = lane_start(L, threadIdx.x + 1);
@@ -2806,6 +2808,7 @@ gila_status launch_blocked(gila_graph* g, const gila_params* prm, double t, cons
     C.n = g->n;
     C.nt = P.nt;
     C.c = B.c;
+    if (B.wt) C.c.d2 = C.c.d2f = 1;  // in the weighted terms already
     C.p = prm->p;
     C.pos_in = pos_in;
     C.part = P.part;

@@ -266,6 +266,25 @@ __device__ __forceinline__ double rcp_r2(double dx, double dy)
     return rcp_newton(__hiloint2double((int)(hi > 0x00100000u ? hi : 0x00100000u), __double2loint(r2)));
 }
 
+// d^2 / r^2, and 0 at distance 0: what a weight of any size is multiplied by
+// (a factor that is only finite there, 2^126 or 2^1022, overflows under a weight,
+// and inf times dx = 0 is NaN). FP64: r^2 is bounded by its high word on both
+// sides, off the FP64 pipe, so that a distance whose square overflows (the
+// padding's, from a vertex beyond 1e154) gives 0 as well.
+__device__ __forceinline__ float rep_scaled(float d2, float dx, float dy)
+{
+    const float r2 = fmaf(dx, dx, dy * dy);
+    return r2 > 0.0f ? d2 * rcp_fast(r2) : 0.0f;
+}
+__device__ __forceinline__ double rep_scaled(double d2, double dx, double dy)
+{
+    const double r2 = fma(dx, dx, dy * dy);
+    const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
+    const unsigned h1 = hi > 0x00100000u ? hi : 0x00100000u;
+    const double c = d2 * rcp_newton(__hiloint2double((int)(h1 < 0x7fdfffffu ? h1 : 0x7fdfffffu), (int)lo));
+    return (hi | lo) != 0 ? c : 0.0;
+}
+
 // Repulsion of one k-hop entry v on u (Section 3.1 with the repelling set
 // of Section 4.5): adds c (x_u - x_v) with c = d^2 / delta^(q+1). For
 // Fruchterman-Reingold (q = 1) in FP32 that is d^2 * rsqrt(r^2)^2, or
@@ -287,7 +306,7 @@ struct Rep {
     template <bool C = COMP>
     __device__ __forceinline__ void operator()(uint32_t v, Acc<T, C>& a) const
     {
-        if constexpr (sizeof(T) == 4 && MODEL == kFR && UNSCALED && SRC == kSrcShared) {
+        if constexpr (sizeof(T) == 4 && MODEL == kFR && (UNSCALED || WEIGHTED) && SRC == kSrcShared) {
             // the blocked kernel's FP32 term with packed two-lane FP32
             // arithmetic (sm_100 and later): one subtraction forms
             // (dx, dy) and one fused multiply-add accumulates c (dx, dy)
@@ -298,8 +317,9 @@ struct Rep {
             asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
             float dx, dy;
             asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
-            float c = NEAR ? rcp_r2(dx, dy) : rep_fr1(dx, dy);
-            if (WEIGHTED) c *= wt[v];
+            float c;
+            if (WEIGHTED) c = rep_scaled(d2, dx, dy) * wt[v];
+            else c = NEAR ? rcp_r2(dx, dy) : rep_fr1(dx, dy);
             if constexpr (C) {
                 add_compensated(a, c * dx, c * dy);
                 return;
@@ -322,7 +342,9 @@ struct Rep {
         dx = xu - pv.x;
         dy = yu - pv.y;
         T c;
-        if (MODEL == kFR) {
+        if (MODEL == kFR && WEIGHTED && SRC == kSrcShared) {
+            c = rep_scaled(d2, dx, dy);
+        } else if (MODEL == kFR) {
             c = !UNSCALED ? rep_fr(d2, dx * dx + dy * dy) : NEAR ? rcp_r2(dx, dy) : rep_fr1(dx, dy);
         } else {
             const T r2 = dx * dx + dy * dy;

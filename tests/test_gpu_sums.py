@@ -158,3 +158,30 @@ def test_step_at_small_distances(prec, e, k, tune, kernel):
         assert kernel in G.gila_profile_read_kernel(h.handle)["name"]
     tol = 1e-12 if prec == G.GILA_FP64 else 1e-4
     assert np.abs(disp.double().cpu().numpy() / s - want).max() <= tol * np.abs(want).max()
+
+
+# large weights: vertices at one place exert nothing on each other whatever
+# they weigh, and with d and the distances scaled by 2^-e the layout is the
+# same layout
+@pytest.mark.parametrize("prec,big,e", [("FP32", 1e9, 0), ("FP32_COMPENSATED", 1e9, 0), ("FP64", 1e8, 0),
+                                        ("FP32", 1e9, 50), ("FP64", 1e9, 480)])
+@pytest.mark.parametrize("tiled", [0, 1])
+def test_large_weights(prec, big, e, tiled):
+    import torch
+    prec = getattr(G, "GILA_" + prec)
+    g = I.barabasi_albert(700, 2, 8)
+    pos = I.uniform_positions(g.n, 95).astype(np.float32).astype(np.float64)
+    pos[1::9] = pos[::9][:pos[1::9].shape[0]]  # pairs at one place
+    w = np.where(np.arange(g.n) % 3 == 0, big, 1.0)
+    krow, kcol = O.khop(g.n, g.row_ptr, g.col_idx, 2)
+    _, want = O.step(g.n, g.row_ptr, g.col_idx, krow, kcol, pos, 1.0, wt=w)
+    s = 2.0 ** -e
+    x = torch.tensor(s * pos, dtype=torch.float64 if prec == G.GILA_FP64 else torch.float32, device="cuda")
+    y, disp = torch.empty_like(x), torch.empty_like(x)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, **(dict(tiled=1, tile_vertices=100) if tiled else dict(tiled=0)))
+        G.gila_graph_set_repulsion_weights(h.handle, w)
+        G.gila_layout_step(h.handle, G.params(k=2, d=s, precision=prec), s, x, y, disp)
+    got = disp.double().cpu().numpy() / s
+    tol = 1e-12 if prec == G.GILA_FP64 else 1e-4
+    assert np.abs(got - want).max() <= tol * np.abs(want).max()
