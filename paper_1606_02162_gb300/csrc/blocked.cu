@@ -319,10 +319,13 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
         Acc<T, COMP> acc, first;
         // compensated mode: the terms of the steps since the last merge,
         // summed plainly; added to acc with its error term at the end of
-        // each ring of steps and before a row closes
+        // each ring of steps and before a row closes. With weights every term
+        // goes through a two-sum, as in the plain kernel, which these graphs
+        // took before
         Acc<T, false> pend;
+        constexpr bool PEND = COMP && !W;
         auto merge_pending = [&]() {
-            if (COMP) {
+            if (PEND) {
                 add_compensated(acc, pend.sx, pend.sy);
                 pend = Acc<T, false>();
             }
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs
         int32_t lim = (re < b) ? re : b;
         int32_t p = a;
         auto eight = [&](const uint4 c) {
-            if (COMP) {
+            if (PEND) {
                 // compensated mode: into the plain pending sum
                 f(c.x & 0xffffu, pend);
                 f(c.x >> 16, pend);

@@ -185,3 +185,19 @@ def test_large_weights(prec, big, e, tiled):
     got = disp.double().cpu().numpy() / s
     tol = 1e-12 if prec == G.GILA_FP64 else 1e-4
     assert np.abs(got - want).max() <= tol * np.abs(want).max()
+
+
+# the compensated wheel on weighted tiles (weights 1, all of a row in one
+# tile): a two-sum per term, as in the plain kernel
+@pytest.mark.parametrize("ones", [5, 14, 31, 60, 200])
+@pytest.mark.parametrize("tiled", [0, 1])
+def test_compensated_weighted_tiles_sum_every_term(ones, tiled):
+    import torch
+    g, pos = wheel(2.0 ** 24, ones, True)
+    x = torch.tensor(pos, dtype=torch.float32, device="cuda")
+    y, disp = torch.empty_like(x), torch.empty_like(x)
+    with G.Graph.from_inputs(g) as h:
+        G.gila_graph_tune(h.handle, tiled=tiled)
+        G.gila_graph_set_repulsion_weights(h.handle, np.ones(g.n))
+        G.gila_layout_step(h.handle, G.params(k=2, precision=G.GILA_FP32_COMPENSATED), 1e9, x, y, disp)
+    assert abs(float(disp[0, 0]) - ones) <= 1e-6 * ones
