@@ -265,7 +265,8 @@ typedef struct gila_batch gila_batch;
 
 typedef struct gila_batch_tuning {
     int32_t threads;     /* threads per CTA: 256, 512 or 1024; 0 = 512 */
-    int32_t ctas_per_sm; /* CTAs per SM (1..8); 0 = 2 when two graphs fit in shared memory */
+    int32_t ctas_per_sm; /* CTAs per SM (1..8); 0: rows per lane as many as threads and shared
+                            memory allow, groups 2 when two graphs fit in shared memory */
     /* all three 0 (default): graphs of short rows (mean at most 64) take a lane
        per vertex, the others the groups below; any of them set: every graph
        takes groups */
@@ -295,8 +296,11 @@ gila_status gila_batch_khop_reset(gila_batch* b);
  * its entries are numbered the same way (a graph's lists stay inside its
  * own id range). GILA_ESTATE when no lists are built. */
 gila_status gila_batch_khop_export(const gila_batch* b, int64_t* krow_host, int32_t* kcol_host);
-/* Set (or read back, defaults filled in for a precision) the launch shape
- * and lanes-per-vertex thresholds of the batched kernel. */
+/* Set (or read back) the launch shape and lanes-per-vertex thresholds of the
+ * batched kernel. What is left to the library reads back as 0 (ctas_per_sm, and
+ * the group fields while all three are 0; where one is set the others read back
+ * with their defaults), for every precision, so that setting a tuning that was
+ * read back, here or by gila_batch_autotune, changes nothing. */
 gila_status gila_batch_tune(gila_batch* b, const gila_batch_tuning* t);
 gila_status gila_batch_get_tuning(const gila_batch* b, int32_t precision, gila_batch_tuning* out);
 /* Time candidate tunings on this batch (probe_iters iterations each, from

@@ -788,7 +788,29 @@ __global__ void pack_kernel(const PackSrc* __restrict__ src, int64_t* __restrict
         col[s.eoff + i] = (int32_t)(s.voff + s.col[s.row[0] + i]);
 }
 
-gila_batch_tuning resolved(const gila_batch* b, size_t esz, int sms)
+// Whether the tuning asks for lane groups on every graph.
+bool wants_groups(const gila_batch_tuning& t)
+{
+    return t.group4_max > 0 || t.group8_max > 0 || t.group16_max > 0;
+}
+
+// The tuning as a caller reads it back: what it leaves to the library stays 0
+// (filled in, the lane groups would ask for the group kernel on every graph), so
+// that setting it again changes nothing.
+gila_batch_tuning reported(const gila_batch_tuning& set)
+{
+    gila_batch_tuning t = set;
+    if (t.threads == 0) t.threads = 512;
+    if (wants_groups(t)) {
+        if (t.group4_max <= 0) t.group4_max = 8;
+        if (t.group8_max <= 0) t.group8_max = 24;
+        if (t.group16_max <= 0) t.group16_max = 64;
+    }
+    return t;
+}
+
+// The tuning that the group kernel runs with.
+gila_batch_tuning resolved(const gila_batch* b, size_t esz)
 {
     gila_batch_tuning t = b->tune;
     if (t.threads != 256 && t.threads != 512 && t.threads != 1024) t.threads = 512;
@@ -802,7 +824,6 @@ gila_batch_tuning resolved(const gila_batch* b, size_t esz, int sms)
         t.ctas_per_sm = (need * 2 <= smem_cap) ? 2 : 1;
     }
     t.ctas_per_sm = std::max(1, std::min(t.ctas_per_sm, 2048 / t.threads));
-    (void)sms;
     return t;
 }
 
@@ -1109,10 +1130,10 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
     if (s != GILA_OK && s != GILA_ENOMEM) return s;
     const bool planned = s == GILA_OK;
     const int sms = sm_count(g->device);
-    const gila_batch_tuning tu = resolved(b, esz, sms);
+    const gila_batch_tuning tu = resolved(b, esz);
     // lane groups set by the tuning ask for the group kernel on every graph
     const int w = esz == 16 ? 1 : 0;
-    const bool groups = !planned || b->tune.group4_max > 0 || b->tune.group8_max > 0 || b->tune.group16_max > 0;
+    const bool groups = !planned || wants_groups(b->tune);
     const int nbig = groups ? 0 : (int)b->big[w].size();
     const int nrows = groups ? 0 : nbig + (int)b->small[w].size();
     const int nrest = b->count - nrows;
@@ -1376,7 +1397,8 @@ gila_status gila_batch_tune(gila_batch* b, const gila_batch_tuning* t)
 gila_status gila_batch_get_tuning(const gila_batch* b, int32_t precision, gila_batch_tuning* out)
 {
     if (!b || !out) return fail(GILA_EINVAL, "batch or out is NULL");
-    *out = resolved(b, is_f64(precision) ? 16 : 8, sm_count(b->g->device));
+    (void)precision;
+    *out = reported(b->tune);
     return GILA_OK;
 }
 
@@ -1441,7 +1463,7 @@ gila_status gila_batch_autotune(gila_batch* b, const gila_params* prm, const voi
     cudaEventDestroy(e1);
     b->tune = (s == GILA_OK) ? best : saved;
     if (s != GILA_OK) return s;
-    if (chosen) *chosen = resolved(b, esz, sm_count(g->device));
+    if (chosen) *chosen = reported(b->tune);
     return GILA_OK;
 }
 
