@@ -253,8 +253,10 @@ gila_status gila_layout_metrics(gila_graph* g, const gila_params* prm, const voi
  * carries it through all iterations with its placement staged in shared
  * memory. The launch is captured in a CUDA graph and replayed while the
  * arguments stay the same. CTAs of a cluster bound their waits for each
- * other's positions; one that gives up is reported as GILA_ECUDA by the next
- * gila_layout_batch_run in the process. Every graph follows its own temperature schedule
+ * other's positions; one that gives up leaves its graphs' placements incomplete
+ * and is reported as GILA_ECUDA, by gila_layout_batch_run at its end, or after
+ * gila_layout_batch_device by the next call that lays out or tunes the same batch
+ * once the launch has ended. Every graph follows its own temperature schedule
  * (default t0 from its own n and initial bounding box). A graph's result
  * depends only on the graph, its placement, the parameters and the batch
  * tuning, not on the other graphs of the batch. Precisions: GILA_FP32,
@@ -476,6 +478,11 @@ gila_status gila_layout_components_run(gila_graph* g, const gila_params* prm, do
  * in flight and the CUDA context stays usable; turn it off (0) to resume
  * normal iterations. For tests only. */
 gila_status gila_graph_set_wait_test(gila_graph* g, int32_t on);
+
+/* The same for batches: while on (1), CTAs of a cluster announce each other's
+ * positions but push none, so that their waits run out after 1 ms and the launch
+ * ends; graphs that a single CTA takes are laid out as always. For tests only. */
+gila_status gila_batch_set_wait_test(gila_batch* b, int32_t on);
 
 /* Temperature of iteration i under prm (t0 = resolved initial temperature). */
 double gila_temperature(const gila_params* prm, double t0, int32_t i);

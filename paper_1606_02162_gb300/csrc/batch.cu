@@ -69,6 +69,8 @@ struct gila_batch {
     uint16_t* cuts = nullptr;
     uint16_t* tk = nullptr;
     size_t tk_cap = 0;
+    int* wait_failed = nullptr;    // host memory the kernel writes: a cluster's wait ran out
+    int wait_test = 0;             // test hook: clusters push nothing, so that their waits run out
     cudaStream_t side = nullptr;   // capture fork: the group kernel beside the row-per-lane one
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
@@ -291,11 +293,8 @@ constexpr int kBrSmem = 227 * 1024 - 2048;
 // fewest slices worth a cluster: below, an exchange an iteration costs more
 // than the split saves (FP64 slices take about ten times as long)
 constexpr int64_t kBrBigSlices[2] = {16, 4};
-constexpr uint64_t kBrWaitNs = 1000000000ull;  // bound on a wait for peers' positions
-
-// Set when a wait for peers' positions ran out; read and cleared by the next
-// synchronising batch call.
-__device__ int g_batch_wait_failed = 0;
+constexpr uint64_t kBrWaitNs = 1000000000ull;    // bound on a wait for peers' positions
+constexpr uint64_t kBrTestWaitNs = 1000000ull;   // ... while the wait test hook is on
 
 struct BatchRowsArgs {
     const int64_t* voff;
@@ -316,6 +315,8 @@ struct BatchRowsArgs {
     void* pos;
     int stride;              // positions per buffer, far slot included (even)
     uint64_t wait_ns;
+    int skip_push;           // test hook: announce the peers' positions but push none
+    int* wait_failed;        // the batch's, in host memory: set when a wait ran out
 };
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
         mbar_init(&s_bar[1], 1);
     }
     uint32_t phase = 0;  // bit i: parity of the phase of s_bar[i] that this CTA waits for next
-    bool failed = false;
+    bool gave_up = false;  // a wait of this thread ran out
 
     // one graph, its slices [s0 + ca, s0 + cb) on this CTA
     auto layout = [&](int gid, bool big) {
@@ -561,25 +562,27 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
             if (big) {
                 // push this CTA's new positions to its peers and wait for theirs
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncthreads();
+                // once a thread of the CTA has given up, the CTA neither
+                // announces, pushes nor waits any more
+                const bool failed = __syncthreads_or(gave_up) != 0;
                 uint64_t* bar = &s_bar[it & 1];
                 const uint32_t parity = (phase >> (it & 1)) & 1;
                 const uint32_t mine = (uint32_t)(cb - ca) * 32u * (uint32_t)sizeof(P2);
-                if (threadIdx.x == 0)
-                    mbar_arrive_expect_tx(bar, (uint32_t)npad * (uint32_t)sizeof(P2) - mine);
                 if (threadIdx.x == 0 && !failed) {
+                    mbar_arrive_expect_tx(bar, (uint32_t)npad * (uint32_t)sizeof(P2) - mine);
                     const uint32_t src = smem_addr(nxt + ca * 32), b = smem_addr(bar);
-                    for (uint32_t r = 1; r < csize; ++r) {
+                    for (uint32_t r = 1; r < csize && !A.skip_push; ++r) {
                         const uint32_t to = (rank + r) & (csize - 1);
                         if ((peers >> to) & 1)
                             bulk_s2s(cluster_map(src, to), src, mine, cluster_map(b, to));
                     }
                 }
                 if (!failed && !mbar_wait(bar, parity, A.wait_ns)) {
-                    // give up: flag it, let what is in flight land (bounded),
-                    // push and wait no more; the cluster leaves together
-                    failed = true;
-                    atomicExch(&g_batch_wait_failed, 1);
+                    // give up: flag it, let what is in flight land (bounded);
+                    // the cluster leaves together
+                    gave_up = true;
+                    *(volatile int*)A.wait_failed = 1;
+                    __threadfence_system();
                     mbar_wait(bar, parity, A.wait_ns);
                 }
                 phase ^= 1u << (it & 1);
@@ -913,6 +916,8 @@ gila_status batch_finish_create(gila_batch* b)
     if (count > 0)
         GILA_CUDA(cudaMemcpy(b->order, order.data(), sizeof(int32_t) * count,
                              cudaMemcpyHostToDevice));
+    GILA_CUDA(cudaHostAlloc((void**)&b->wait_failed, sizeof(int), cudaHostAllocMapped));
+    *b->wait_failed = 0;
     GILA_CUDA(cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking));
     GILA_CUDA(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
     GILA_CUDA(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
@@ -1093,19 +1098,13 @@ gila_status batch_plan(gila_batch* b)
     return GILA_OK;
 }
 
-// GILA_ECUDA (and clears the flag) when a cluster gave up waiting for its
-// peers' positions since the last call; synchronises st.
-gila_status batch_wait_failed(cudaStream_t st)
+// GILA_ECUDA (and clears the flag) when a cluster of a launch of this batch
+// gave up waiting for its peers' positions since the last call. Does not
+// synchronise: launches that have not ended are told of by a later call.
+gila_status batch_wait_failed(gila_batch* b)
 {
-    int h = 0;
-    const int zero = 0;
-    GILA_CUDA(cudaMemcpyFromSymbolAsync(&h, g_batch_wait_failed, sizeof(int), 0,
-                                        cudaMemcpyDeviceToHost, st));
-    GILA_CUDA(cudaStreamSynchronize(st));
-    if (!h) return GILA_OK;
-    GILA_CUDA(cudaMemcpyToSymbolAsync(g_batch_wait_failed, &zero, sizeof(int), 0,
-                                      cudaMemcpyHostToDevice, st));
-    GILA_CUDA(cudaStreamSynchronize(st));
+    if (!*(volatile int*)b->wait_failed) return GILA_OK;
+    *(volatile int*)b->wait_failed = 0;
     return fail(GILA_ECUDA, "a cluster of the batch kernel did not receive its positions in time");
 }
 
@@ -1115,8 +1114,9 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
 {
     gila_graph* g = b->g;
     const size_t esz = is_f64(prm->precision) ? 16 : 8;
+    gila_status s = batch_wait_failed(b);  // of an earlier launch
+    if (s != GILA_OK) return s;
     if (b->count == 0 || g->n == 0 || prm->iters == 0) return GILA_OK;
-    gila_status s;
     if (prm->schedule == GILA_COOL_GEOMETRIC) {
         s = ensure((void**)&b->geo, &b->geo_cap, sizeof(double) * (size_t)prm->iters);
         if (s != GILA_OK) return s;
@@ -1193,7 +1193,9 @@ gila_status batch_run(gila_batch* b, const gila_params* prm, void* pos)
     R.q = prm->q;
     R.pos = pos;
     R.stride = (int)((b->max_rows_n[w] + 31) / 32 * 32 + 2);
-    R.wait_ns = kBrWaitNs;
+    R.wait_ns = b->wait_test ? kBrTestWaitNs : kBrWaitNs;
+    R.skip_push = b->wait_test;
+    R.wait_failed = b->wait_failed;
     const size_t rsmem = 2 * (size_t)R.stride * esz;
     // as many CTAs per SM as the tuning and the buffers allow, in clusters
     const int64_t fit = std::max<int64_t>(1, (kBrSmem + 2048) / (int64_t)(rsmem + 2048));
@@ -1341,6 +1343,7 @@ void gila_batch_destroy(gila_batch* b)
                     (void*)b->base, (void*)b->units, (void*)b->skip, (void*)b->sdesc,
                     (void*)b->deg, (void*)b->perm, (void*)b->rank, (void*)b->cuts, (void*)b->tk})
         cudaFree(p);
+    if (b->wait_failed) cudaFreeHost(b->wait_failed);
     cudaFree(b->tmp);
     cudaFree(b->pos[0]);
     cudaFree(b->pos[1]);
@@ -1354,6 +1357,13 @@ gila_status gila_batch_set_stream(gila_batch* b, void* cuda_stream)
     if (!b) return fail(GILA_EINVAL, "batch is NULL");
     b->user = (cudaStream_t)cuda_stream;
     return gila_graph_set_stream(b->g, cuda_stream);
+}
+
+gila_status gila_batch_set_wait_test(gila_batch* b, int32_t on)
+{
+    if (!b) return fail(GILA_EINVAL, "batch is NULL");
+    b->wait_test = on ? 1 : 0;
+    return GILA_OK;
 }
 
 gila_status gila_batch_info(const gila_batch* b, int32_t* count, int64_t* total_n,
@@ -1453,6 +1463,7 @@ gila_status gila_batch_autotune(gila_batch* b, const gila_params* prm, const voi
                     s = cuda_fail(e, "autotune timing");
                     break;
                 }
+                if ((s = batch_wait_failed(b)) != GILA_OK) break;
                 if (ms < best_ms) {
                     best_ms = ms;
                     best = c;
@@ -1512,7 +1523,7 @@ gila_status gila_layout_batch_run(gila_batch* b, const gila_params* prm, const d
         GILA_CUDA(cudaMemcpyAsync(pos_out_host, b->stage, 16 * n, cudaMemcpyDeviceToHost, b->user));
     }
     GILA_CUDA(cudaStreamSynchronize(b->user));
-    return batch_wait_failed(b->user);
+    return batch_wait_failed(b);
 }
 
 gila_status gila_layout_batch(gila_graph* const* gs, int32_t count, const gila_params* prm,

@@ -132,6 +132,7 @@ SIGNATURES = [
     ("gila_layout_pruned_run", ctypes.c_int, [P, PP, P, P]),
     ("gila_graph_components", ctypes.c_int, [P, P, ctypes.POINTER(I32)]),
     ("gila_graph_set_wait_test", ctypes.c_int, [P, I32]),
+    ("gila_batch_set_wait_test", ctypes.c_int, [P, I32]),
     ("gila_layout_components_run", ctypes.c_int, [P, PP, D, P, P, ctypes.POINTER(I32)]),
 ]
 
@@ -728,3 +729,8 @@ def gila_layout_components_run(g, prm, pos_in, gap=0.0, pos_out=None):
 def gila_graph_set_wait_test(g, on) -> None:
     """Failure-detection test hook (see include/gila.h)."""
     _check(load().gila_graph_set_wait_test(g, 1 if on else 0))
+
+
+def gila_batch_set_wait_test(b, on) -> None:
+    """Test hook: clusters push no positions, so that their waits run out."""
+    _check(load().gila_batch_set_wait_test(b, 1 if on else 0))
