@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 // time (once per k-hop build) each graph's vertices are sorted by row length,
 // and 32 consecutive ones of that order form a slice, stored step-major (four
 // 16-bit ids of every lane, 256 bytes a step) and padded to the slice's
-// longest row with the id of a far slot. A row's first ids are its neighbours,
+// longest row with the row's own id (at distance 0, where a term is zero,
+// whatever the coordinates). A row's first ids are its neighbours,
 // whose attraction is formed from the same shared-memory positions. A lane
 // sums its row in registers and moves its vertex: no reduction over lanes, no
 // lane without a row in the finish (a square root and a division per vertex,
@@ -553,9 +554,10 @@ __global__ void __launch_bounds__(1024) batch_rows_kernel(const BatchRowsArgs A)
                 acc.merge(at.sx, at.sy, at.cx, at.cy);
                 T mx, my;
                 capped<T>(t, acc.fx(), acc.fy(), mx, my);
+                // (padding is all an isolated vertex has: 0 at a finite place)
                 P2 o;
-                o.x = pu.x + mx;
-                o.y = pu.y + my;
+                o.x = deg > 0 ? pu.x + mx : pu.x;
+                o.y = deg > 0 ? pu.y + my : pu.y;
                 nxt[i] = o;
                 sd = sn;
             }
@@ -711,7 +713,8 @@ batch_sort_kernel(const int64_t* __restrict__ voff, const int32_t* __restrict__ 
 
 // Plan, a warp per slice and a row per lane: the slice's start becomes its
 // place in tk, and its ids are written, neighbours first (both lists
-// ascending, one merge), then the rest, then the far slot's id. A row whose
+// ascending, one merge), then the rest, then its own as padding (the far slot's
+// in lanes without a row). A row whose
 // neighbours are not all among its k-hop ids (an unsorted or repeated
 // adjacency, a self-loop) sets bad[g]: the graph keeps the group kernel.
 __global__ void __launch_bounds__(128)
@@ -771,7 +774,7 @@ batch_fill_kernel(int64_t nslices, const int32_t* __restrict__ sgraph,
         else put(rank[id]);
     }
     if (found != deg) bad[g] = 1;
-    while (w < slots) put((uint32_t)npad);
+    while (w < slots) put((uint32_t)(i < n ? i : npad));
 }
 
 // Pack graphs given as device CSRs into the union CSR (one block per graph).

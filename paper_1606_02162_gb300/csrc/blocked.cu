@@ -887,8 +887,9 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 2 : 1) rows_kern
             acc.cx *= d2;
             acc.cy *= d2;
             acc.merge(at.sx, at.sy, at.cx, at.cy);
-            apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u, pu.x, pu.y, acc.fx(),
-                          acc.fy());
+            // (an isolated vertex has padding only: zeros at a finite place)
+            apply_move<T>(const_t<T>(A.c), A.pos_out, A.disp_out, u, pu.x, pu.y,
+                          deg > 0 ? acc.fx() : T(0), deg > 0 ? acc.fy() : T(0));
         }
         sd = sn;
     }

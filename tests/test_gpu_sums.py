@@ -201,3 +201,42 @@ def test_compensated_weighted_tiles_sum_every_term(ones, tiled):
         G.gila_graph_set_repulsion_weights(h.handle, np.ones(g.n))
         G.gila_layout_step(h.handle, G.params(k=2, precision=G.GILA_FP32_COMPENSATED), 1e9, x, y, disp)
     assert abs(float(disp[0, 0]) - ones) <= 1e-6 * ones
+
+
+# vertices without edges feel no force wherever they are: at infinity too, in
+# a slice beside longer rows
+@pytest.mark.parametrize("prec", [G.GILA_FP32, G.GILA_FP32_COMPENSATED, G.GILA_FP64],
+                         ids=["fp32", "fp32c", "fp64"])
+def test_isolated_vertices_at_infinity(prec):
+    import torch
+    g = I.csr_from_edges(70, np.arange(40), np.arange(1, 41))  # a path, 29 isolated vertices
+    pos = I.uniform_positions(g.n, 13)
+    pos[50], pos[51], pos[69] = (np.inf, 0.0), (3e38, -np.inf), (-3e38, 3e38)
+    if prec == G.GILA_FP64:
+        pos[69] = (1e300, -1e300)
+    dt = torch.float64 if prec == G.GILA_FP64 else torch.float32
+    x = torch.tensor(pos, dtype=dt, device="cuda")
+    with G.Batch([g]) as b:
+        y = x.clone()
+        G.gila_layout_batch_device(b.handle, G.params(k=2, iters=3, t0=0.5, precision=prec), y)
+    for tiled in (0, 1):
+        with G.Graph.from_inputs(g) as h:
+            G.gila_graph_tune(h.handle, tiled=tiled)
+            z = x.clone()
+            G.gila_layout_run_device(h.handle, G.params(k=2, iters=3, t0=0.5, precision=prec), z)
+        assert torch.equal(z[41:], x[41:]) and bool(torch.isfinite(z[:41]).all())
+    assert torch.equal(y[41:], x[41:]) and bool(torch.isfinite(y[:41]).all())
+
+
+def test_fp64_batch_far_from_the_origin():
+    """Coordinates of 2^533, whose squares overflow, distances of 2^500, whose
+    squares do not: the layout at the origin, to the coordinates' last place
+    (2^-19 of a unit), which padding far from all vertices turned into NaN."""
+    g = I.erdos_renyi(300, 4.0, 6)
+    pos = np.round(I.uniform_positions(g.n, 14) * 2.0 ** 18) / 2.0 ** 18
+    s, o = 2.0 ** 500, 2.0 ** 533
+    with G.Batch([g]) as b:
+        near = G.gila_layout_batch_run(b.handle, G.params(k=2, iters=1, t0=1.0, precision=G.GILA_FP64), pos)
+        far = G.gila_layout_batch_run(b.handle, G.params(k=2, iters=1, d=s, t0=s, precision=G.GILA_FP64),
+                                      o + s * pos)
+    assert np.abs((far - o) / s - near).max() <= 2.0 ** -18
