@@ -400,7 +400,9 @@ typedef struct gila_pruned gila_pruned;
 
 /* Repulsion weights: the repulsion that vertex v exerts is multiplied by
  * weight_host[v] (double[n], finite, >= 0; copied). NULL removes them.
- * Applied by the plain iteration kernel (automatic tiling then stays off);
+ * With p = 2 and q = 1 applied by the plain kernel and by the tiles, which keep
+ * the weights beside the positions (automatic mode: from 4 10^6 k-hop entries
+ * and 8 a segment on); with other exponents by the plain kernel alone.
  * GILA_FP64_ORDERED rejects weighted graphs with GILA_EINVAL. The quality
  * figures of gila_layout_metrics stay unweighted. */
 gila_status gila_graph_set_repulsion_weights(gila_graph* g, const double* weight_host);
@@ -500,7 +502,8 @@ gila_status gila_profile_read(gila_graph* g, int64_t* builds, double* build_ms,
 
 /* With on = 2 each iteration's repulsion kernel (the one that streams the
  * k-hop lists of Section 4.5: "blocked_kernel", "blocked_kernel (window)",
- * "iteration_kernel" or "ordered_kernel") is also timed on its own, between
+ * "blocked_kernel (window, row per lane)", "iteration_kernel" or
+ * "ordered_kernel") is also timed on its own, between
  * events recorded directly before and after its launch. Returns the number
  * of such launches since the previous call and their total ms, and copies
  * the name of the last kernel timed into name (NUL-terminated, at most

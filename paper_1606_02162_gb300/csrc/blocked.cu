@@ -1069,7 +1069,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const CombineA
     pu.x = T(0);
     pu.y = T(0);
     if (live) {
-        // tile partials first (independent loads), lane gl takes tiles gl, gl + 8, ...
+        // tile partials first (independent loads), lane gl takes tiles gl, gl + 4, ...
         for (int jj = gl; jj < A.nt; jj += kCombineLanes) add_cell<T, COMP>(A.part, A.n, jj, u, rep);
         pu = pos_in[u];
         att.xu = pu.x;
@@ -1450,7 +1450,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32, 4) block_layout_kernel(
     const int32_t* __restrict__ start, const int32_t* __restrict__ toff,
     const int64_t* __restrict__ blk, const int4* __restrict__ bdesc, uint16_t* __restrict__ tk_all)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SpreadSmem& S = reinterpret_cast<SpreadSmem*>(smem_raw)[warp];
     const int64_t b = blockIdx.x;
@@ -2072,19 +2072,15 @@ int64_t cut_rows(const int64_t* pre, int64_t n, int64_t cap, int64_t limit, int6
 
 // The same on the host, for window mode (its rows, or slices of rows, as one
 // tile): the smallest block cost for which the greedy cut gives at most
-// `target` ranges (or the fewest the row limit allows). pre: nt prefix-sum
-// arrays of n + 1 costs, tile after tile.
-std::vector<std::vector<int32_t>> partition_blocks(const std::vector<int64_t>& pre, int64_t n,
-                                                   int64_t nt, int64_t target, int64_t max_rows)
+// `target` ranges (or the fewest the row limit allows). pre: prefix sums of n
+// costs (n + 1 values).
+std::vector<int32_t> partition_rows(const std::vector<int64_t>& pre, int64_t n, int64_t target,
+                                    int64_t max_rows)
 {
     auto count = [&](int64_t cap, int64_t limit) {
-        int64_t c = 0;
-        for (int64_t j = 0; j < nt && c <= limit; ++j)
-            c += cut_rows(pre.data() + j * (n + 1), n, cap, limit - c, max_rows, nullptr);
-        return c;
+        return cut_rows(pre.data(), n, cap, limit, max_rows, nullptr);
     };
-    int64_t hi = 0;  // a cap every tile fits in whole: the fewest ranges
-    for (int64_t j = 0; j < nt; ++j) hi = std::max<int64_t>(hi, pre[(size_t)(j * (n + 1) + n)]);
+    int64_t hi = pre[(size_t)n];  // a cap that all rows fit in: the fewest ranges
     target = std::max<int64_t>(target, count(hi, INT64_MAX));
     int64_t lo = 0;  // count(lo) > target unless single rows already fit
     if (count(lo, target) <= target) hi = lo;
@@ -2092,10 +2088,9 @@ std::vector<std::vector<int32_t>> partition_blocks(const std::vector<int64_t>& p
         const int64_t mid = lo + (hi - lo) / 2;
         if (count(mid, target) <= target) hi = mid; else lo = mid;
     }
-    std::vector<std::vector<int32_t>> rs((size_t)nt);
-    for (int64_t j = 0; j < nt; ++j)
-        cut_rows(pre.data() + j * (n + 1), n, hi, INT64_MAX, max_rows, &rs[(size_t)j]);
-    return rs;
+    std::vector<int32_t> cuts;
+    cut_rows(pre.data(), n, hi, INT64_MAX, max_rows, &cuts);
+    return cuts;
 }
 
 // CTAs per SM the blocked grid aims at by default (blocks of equal cost,
@@ -2302,7 +2297,7 @@ gila_status plan_rows(gila_graph* g, size_t esz, TilePlan& P, const std::vector<
     std::vector<int64_t> wb;
     int64_t nr = 0, wmax = 0, wsum = 0;
     auto windows = [&](int64_t target) {
-        rs = partition_blocks(pre, nsl, 1, target, nsl)[0];
+        rs = partition_rows(pre, nsl, target, nsl);
         nr = (int64_t)rs.size() - 1;
         wb.assign(2 * (size_t)nr, 0);
         wmax = wsum = 0;
@@ -2381,11 +2376,11 @@ gila_status plan_rows(gila_graph* g, size_t esz, TilePlan& P, const std::vector<
 // small enough to fit whole), read their positions from that window. Each
 // row then lies wholly in its range's block, so the CTA finishes its rows
 // itself (no partials, no second kernel). *fits tells whether every range's
-// window fits; `len` receives the row lengths, `rs` the ranges, `wb` the
-// windows (2 nr: first id, length).
+// window fits; `rs` receives the ranges, `wb` the windows (2 nr: first id,
+// length).
 gila_status plan_window(gila_graph* g, size_t esz, TilePlan& P, bool* fits,
-                        std::vector<int64_t>& len, std::vector<int32_t>& rs,
-                        std::vector<int64_t>& wb, int64_t* wmax_out, int64_t* rmax_out)
+                        std::vector<int32_t>& rs, std::vector<int64_t>& wb, int64_t* wmax_out,
+                        int64_t* rmax_out)
 {
     *fits = false;
     const int64_t n = g->n;
@@ -2412,17 +2407,13 @@ gila_status plan_window(gila_graph* g, size_t esz, TilePlan& P, bool* fits,
     GILA_CUDA(cudaStreamSynchronize(g->stream));
     bool done = false;
     if ((s = plan_rows(g, esz, P, krow, span, &done)) != GILA_OK || done) return s;
-    len.assign((size_t)n, 0);
     std::vector<int64_t> pre((size_t)n + 1, 0);
-    for (int64_t u = 0; u < n; ++u) {
-        len[(size_t)u] = krow[(size_t)u + 1] - krow[(size_t)u];
-        pre[(size_t)u + 1] = pre[(size_t)u] + row_cost(len[(size_t)u]);
-    }
+    for (int64_t u = 0; u < n; ++u)
+        pre[(size_t)u + 1] = pre[(size_t)u] + row_cost(krow[(size_t)u + 1] - krow[(size_t)u]);
     // enough ranges for several CTAs per SM, but at least about 16 entries
     // per thread of a CTA (a small graph is one or a few ranges)
     const int64_t by_work = std::max<int64_t>(1, pre[(size_t)n] / ((int64_t)kBThreads * 16));
-    rs = partition_blocks(pre, n, 1, std::min<int64_t>(blocks_target(g, true), by_work),
-                          kMaxRows)[0];
+    rs = partition_rows(pre, n, std::min<int64_t>(blocks_target(g, true), by_work), kMaxRows);
     const int64_t nr = (int64_t)rs.size() - 1;
     wb.assign(2 * (size_t)nr, 0);
     int64_t wmax = 0, rmax = 0;
@@ -2636,10 +2627,10 @@ gila_status plan_tiles(gila_graph* g, size_t esz, TilePlan& P)
         if (!weighted && g->tune.tile_vertices <= 0 &&
             (g->tune.tiled > 0 || g->nnz_khop >= kBlockedMinNnz)) {
             bool fits = false;
-            std::vector<int64_t> len, wb;
+            std::vector<int64_t> wb;
             std::vector<int32_t> rs;
             int64_t wmax = 0, rmax = 0;
-            gila_status s = plan_window(g, esz, P, &fits, len, rs, wb, &wmax, &rmax);
+            gila_status s = plan_window(g, esz, P, &fits, rs, wb, &wmax, &rmax);
             if (s != GILA_OK || P.rows) return s;
             if (fits) {
                 if ((s = ensure((void**)&P.len, &P.len_cap, 2 * sizeof(int32_t) * (size_t)n)) != GILA_OK)

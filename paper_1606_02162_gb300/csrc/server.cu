@@ -110,7 +110,10 @@ namespace {
 
 size_t pos_size(int precision) { return is_f64(precision) ? 16 : 8; }
 
-// Device bytes a job holds while it runs (upper estimate, exact list size).
+// Device bytes a job holds while it runs (upper estimate, exact list size). A
+// tile plan's scratch of up to 64 MB lies within what the window-mode part and
+// four spare bytes a cell leave (14 MB or more over all n up to 5 10^6 and 4 10^6
+// to 4 10^10 entries).
 size_t job_bytes(int64_t n, int64_t nnz_adj, int64_t nnz_khop, int precision,
                  const gila_tuning& tune)
 {
