@@ -281,8 +281,8 @@ __global__ void __launch_bounds__(1024) batch_kernel(const BatchArgs A)
 // keep), whose bound was the latency of one group's chain (offsets, ids,
 // positions, reduction) and, in FP64, lanes without work on the two FP64
 // operations a clock of an SM: 500 graphs of 50..5000 vertices, k = 2, 50
-// iterations in FP32 6.5 -> 0.58 ms, 3000 graphs 9.2 -> 1.6 ms (30
-// iterations), 250 graphs in FP64 20.8 -> 3.9 ms (20 iterations; its FP64
+// iterations in FP32 6.5 -> 0.62 ms, 3000 graphs 9.2 -> 1.6 ms (30
+// iterations), 250 graphs in FP64 20.8 -> 3.6 ms (20 iterations; its FP64
 // pipe is 63% busy, the FP32 form issues in 52% of the cycles, the rest mostly
 // the barrier between iterations).
 constexpr int kBrCluster = 8;             // largest cluster

@@ -172,7 +172,7 @@ __host__ __device__ __forceinline__ size_t weights_at(int64_t tv, int64_t rmax, 
 // W (tile mode): the tile's repulsion weights beside its positions, one more
 // shared-memory read and product per entry. (The plain kernel gathers a
 // position and a weight per entry through L2, 62% busy: the pruned Chung-Lu
-// graph of 100,000 vertices, k = 2, 2.2e7 entries, 104 -> 44 us an iteration.)
+// graph of 100,000 vertices, k = 2, 2.2e7 entries, 104 -> 45 us an iteration.)
 template <class T, int MODEL, bool COMP, bool WIN, bool W>
 __global__ void __launch_bounds__(kBThreads, 1) blocked_kernel(const BlockedArgs A)
 {
@@ -704,7 +704,7 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
 // keeps their gathers free of bank conflicts without any reordering. 512
 // threads at 64 registers put two CTAs on an SM, one loading its window
 // while the other computes.
-// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration (29.7
+// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration (29.9
 // since, with early launches and fr_entry)
 // against the shares of blocked_kernel; 700 x 700, FP32: 35.3 -> 17.6.
 //

@@ -36,15 +36,15 @@ constexpr int kThreads = 256;
 // Threads per block of the iteration kernel on small graphs: FP64 issues two
 // lanes a clock on an SM, and the latency chain of a row is the same
 // everywhere, so a grid that does not fill the SMs with 256 threads a block
-// is spread over more of them (32 x 32 grid, FP64: 7.2 -> 5.9 us per
-// iteration; with the early launches and staged rows below 12.5 -> 5.9).
-// Four warps, one for each of an SM's schedulers.
+// is spread over more of them (32 x 32 grid, FP64: 8.3 -> 5.9 us per
+// iteration; 64 x 50 18.6 -> 10.4). Four warps, one for each of an SM's
+// schedulers.
 constexpr int kThreadsSmall = 128;
 // FP32: rows of the warp class longer than this are taken by the whole block in
-// small grids (BA n = 10,000, k = 2: 17.6 -> 12.0 us per iteration with it,
-// the early launches and batched adjacency loads; at 512 14.7, at 256 18.4;
-// from 16 blocks per SM on, hubs' warps no longer stand out: the pruned
-// Chung-Lu graph n = 100,000 103 -> 115 with it)
+// small grids (BA n = 10,000, k = 2: 12.8 -> 10.4 us per iteration; a fifth
+// slower from 512 entries on, half from 256; from 16 blocks per SM on, hubs'
+// warps no longer stand out: the pruned Chung-Lu graph n = 100,000 103 -> 115
+// with it)
 constexpr int kCoopRow = 1024;
 
 struct IterArgs {
@@ -407,11 +407,11 @@ ordered_kernel(int64_t n, const int64_t* __restrict__ row, const int32_t* __rest
 template <class T, int MODEL, bool COMP>
 cudaError_t launch_typed(const IterArgs& A, int nt, unsigned grid, int64_t sms, cudaStream_t st)
 {
-    // Early start of the next iteration's blocks saves 1.5 to 2.5 us an
-    // iteration (grid 32 x 32: FP32 4.3 -> 2.9, FP64 7.4 -> 5.9). FP64 takes
-    // it up to one block per SM: blocks that come early are not spread evenly,
-    // and two that share an SM share its two FP64 lanes (64 x 50 grid, 200
-    // blocks: 16.9 us with it, 9.7 without).
+    // Early start of the next iteration's blocks saves 2 to 3 us an iteration
+    // (grid 32 x 32: FP32 6.2 -> 3.0, FP64 8.3 -> 5.9). FP64 takes it up to one
+    // block per SM: blocks that come early are not spread evenly, and two that
+    // share an SM share its two FP64 lanes (64 x 50 grid, 200 blocks: 20.4 us
+    // with it, 10.4 without).
     const bool early = sizeof(T) == 4 || (int64_t)grid <= sms;
     cudaError_t e;
     if (nt == kThreadsSmall)
