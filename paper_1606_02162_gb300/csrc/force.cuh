@@ -252,37 +252,35 @@ struct PosSource {
 };
 
 // 1 / r^2 at every distance whose square is a normal number (FP32 from 1.1e-19,
-// FP64 from 1.5e-154), and finite at distance 0, where it multiplies
-// dx = dy = 0: the pair adds nothing. FP64 bounds r^2 by its high word, off the
-// FP64 pipe.
+// FP64 from 1.5e-154). At distance 0 a pair adds nothing (in FP64 the factor is
+// finite and multiplies dx = dy = 0), and neither does a coordinate that is NaN
+// add anything along the other one. FP64 bounds r^2 by its high word on both
+// sides, off the FP64 pipe. (FP32 by fmaxf instead of the comparison: 500 graphs
+// 616 instead of 625 us, but a NaN would come out as the smallest distance.)
 __device__ __forceinline__ float rcp_r2(float dx, float dy)
 {
-    return rcp_fast(fmaxf(fmaf(dx, dx, dy * dy), 0x1p-126f));
+    const float r2 = fmaf(dx, dx, dy * dy);
+    return r2 > 0.0f ? rcp_fast(r2) : 0.0f;
 }
 __device__ __forceinline__ double rcp_r2(double dx, double dy)
 {
     const double r2 = fma(dx, dx, dy * dy);
     const unsigned hi = (unsigned)__double2hiint(r2);
-    return rcp_newton(__hiloint2double((int)(hi > 0x00100000u ? hi : 0x00100000u), __double2loint(r2)));
+    const unsigned h1 = hi > 0x00100000u ? hi : 0x00100000u;
+    return rcp_newton(__hiloint2double((int)(h1 < 0x7fdfffffu ? h1 : 0x7fdfffffu), __double2loint(r2)));
 }
 
 // d^2 / r^2, and 0 at distance 0: what a weight of any size is multiplied by
-// (a factor that is only finite there, 2^126 or 2^1022, overflows under a weight,
-// and inf times dx = 0 is NaN). FP64: r^2 is bounded by its high word on both
-// sides, off the FP64 pipe, so that a distance whose square overflows (the
-// padding's, from a vertex beyond 1e154) gives 0 as well.
+// (FP64's factor that is only finite there, 2^1022, overflows under a weight, and
+// inf times dx = 0 is NaN).
 __device__ __forceinline__ float rep_scaled(float d2, float dx, float dy)
 {
-    const float r2 = fmaf(dx, dx, dy * dy);
-    return r2 > 0.0f ? d2 * rcp_fast(r2) : 0.0f;
+    return d2 * rcp_r2(dx, dy);
 }
 __device__ __forceinline__ double rep_scaled(double d2, double dx, double dy)
 {
-    const double r2 = fma(dx, dx, dy * dy);
-    const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
-    const unsigned h1 = hi > 0x00100000u ? hi : 0x00100000u;
-    const double c = d2 * rcp_newton(__hiloint2double((int)(h1 < 0x7fdfffffu ? h1 : 0x7fdfffffu), (int)lo));
-    return (hi | lo) != 0 ? c : 0.0;
+    const double c = d2 * rcp_r2(dx, dy), r2 = fma(dx, dx, dy * dy);
+    return (__double2hiint(r2) | __double2loint(r2)) != 0 ? c : 0.0;
 }
 
 // Repulsion of one k-hop entry v on u (Section 3.1 with the repelling set
@@ -419,10 +417,9 @@ struct Att {
 // A k-hop entry at pv that may be a neighbour as well (FP32,
 // Fruchterman-Reingold): the repulsion as Rep forms it, into `rep` without the
 // factor d^2, and with `edge` the attraction from the same difference and
-// r^2 (at least the smallest normal number, as in rcp_r2; at distance 0 the
-// square root multiplies zero). One subtraction and one r^2 serve both: the mesh
+// r^2 (both as in rcp_r2). One subtraction and one r^2 serve both: the mesh
 // 1000 x 1000, k = 3, 33.1 -> 29.7 us an iteration, 500 graphs of the batch
-// 634 -> 583 us a pass (29.9 and 616 since r^2 is kept exact at small distances
+// 634 -> 583 us a pass (30.2 and 625 since r^2 is kept exact at small distances
 // and the batch adds in four sums).
 template <bool CR, bool CA>
 __device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float inv_d, bool edge,
@@ -434,8 +431,8 @@ __device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float in
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(dd) : "l"(pu), "l"(pp));
     float dx, dy;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(dx), "=f"(dy) : "l"(dd));
-    const float r2 = fmaxf(fmaf(dx, dx, dy * dy), 0x1p-126f);
-    const float c = rcp_fast(r2);
+    const float r2 = fmaf(dx, dx, dy * dy);
+    const float c = r2 > 0.0f ? rcp_fast(r2) : 0.0f;
     if constexpr (CR) {
         add_compensated(rep, c * dx, c * dy);
     } else {
@@ -444,7 +441,7 @@ __device__ __forceinline__ void fr_entry(float2 pv, float xu, float yu, float in
         asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ac) : "l"(cc), "l"(dd));
         asm("mov.b64 {%0, %1}, %2;" : "=f"(rep.sx), "=f"(rep.sy) : "l"(ac));
     }
-    if (edge) {
+    if (edge && r2 > 0.0f) {
         const float s = -(r2 * rsqrt_fast(r2)) * inv_d;
         if constexpr (CA) {
             add_compensated(at, s * dx, s * dy);

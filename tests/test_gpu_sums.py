@@ -240,3 +240,26 @@ def test_fp64_batch_far_from_the_origin():
         far = G.gila_layout_batch_run(b.handle, G.params(k=2, iters=1, d=s, t0=s, precision=G.GILA_FP64),
                                       o + s * pos)
     assert np.abs((far - o) / s - near).max() <= 2.0 ** -18
+
+
+# a coordinate that is NaN says nothing along the other one: the pattern of
+# NaN in a batch's placement after an iteration is the group kernel's, and the
+# finite coordinates agree
+@pytest.mark.parametrize("prec", [G.GILA_FP32, G.GILA_FP32_COMPENSATED, G.GILA_FP64],
+                         ids=["fp32", "fp32c", "fp64"])
+def test_nan_coordinate_in_a_batch(prec):
+    g = I.grid(12, 13)
+    pos = I.uniform_positions(g.n, 17)
+    pos[60, 1] = np.nan
+    pos[100, 0] = np.nan
+    prm = G.params(k=2, iters=1, t0=1e9, precision=prec)
+    out = []
+    for tune in ({}, dict(group4_max=8)):
+        with G.Batch([g]) as b:
+            G.gila_batch_tune(b.handle, **tune)
+            out.append(G.gila_layout_batch_run(b.handle, prm, pos))
+    rows, groups = out
+    assert np.array_equal(np.isnan(rows), np.isnan(groups)) and np.isnan(rows).sum() < 40
+    fine = ~np.isnan(groups)
+    tol = 1e-12 if prec == G.GILA_FP64 else 1e-5
+    assert np.abs(rows - groups)[fine].max() <= tol * np.abs(groups[fine]).max()
