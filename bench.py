@@ -87,10 +87,10 @@ KERNEL_SOURCES = ("paper_1606_02162_gb300/csrc/blocked.cu",
                   "paper_1606_02162_gb300/csrc/force.cuh",
                   "paper_1606_02162_gb300/csrc/device_util.cuh")
 NCU_TRAFFIC = {
-    "chunglu250k_k3": {"bytes": 22759961600 + 96342272 + 52051200 + 1280,
+    "chunglu250k_k3": {"bytes": 22759395584 + 96012032 + 52050688,
                        "kernels": "blocked_kernel + combine_kernel (one iteration)",
                        "profile": "profiles/launches_chunglu250k_k3.md",
-                       "sources_sha256": "9db54203791b0109e79627eff8b1d98ccc27bb7983cc72c5d95fc411147df3f2"},
+                       "sources_sha256": "6fd99648f9264a2b07e0b5e54c02f247e4a4d6fccdde080ee1edb90da7b34a35"},
 }
 
 

@@ -704,7 +704,7 @@ __device__ __forceinline__ void window_finish(const BlockedArgs& A,
 // keeps their gathers free of bank conflicts without any reordering. 512
 // threads at 64 registers put two CTAs on an SM, one loading its window
 // while the other computes.
-// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration (29.9
+// The mesh 1000 x 1000, k = 3, compensated: 63.5 -> 35 us per iteration (30.2
 // since, with early launches and fr_entry)
 // against the shares of blocked_kernel; 700 x 700, FP32: 35.3 -> 17.6.
 //
